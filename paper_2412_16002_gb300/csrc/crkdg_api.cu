@@ -207,12 +207,27 @@ void build_tables(NodalTables *tab) {
             T.momyf[q] = (float)(T.mom2[q] * T.xg[qb]);
         }
         for (int a = 0; a < n; ++a) T.pm1[a] = (3.0 * T.w1[a]) * T.xg[a];
+        for (int a = 0; a < n; ++a) {
+            T.tlx[0][a] = fx_coef(T.lm[a], kFxTrace);
+            T.tlx[1][a] = fx_coef(T.lp[a], kFxTrace);
+            T.w1x[a] = fx_coef(T.w1[a], kFxAvg);
+        }
+        for (int q = 0; q < n * n; ++q) T.w2x[q] = fx_coef(T.w2[q], kFxAvg);
     }
 }
 
 }  // namespace
 
 void crkdg_build_tables(NodalTables *tab) { build_tables(tab); }
+
+const NodalTables *crkdg_host_tables() {
+    struct Tables {
+        NodalTables t[3];
+        Tables() { build_tables(t); }
+    };
+    static const Tables tables;  // built on first use, safe with several threads
+    return tables.t;
+}
 
 struct crkdg_ctx {
     crkdg_mesh mesh;
@@ -297,6 +312,7 @@ Params base_params(const crkdg_ctx *h) {
     P.gamma = h->flux.gamma;
     P.velx = h->flux.velocity[0];
     P.vely = h->flux.velocity[1];
+    fx_operator(P, crkdg_host_tables()[h->n - 2], h->dim, h->n);
     P.lo = h->bounds.lo;
     P.hi = h->bounds.hi;
     P.eps = h->bounds.eps;
@@ -355,10 +371,8 @@ bool slots_ok(const Params &P, const void *tr, const void *tavg) {
 
 cudaError_t launch(crkdg_ctx *h, int kernel, const Params &P, const Bufs &B) {
     if ((kernel == K_INNER || kernel == K_FINAL) && !slots_ok(P, B.tr, B.tavg)) return cudaErrorInvalidValue;
-    int ncb = cells_per_block(h->dim, h->n);
-    int nblocks = (h->ncell + ncb - 1) / ncb;
-    if (h->dim == 1) return crkdg_launch_1d(kernel, h->n, h->phys, nblocks, h->st, P, B);
-    return crkdg_launch_2d(kernel, h->n, h->phys, nblocks, h->st, P, B);
+    if (h->dim == 1) return crkdg_launch_1d(kernel, h->n, h->phys, h->st, P, B);
+    return crkdg_launch_2d(kernel, h->n, h->phys, h->st, P, B);
 }
 
 MixBufs base_xbufs(const crkdg_ctx *h) {

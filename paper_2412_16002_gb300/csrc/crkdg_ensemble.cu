@@ -421,6 +421,7 @@ crkdg_status crkdg_ensemble_create(int count, const crkdg_ens_problem *problems,
         P.gamma = flux->gamma;
         P.velx = flux->velocity[0];
         P.vely = flux->velocity[1];
+        fx_operator(P, crkdg_host_tables()[q.k - 1], 2, q.k + 1);
         P.lo = bounds->lo;
         P.hi = bounds->hi;
         P.eps = bounds->eps;
@@ -495,20 +496,18 @@ crkdg_status crkdg_ensemble_set_state(crkdg_ens_t e, int i, const double *nodal,
     ECK(e, cudaMemcpyAsync(scratch, nodal, count * sizeof(double),
                            on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, e->st));
     // limiter (as crkdg_set_state), then the rate of the limited state (as crkdg_max_dt)
-    const int nblocks = (p.P.ncell + crkdg_ens_cells_per_block(ENS_INNER, p.n) - 1) /
-                        crkdg_ens_cells_per_block(ENS_INNER, p.n);
     Bufs B = single_bufs(p);
     B.un = scratch;
     B.unew = p.u[p.cur];
     Params P = p.P;
-    ECK(e, crkdg_launch_2d(K_LIMIT, p.n, PH_EULER, nblocks, e->st, P, B));
+    ECK(e, crkdg_launch_2d(K_LIMIT, p.n, PH_EULER, e->st, P, B));
     EnsScal init;
     memset(&init, 0, sizeof(init));
     init.thmin = to_bits(1.0);
     init.ord[0] = init.ord[1] = ~0ull;
     ECK(e, cudaMemcpyAsync(p.sc, &init, sizeof(init), cudaMemcpyHostToDevice, e->st));
     B = single_bufs(p);
-    ECK(e, crkdg_launch_2d(K_A0, p.n, PH_EULER, nblocks, e->st, P, B));
+    ECK(e, crkdg_launch_2d(K_A0, p.n, PH_EULER, e->st, P, B));
     EnsScal back;
     ECK(e, cudaMemcpyAsync(&back, p.sc, sizeof(back), cudaMemcpyDeviceToHost, e->st));
     ECK(e, cudaStreamSynchronize(e->st));

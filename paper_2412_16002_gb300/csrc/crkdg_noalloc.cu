@@ -101,6 +101,7 @@ extern "C" crkdg_status crkdg_apply_F_noalloc(const crkdg_mesh *mesh, int k, int
         P.bc[side] = (mesh->dim == 1 && side >= 2) ? BC_OUTFLOW : mesh->bc[side];
         for (int c = 0; c < MAXM; ++c) P.bcs[side][c] = mesh->bc_state[side][c];
     }
+    fx_operator(P, crkdg_host_tables()[n - 2], mesh->dim, n);
     for (int i = 0; i < MAXS; ++i) P.slot[i] = -1;
     P.s = 1;
     P.dt = 1.0;
@@ -117,11 +118,9 @@ extern "C" crkdg_status crkdg_apply_F_noalloc(const crkdg_mesh *mesh, int k, int
     B.unew = out_dev;
 
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    int ncb = cells_per_block(mesh->dim, n);
-    int nblocks = (ncell + ncb - 1) / ncb;
     auto go = [&](int kernel) {
-        return mesh->dim == 1 ? crkdg_launch_1d(kernel, n, flux->kind, nblocks, st, P, B)
-                              : crkdg_launch_2d(kernel, n, flux->kind, nblocks, st, P, B);
+        return mesh->dim == 1 ? crkdg_launch_1d(kernel, n, flux->kind, st, P, B)
+                              : crkdg_launch_2d(kernel, n, flux->kind, st, P, B);
     };
     P.mode = MODE_OP_G;
     if (go(K_INNER) != cudaSuccess) return CRKDG_E_CUDA;

@@ -9,9 +9,9 @@ cudaError_t crkdg_upload_tables_1d(const NodalTables *t) {
     return cudaMemcpyToSymbol(c_tab, t, sizeof(NodalTables) * 3);
 }
 
-cudaError_t crkdg_launch_1d(int kernel, int n, int phys, int nblocks, cudaStream_t st, const Params &P,
+cudaError_t crkdg_launch_1d(int kernel, int n, int phys, cudaStream_t st, const Params &P,
                             const Bufs &B) {
-    return launch_dim<1>(kernel, n, phys, nblocks, st, P, B);
+    return launch_dim<1>(kernel, n, phys, st, P, B);
 }
 
 cudaError_t crkdg_run_1d(int n, int phys, cudaStream_t st, const Params &P, double *u0, double *u1, RunCtl *ctl,

@@ -9,9 +9,9 @@ cudaError_t crkdg_upload_tables_2d(const NodalTables *t) {
     return cudaMemcpyToSymbol(c_tab, t, sizeof(NodalTables) * 3);
 }
 
-cudaError_t crkdg_launch_2d(int kernel, int n, int phys, int nblocks, cudaStream_t st, const Params &P,
+cudaError_t crkdg_launch_2d(int kernel, int n, int phys, cudaStream_t st, const Params &P,
                             const Bufs &B) {
-    return launch_dim<2>(kernel, n, phys, nblocks, st, P, B);
+    return launch_dim<2>(kernel, n, phys, st, P, B);
 }
 
 cudaError_t crkdg_launch_mx_2d(int kernel, int n, int phys, int nblocks, cudaStream_t st, const Params &P,

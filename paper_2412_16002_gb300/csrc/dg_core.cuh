@@ -3,11 +3,11 @@
 // Included by exactly one translation unit per dimension (dg_1d.cu, dg_2d.cu),
 // each of which owns its copy of the constant tables.
 //
-// Work decomposition: one thread per (cell, node).  A block holds NCB cells of
-// n^d nodes each; the line operators (volume term, traces, lift, S_K
-// interpolation) exchange node data through shared memory.  Per-cell
-// reductions (average, min/max over S_K) are taken by one leader thread per
-// cell in a fixed order, so every result is deterministic.
+// Work decomposition: one thread per (cell, node), whole cells per warp (CfgW), so that
+// every exchange inside a cell is warp-synchronous.  The line operators (volume term,
+// traces, lift, S_K interpolation) exchange node data through shared memory.  Per-cell
+// reductions (min/max over S_K) are taken by one leader thread per cell in a fixed
+// order, so every result is deterministic.
 //
 // Nodal Q^k form of the operators (collocation at the Gauss points, exact
 // diagonal mass matrix), per x-line of a cell with traces u_L = sum_a l_a(-1) u_a,
@@ -22,6 +22,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include "dg_fixed.h"
 #include "dg_types.h"
 
 namespace crkdg {
@@ -392,24 +393,82 @@ struct Cfg {
     static constexpr int NT = NCB * NN;                   // threads per block (multiple of 32)
     static constexpr int PPT = (NSK + NN - 1) / NN;       // S_K points per thread
     static constexpr int FPT = (NTR + NN - 1) / NN;       // face points per thread
+    static constexpr bool WARP = false;                   // cells may straddle warps
 };
 
+// The same with whole cells per warp: 32 / NN cells on a warp's first lanes, the remaining lanes
+// (Q^2: 5 of 32) shadowing the last one (same cell, node and values).  A cell's exchanges then
+// need a warp barrier instead of a block barrier, and a warp whose cells need the limiter's or
+// the operator's slow path does not hold up the others.
+template <int DIM, int N, int PHYS>
+struct CfgW : Cfg<DIM, N, PHYS> {
+    static constexpr int CPW = 32 / Cfg<DIM, N, PHYS>::NN;  // cells per warp
+    static constexpr int NT = kWarpThreads;
+    static constexpr int NCB = CPW * (NT / 32);
+    static constexpr bool WARP = true;
+};
+
+// this thread's cell within the block and node within the cell
+template <class C>
+__device__ __forceinline__ void place(int &lc, int &node) {
+    if constexpr (C::WARP) {
+        int l = threadIdx.x & 31;
+        if (l >= C::CPW * C::NN) l = C::CPW * C::NN - 1;
+        const int w = l / C::NN;
+        lc = (threadIdx.x >> 5) * C::CPW + w;
+        node = l - w * C::NN;
+    } else {
+        lc = threadIdx.x / C::NN;
+        node = threadIdx.x - lc * C::NN;
+    }
+}
+
+// barrier (with a vote) over the threads that share a cell's data
+template <class C>
+__device__ __forceinline__ void cell_sync() {
+    if constexpr (C::WARP)
+        __syncwarp();
+    else
+        __syncthreads();
+}
+template <class C>
+__device__ __forceinline__ bool cell_sync_or(bool x) {
+    if constexpr (C::WARP) {
+        const bool r = __any_sync(0xffffffffu, x);
+        __syncwarp();
+        return r;
+    } else
+        return __syncthreads_or(x);
+}
+
+// Shared memory of one cell.  Warps run ahead of one another, so nothing of a cell overlaps
+// another cell's part; the size is 48 bytes modulo 128, which puts the same element of a warp's
+// cells on different banks.
+template <class C>
+struct CellData {
+    double u[C::M][C::NN];
+    union {  // fluxes live inside eval_G only; the FP32 node copies inside the limiter only
+        double f[C::D][C::M][C::NN];
+        float uf[C::M][C::NN];
+    };
+    double tf[C::NTR][C::M];
+    double avg[C::M];
+    union {  // the limiter's reductions and the final kernel's edge speeds never overlap
+        unsigned long long red[C::NN][2];  // ordbits keys
+        double ts[C::NTR];  // spectral radii of the traces (eval_G of a traced stage)
+        double al[C::NTR];
+    };
+    double th[2];
+    int bad;
+};
+template <class C>
+struct alignas(16) PadCell : CellData<C> {
+    static constexpr int kPad = (128 + 48 - (int)sizeof(CellData<C>) % 128) % 128;
+    char pad[kPad ? kPad : 128];
+};
 template <class C>
 struct Smem {
-    double u[C::NCB][C::M][C::NN];
-    union {  // fluxes live inside eval_G only; the FP32 node copies inside the limiter only
-        double f[C::D][C::NCB][C::M][C::NN];
-        float uf[C::NCB][C::M][C::NN];
-    };
-    double tf[C::NCB][C::NTR][C::M];
-    double avg[C::NCB][C::M];
-    union {  // the limiter's reductions and the final kernel's edge speeds never overlap
-        unsigned long long red[C::NCB][C::NN][2];  // ordbits keys
-        double ts[C::NCB][C::NTR];  // spectral radii of the traces (eval_G of a traced stage)
-        double al[C::NCB][C::NTR];
-    };
-    double th[C::NCB][2];
-    int bad[C::NCB];
+    PadCell<C> c[C::NCB];
 };
 
 // value of every component at S_K point p of the cell whose nodes are su
@@ -587,41 +646,42 @@ __device__ void limit_block(const Params &P, const Bufs &B, Smem<C> &S, int lc, 
     const NodalTables &T = c_tab[N - 2];
 
     // 1. publish node values (and FP32 copies for the screen)
+    cell_sync<C>();  // earlier readers of the cell's arrays are done
 #pragma unroll
     for (int c = 0; c < M; ++c) {
-        S.u[lc][c][node] = u[c];
-        S.uf[lc][c][node] = (float)u[c];
+        S.c[lc].u[c][node] = u[c];
+        S.c[lc].uf[c][node] = (float)u[c];
     }
-    __syncthreads();
+    cell_sync<C>();
     // 2. cell averages (Gauss weights; the mass matrix is exact); FP32 screen of this
     //    thread's S_K points
-    cell_averages<C>(S.u[lc], node, [&](int c, double s) { S.avg[lc][c] = s; });
+    cell_averages<C>(S.c[lc].u, node, [&](int c, double s) { S.c[lc].avg[c] = s; });
     bool unsafe = false;
 #pragma unroll
     for (int j = 0; j < PPT; ++j) {
         int p = node + j * NN;
         if (p < NSK) {
             float v[M], e[M];
-            sk_eval_screen<DIM, N, M, NN>(S.uf[lc], p, v, e);
+            sk_eval_screen<DIM, N, M, NN>(S.c[lc].uf, p, v, e);
             if (!screen_point<PHYS, DIM>(P, v, e)) unsafe = true;
         }
     }
-    __syncthreads();
+    cell_sync<C>();
     if (node == 0) {  // the average (FP32 rounding of the FP64 value: 2^-22 of it)
         float v[M], e[M];
 #pragma unroll
         for (int c = 0; c < M; ++c) {
-            v[c] = (float)S.avg[lc][c];
+            v[c] = (float)S.c[lc].avg[c];
             e[c] = 2.384185791015625e-07f * fabsf(v[c]);
         }
         if (!screen_point<PHYS, DIM>(P, v, e)) unsafe = true;
     }
-    if (!__syncthreads_or(unsafe)) {  // every cell of the block cleared
+    if (!cell_sync_or<C>(unsafe)) {  // every cell of the block cleared
         if (need_pts) {
 #pragma unroll
             for (int j = 0; j < PPT; ++j) {
                 int p = node + j * NN;
-                if (p < NSK) sk_eval<DIM, N, M, NN>(S.u[lc], p, pts[j]);
+                if (p < NSK) sk_eval<DIM, N, M, NN>(S.c[lc].u, p, pts[j]);
             }
         }
         return;
@@ -632,7 +692,7 @@ __device__ void limit_block(const Params &P, const Bufs &B, Smem<C> &S, int lc, 
     for (int j = 0; j < PPT; ++j) {
         int p = node + j * NN;
         if (p < NSK) {
-            sk_eval<DIM, N, M, NN>(S.u[lc], p, pts[j]);
+            sk_eval<DIM, N, M, NN>(S.c[lc].u, p, pts[j]);
             if (isnan_bits(pts[j][0])) {
                 kmin = kKeyNegInf;  // NaN counts as a violation
             } else {
@@ -642,19 +702,19 @@ __device__ void limit_block(const Params &P, const Bufs &B, Smem<C> &S, int lc, 
             }
         }
     }
-    S.red[lc][node][0] = kmin;
-    S.red[lc][node][1] = kmax;
+    S.c[lc].red[node][0] = kmin;
+    S.c[lc].red[node][1] = kmax;
     double ub[M];
 #pragma unroll
-    for (int c = 0; c < M; ++c) ub[c] = S.avg[lc][c];
-    __syncthreads();
+    for (int c = 0; c < M; ++c) ub[c] = S.c[lc].avg[c];
+    cell_sync<C>();
     // 4. leader: admissibility of the average and theta (theta_1 for Euler)
     double reb = 0.0;  // leader: rho e of the average (Euler)
     if (node == 0) {
         unsigned long long kmn = kKeyPosInf, kmx = kKeyNegInf;
         for (int q = 0; q < NN; ++q) {
-            kmn = umin64(kmn, S.red[lc][q][0]);
-            kmx = umax64(kmx, S.red[lc][q][1]);
+            kmn = umin64(kmn, S.c[lc].red[q][0]);
+            kmx = umax64(kmx, S.c[lc].red[q][1]);
         }
         const double mn = ordbits_inv(kmn), mx = ordbits_inv(kmx);
         if constexpr (PHYS == PH_EULER) {
@@ -670,12 +730,12 @@ __device__ void limit_block(const Params &P, const Bufs &B, Smem<C> &S, int lc, 
             if (mx > P.hi) th = fmin(th, ratio01(P.hi - ub[0], mx - ub[0]));
             if (mn < P.lo) th = fmin(th, ratio01(ub[0] - P.lo, ub[0] - mn));
         }
-        S.th[lc][0] = below_one(th) ? th * kMargin : th;
-        S.th[lc][1] = 1.0;
-        S.bad[lc] = 0;
+        S.c[lc].th[0] = below_one(th) ? th * kMargin : th;
+        S.c[lc].th[1] = 1.0;
+        S.c[lc].bad = 0;
     }
-    __syncthreads();
-    double th1 = S.th[lc][0];
+    cell_sync<C>();
+    double th1 = S.c[lc].th[0];
     double th2 = 1.0;
     if constexpr (PHYS == PH_EULER) {
         // 5. rho e at S_K with the density already scaled by theta_1
@@ -695,22 +755,22 @@ __device__ void limit_block(const Params &P, const Bufs &B, Smem<C> &S, int lc, 
                     kt = umin64(kt, ordbits(isnan_bits(re) ? 0.0 : theta2_point<DIM>(ub, v, P.eps)));
             }
         }
-        S.red[lc][node][1] = km;
-        S.red[lc][node][0] = kt;
-        __syncthreads();
+        S.c[lc].red[node][1] = km;
+        S.c[lc].red[node][0] = kt;
+        cell_sync<C>();
         if (node == 0) {
             unsigned long long kmn = kKeyPosInf, ktn = ordbits(1.0);
             for (int q = 0; q < NN; ++q) {
-                kmn = umin64(kmn, S.red[lc][q][1]);
-                ktn = umin64(ktn, S.red[lc][q][0]);
+                kmn = umin64(kmn, S.c[lc].red[q][1]);
+                ktn = umin64(ktn, S.c[lc].red[q][0]);
             }
             const double mn = ordbits_inv(kmn);
-            S.th[lc][1] = ge_pos_bits(mn, P.eps) ? 1.0
+            S.c[lc].th[1] = ge_pos_bits(mn, P.eps) ? 1.0
                           : P.theta2_exact        ? ordbits_inv(ktn) * kMargin
                                                   : ratio01(reb - P.eps, reb - mn) * kMargin;
         }
-        __syncthreads();
-        th2 = S.th[lc][1];
+        cell_sync<C>();
+        th2 = S.c[lc].th[1];
     }
     // 6. rescale towards the average
     bool limited = below_one(th1) || below_one(th2);
@@ -732,29 +792,29 @@ __device__ void limit_block(const Params &P, const Bufs &B, Smem<C> &S, int lc, 
     if (limited) apply(th2);
     // 7. verify the limited cells on S_K with the same interpolation; shrink on a
     //    rounding violation (the final scaling factor towards the average)
-    bool any_limited = __syncthreads_or(limited);
+    bool any_limited = cell_sync_or<C>(limited);
     if (any_limited) {
         for (int attempt = 0; attempt <= 4; ++attempt) {
 #pragma unroll
-            for (int c = 0; c < M; ++c) S.u[lc][c][node] = u[c];
-            __syncthreads();
+            for (int c = 0; c < M; ++c) S.c[lc].u[c][node] = u[c];
+            cell_sync<C>();
             bool viol = false;
             if (limited) {
 #pragma unroll
                 for (int j = 0; j < PPT; ++j) {
                     int p = node + j * NN;
                     if (p < NSK) {
-                        sk_eval<DIM, N, M, NN>(S.u[lc], p, pts[j]);
+                        sk_eval<DIM, N, M, NN>(S.c[lc].u, p, pts[j]);
                         if (!point_ok<PHYS, DIM>(P, pts[j])) viol = true;
                     }
                 }
             }
-            if (viol) S.bad[lc] = 1;
-            bool again = __syncthreads_or(viol);
+            if (viol) S.c[lc].bad = 1;
+            bool again = cell_sync_or<C>(viol);
             if (!again || attempt == 4) break;
-            bool mine = S.bad[lc] != 0;
-            __syncthreads();
-            if (node == 0) S.bad[lc] = 0;
+            bool mine = S.c[lc].bad != 0;
+            cell_sync<C>();
+            if (node == 0) S.c[lc].bad = 0;
             if (mine) {
                 // Euler: theta_2 (all components); scalars: th2 == 1 so the factor multiplies theta
                 tfin = th2 * retry_factor(attempt + 1);
@@ -792,24 +852,24 @@ __device__ void eval_G(const Params &P, Smem<C> &S, int lc, int node, const doub
         }
 #pragma unroll
         for (int c = 0; c < M; ++c) {
-            S.u[lc][c][node] = u[c];
-            S.f[0][lc][c][node] = fx[c];
-            if constexpr (DIM == 2) S.f[1][lc][c][node] = fy[c];
+            S.c[lc].u[c][node] = u[c];
+            S.c[lc].f[0][c][node] = fx[c];
+            if constexpr (DIM == 2) S.c[lc].f[1][c][node] = fy[c];
         }
     }
-    __syncthreads();
+    cell_sync<C>();
     // 2. volume term and interior traces
     double vx[M], vy[M];
 #pragma unroll
     for (int c = 0; c < M; ++c) {
         double s = 0.0;
 #pragma unroll
-        for (int q = 0; q < N; ++q) s = fma(T.Dhat[a][q], S.f[0][lc][c][b * N + q], s);
+        for (int q = 0; q < N; ++q) s = fma(T.Dhat[a][q], S.c[lc].f[0][c][b * N + q], s);
         vx[c] = s;
         if constexpr (DIM == 2) {
             double t = 0.0;
 #pragma unroll
-            for (int r = 0; r < N; ++r) t = fma(T.Dhat[b][r], S.f[1][lc][c][r * N + a], t);
+            for (int r = 0; r < N; ++r) t = fma(T.Dhat[b][r], S.c[lc].f[1][c][r * N + a], t);
             vy[c] = t;
         }
     }
@@ -824,10 +884,10 @@ __device__ void eval_G(const Params &P, Smem<C> &S, int lc, int node, const doub
                 double s = 0.0;
                 if (DIM == 1 || face < 2) {
 #pragma unroll
-                    for (int q = 0; q < N; ++q) s = fma(l[q], S.u[lc][c][pos * N + q], s);
+                    for (int q = 0; q < N; ++q) s = fma(l[q], S.c[lc].u[c][pos * N + q], s);
                 } else {
 #pragma unroll
-                    for (int q = 0; q < N; ++q) s = fma(l[q], S.u[lc][c][q * N + pos], s);
+                    for (int q = 0; q < N; ++q) s = fma(l[q], S.c[lc].u[c][q * N + pos], s);
                 }
                 trs[j][c] = s;
             }
@@ -835,21 +895,304 @@ __device__ void eval_G(const Params &P, Smem<C> &S, int lc, int node, const doub
             const double ri = recip_rho<PHYS>(trs[j]);
             flux_dir_ri<PHYS, DIM>(P, trs[j], face >> 1, ri, f);
 #pragma unroll
-            for (int c = 0; c < M; ++c) S.tf[lc][fp][c] = f[c];
-            if (want_speed) S.ts[lc][fp] = speed_dir_ri<PHYS, DIM>(P, trs[j], face >> 1, ri);
+            for (int c = 0; c < M; ++c) S.c[lc].tf[fp][c] = f[c];
+            if (want_speed) S.c[lc].ts[fp] = speed_dir_ri<PHYS, DIM>(P, trs[j], face >> 1, ri);
         }
     }
-    __syncthreads();
+    cell_sync<C>();
     // 3. lift the interior-trace edge terms
 #pragma unroll
     for (int c = 0; c < M; ++c) {
-        double gx = vx[c] - T.liftp[a] * S.tf[lc][NF + b][c] + T.liftm[a] * S.tf[lc][b][c];
+        double gx = vx[c] - T.liftp[a] * S.c[lc].tf[NF + b][c] + T.liftm[a] * S.c[lc].tf[b][c];
         double gv = P.rhx * gx;
         if constexpr (DIM == 2) {
-            double gy = vy[c] - T.liftp[b] * S.tf[lc][3 * NF + a][c] + T.liftm[b] * S.tf[lc][2 * NF + a][c];
+            double gy = vy[c] - T.liftp[b] * S.c[lc].tf[3 * NF + a][c] + T.liftm[b] * S.c[lc].tf[2 * NF + a][c];
             gv = fma(P.rhy, gy, gv);
         }
         g[c] = gv;
+    }
+}
+
+// G at a warp's nodes with the FP64 form's arithmetic (eval_G), for the warps that the
+// fixed-point form below refuses.  Out of line: it is rare.
+template <class C>
+__device__ __noinline__ void eval_G_slow(const Params &P, Smem<C> &S, int lc, int node, const double *u, double *g,
+                                         double (&trs)[C::FPT][C::M], bool want_speed) {
+    cell_sync<C>();
+    eval_G<C>(P, S, lc, node, u, g, trs, want_speed);
+}
+
+// Fixed-point coefficients and the tableau's products with dt, in shared memory.
+template <class C>
+struct alignas(16) BlockTab {
+    Fx cx[C::NP][C::NP], cy[C::NP][C::NP], lx[C::NP][2], ly[C::NP][2];
+    Fx tl[2][C::NP], w[C::NN];
+    double dtA[MAXS][MAXS], dtb[MAXS];
+};
+// Filled by the whole block (the caller's barrier follows).
+template <class C>
+__device__ __forceinline__ void fill_tab(const Params &P, BlockTab<C> &B) {
+    constexpr int N = C::NP;
+    const NodalTables &T = c_tab[N - 2];
+    for (int t = threadIdx.x; t < N * N; t += C::NT) {
+        B.cx[t / N][t % N] = P.fx.cx[t / N][t % N];
+        if constexpr (C::D == 2) B.cy[t / N][t % N] = P.fx.cy[t / N][t % N];
+        if (t < 2 * N) {
+            B.lx[t / 2][t & 1] = P.fx.lx[t / 2][t & 1];
+            if constexpr (C::D == 2) B.ly[t / 2][t & 1] = P.fx.ly[t / 2][t & 1];
+            B.tl[t / N][t % N] = T.tlx[t / N][t % N];
+        }
+        if (t < C::NN) B.w[t] = C::D == 2 ? T.w2x[t] : T.w1x[t];
+    }
+    for (int t = (int)threadIdx.x - 64; t >= 0 && t < MAXS * MAXS + MAXS; t += C::NT) {  // the third warp
+        if (t < MAXS * MAXS)
+            B.dtA[t / MAXS][t % MAXS] = P.dt * P.A[t / MAXS][t % MAXS];
+        else
+            B.dtb[t - MAXS * MAXS] = P.dt * P.b[t - MAXS * MAXS];
+    }
+}
+
+// n consecutive limbs from shared memory (16-byte accesses where the rows are aligned)
+template <int N>
+__device__ __forceinline__ void load_fx(const Fx *p, Fx (&v)[N]) {
+    if constexpr (N % 2 == 0) {
+#pragma unroll
+        for (int q = 0; q < N; q += 2) {
+            const int4 r = *reinterpret_cast<const int4 *>(p + q);
+            v[q] = Fx{r.x, r.y};
+            v[q + 1] = Fx{r.z, r.w};
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < N; ++q) v[q] = p[q];
+    }
+}
+
+// Largest of each 16-bit half over the threads of a cell.
+template <class C>
+__device__ __forceinline__ unsigned cell_max_halves(unsigned w, int node) {
+    auto vmax = [](unsigned a, unsigned b) {
+        unsigned r;
+        asm("max.u16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+        return r;
+    };
+    constexpr int NN = C::NN;
+    if constexpr ((NN & (NN - 1)) == 0) {
+#pragma unroll
+        for (int o = 1; o < NN; o <<= 1) w = vmax(w, __shfl_xor_sync(0xffffffffu, w, o));
+    } else {  // rotations within the cell's lanes: windows of 2, 4, ... nodes until all are covered
+        int l = threadIdx.x & 31;
+        if (l >= C::CPW * NN) l = C::CPW * NN - 1;
+        const int base = l - node;
+        int have = 1;
+#pragma unroll
+        for (int o = 1; o < NN; o <<= 1) {
+            const int k = have + o <= NN && o == have ? o : NN - have;
+            int src = node + k;
+            if (src >= NN) src -= NN;
+            w = vmax(w, __shfl_sync(0xffffffffu, w, base + src));
+            have += k;
+            if (have >= NN) break;
+        }
+    }
+    return w;
+}
+
+// Exponents outside this range (u's components; zero is fine) take the FP64 form: products of
+// three such values and their differences stay far from overflow and underflow.
+constexpr int kFxExpLo = 1023 - 150, kFxExpHi = 1023 + 150;
+
+// G(u) with its linear maps in fixed point (dg_fixed.h): the stage's node values, then the
+// node and trace fluxes, share one exponent per cell and component, and the volume term, both
+// lifts and their sum are one sum of 2 n + 4 products (2D) per node and component on the integer units,
+// as are the traces and the cell average.  Fluxes and radii are FP64 functions of FP64 states.
+// tfl, tsp: normal fluxes and (want_speed) radii of this thread's traces; avg(c, value) is
+// called once per cell and component with want_avg.  Warp collective.
+//
+// Near vacuum (a density at a node or a trace 2^-20 below the cell's largest, or not positive)
+// and for values outside the exponent range the whole warp takes the FP64 form.
+//
+// Bound by the FP64 fluxes that remain (about 70 FP64 instructions per warp and stage in Q^3 against
+// 145 with FP64 maps).  Set state, steps, get state: 513^2 Q^3, 2 RK4 steps 15.9 -> 11.8 ms; 1024^2
+// Q^2, 3 Heun steps 49.7 -> 40.0 ms (with the warp-synchronous layout of CfgW).
+template <class C, class Fn>
+__device__ __forceinline__ void eval_G_fx(const Params &P, Smem<C> &S, const BlockTab<C> &Tb, int lc, int node,
+                                          const double *u, double *g, double (&trs)[C::FPT][C::M],
+                                          double (&tfl)[C::FPT][C::M], double (&tsp)[C::FPT], bool want_speed,
+                                          bool want_avg, Fn avg) {
+    constexpr int DIM = C::D, N = C::NP, PHYS = C::PH;
+    constexpr int M = C::M, NN = C::NN, NF = C::NF, NTR = C::NTR, FPT = C::FPT;
+    constexpr int W = (M + 1) / 2;  // words of two 16-bit exponents
+    const int a = node % N, b = DIM == 2 ? node / N : 0;
+    auto field = [](const unsigned (&w)[W], int c) { return (int)((w[c >> 1] >> (16 * (c & 1))) & 0xffffu); };
+    // 1. node values in fixed point; node fluxes
+    unsigned eu[W];
+    bool bad = P.fx.on == 0;
+#pragma unroll
+    for (int k = 0; k < W; ++k) eu[k] = 0u;
+#pragma unroll
+    for (int c = 0; c < M; ++c) {
+        const int e = fx_exp(u[c]);
+        if (e == 0 ? nonzero_bits(u[c]) : (e < kFxExpLo || e > kFxExpHi)) bad = true;
+        eu[c >> 1] |= (unsigned)e << (16 * (c & 1));
+    }
+    const int e0 = eu[0] & 0xffffu;  // this node's density
+#pragma unroll
+    for (int k = 0; k < W; ++k) eu[k] = cell_max_halves<C>(eu[k], node);
+    if constexpr (PHYS == PH_EULER) {
+        if (!positive_bits(u[0]) || e0 < field(eu, 0) - 20) bad = true;
+    }
+    CellData<C> &D = S.c[lc];
+    Fx(&fu)[M][NN] = reinterpret_cast<Fx(&)[M][NN]>(D.u);
+    Fx(&ff)[C::D][M][NN] = reinterpret_cast<Fx(&)[C::D][M][NN]>(D.f);
+    Fx(&ft)[M][NTR] = reinterpret_cast<Fx(&)[M][NTR]>(D.tf);
+    cell_sync<C>();  // earlier readers of the cell's arrays are done
+#pragma unroll
+    for (int c = 0; c < M; ++c) fu[c][node] = fx_of(u[c], field(eu, c));
+    double fx[M], fy[M];
+    if constexpr (DIM == 2) {
+        flux_xy<PHYS>(P, u, fx, fy);
+    } else {
+        flux_dir<PHYS, DIM>(P, u, 0, fx);
+    }
+    cell_sync<C>();
+    // 2. traces of this thread's face points, their fluxes and radii
+#pragma unroll
+    for (int j = 0; j < FPT; ++j) {
+        const int fp = node + j * NN;
+        if (fp < NTR) {
+            const int face = fp / NF, pos = fp - face * NF;
+            const bool row = DIM == 1 || face < 2;
+            Fx l[N];
+            load_fx<N>(Tb.tl[face & 1], l);
+#pragma unroll
+            for (int c = 0; c < M; ++c) {
+                FxSum s{0, 0};
+                if (row) {
+                    Fx v[N];
+                    load_fx<N>(&fu[c][pos * N], v);
+#pragma unroll
+                    for (int q = 0; q < N; ++q) fx_mac(s, v[q], l[q]);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < N; ++q) fx_mac(s, fu[c][q * N + pos], l[q]);
+                }
+                trs[j][c] = fx_double(fx_sum(s), fx_shift(field(eu, c), kFxTrace));
+            }
+            if constexpr (PHYS == PH_EULER) {
+                if (!positive_bits(trs[j][0]) || fx_exp(trs[j][0]) < field(eu, 0) - 20) bad = true;
+            }
+        }
+    }
+    if (__any_sync(0xffffffffu, bad)) {  // the FP64 form, for the whole warp
+        double uu[M], gg[M], tt[FPT][M];
+#pragma unroll
+        for (int c = 0; c < M; ++c) uu[c] = u[c];
+        eval_G_slow<C>(P, S, lc, node, uu, gg, tt, want_speed);
+#pragma unroll
+        for (int c = 0; c < M; ++c) g[c] = gg[c];
+#pragma unroll
+        for (int j = 0; j < FPT; ++j) {
+            const int fp = node + j * NN;
+            if (fp < NTR) {
+#pragma unroll
+                for (int c = 0; c < M; ++c) {
+                    trs[j][c] = tt[j][c];
+                    tfl[j][c] = D.tf[fp][c];
+                }
+                if (want_speed) tsp[j] = D.ts[fp];
+            }
+        }
+        if (want_avg) cell_averages<C>(D.u, node, avg);
+        cell_sync<C>();
+        return;
+    }
+#pragma unroll
+    for (int j = 0; j < FPT; ++j) {
+        const int fp = node + j * NN;
+        if (fp < NTR) {
+            const int face = fp / NF;
+            const double ri = recip_rho<PHYS>(trs[j]);
+            flux_dir_ri<PHYS, DIM>(P, trs[j], face >> 1, ri, tfl[j]);
+            if (want_speed) tsp[j] = speed_dir_ri<PHYS, DIM>(P, trs[j], face >> 1, ri);
+        }
+    }
+    // 3. the fluxes of the cell in fixed point
+    unsigned ef[W];
+#pragma unroll
+    for (int k = 0; k < W; ++k) ef[k] = 0u;
+#pragma unroll
+    for (int c = 0; c < M; ++c) {
+        int e = fx_exp(fx[c]);
+        if constexpr (DIM == 2) e = max(e, fx_exp(fy[c]));
+#pragma unroll
+        for (int j = 0; j < FPT; ++j)
+            if (node + j * NN < NTR) e = max(e, fx_exp(tfl[j][c]));
+        ef[c >> 1] |= (unsigned)e << (16 * (c & 1));
+    }
+#pragma unroll
+    for (int k = 0; k < W; ++k) ef[k] = cell_max_halves<C>(ef[k], node);
+#pragma unroll
+    for (int c = 0; c < M; ++c) {
+        const int E = field(ef, c);
+        ff[0][c][node] = fx_of(fx[c], E);
+        if constexpr (DIM == 2) ff[1][c][node] = fx_of(fy[c], E);
+#pragma unroll
+        for (int j = 0; j < FPT; ++j) {
+            const int fp = node + j * NN;
+            if (fp < NTR) ft[c][fp] = fx_of(tfl[j][c], E);
+        }
+    }
+    cell_sync<C>();
+    // 4. G: the row, the column and the four lifted face fluxes
+    {
+        Fx cx[N], cy[N], lx[2], ly[2];
+        load_fx<N>(Tb.cx[a], cx);
+        load_fx<2>(Tb.lx[a], lx);
+        if constexpr (DIM == 2) {
+            load_fx<N>(Tb.cy[b], cy);
+            load_fx<2>(Tb.ly[b], ly);
+        }
+#pragma unroll
+        for (int c = 0; c < M; ++c) {
+            FxSum s{0, 0};
+            Fx v[N];
+            load_fx<N>(&ff[0][c][b * N], v);
+#pragma unroll
+            for (int q = 0; q < N; ++q) fx_mac(s, v[q], cx[q]);
+            fx_mac(s, ft[c][b], lx[0]);
+            fx_mac(s, ft[c][NF + b], lx[1]);
+            if constexpr (DIM == 2) {
+#pragma unroll
+                for (int q = 0; q < N; ++q) fx_mac(s, ff[1][c][q * N + a], cy[q]);
+                fx_mac(s, ft[c][2 * NF + a], ly[0]);
+                fx_mac(s, ft[c][3 * NF + a], ly[1]);
+            }
+            g[c] = fx_double(fx_sum(s), fx_shift(field(ef, c), P.fx.k));
+        }
+    }
+    if (want_avg) {
+        if constexpr (DIM == 2 && NN == 16 && M == 4) {  // four lanes of four nodes per component
+            const int c = node >> 2, r = node & 3;
+            FxSum s{0, 0};
+            Fx v[4], w[4];
+            load_fx<4>(&fu[c][4 * r], v);
+            load_fx<4>(&Tb.w[4 * r], w);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) fx_mac(s, v[q], w[q]);
+            long long x = fx_sum(s);
+            x += __shfl_xor_sync(0xffffffffu, x, 1);
+            x += __shfl_xor_sync(0xffffffffu, x, 2);
+            const double m = fx_double(x, fx_shift(field(eu, c), kFxAvg));
+            if (r == 0) avg(c, m);
+        } else {
+            for (int c = node; c < M; c += NN) {
+                FxSum s{0, 0};
+#pragma unroll
+                for (int q = 0; q < NN; ++q) fx_mac(s, fu[c][q], Tb.w[q]);
+                avg(c, fx_double(fx_sum(s), fx_shift(field(eu, c), kFxAvg)));
+            }
+        }
     }
 }
 
@@ -889,18 +1232,18 @@ __device__ __forceinline__ void project_pk(Smem<C> &S, int lc, int node, double 
     if constexpr (C::D == 2) {
         constexpr int M = C::M, NN = C::NN;
         const NodalTables &T = c_tab[C::NP - 2];
-        __syncthreads();  // earlier readers of S.u are done
+        cell_sync<C>();  // earlier readers of S.u are done
 #pragma unroll
-        for (int c = 0; c < M; ++c) S.u[lc][c][node] = v[c];
-        __syncthreads();
+        for (int c = 0; c < M; ++c) S.c[lc].u[c][node] = v[c];
+        cell_sync<C>();
 #pragma unroll
         for (int c = 0; c < M; ++c) {
             double s = 0.0;
 #pragma unroll
-            for (int q = 0; q < NN; ++q) s = fma(T.pk[node][q], S.u[lc][c][q], s);
+            for (int q = 0; q < NN; ++q) s = fma(T.pk[node][q], S.c[lc].u[c][q], s);
             v[c] = s;
         }
-        __syncthreads();  // S.u is free again
+        cell_sync<C>();  // S.u is free again
     }
 }
 
@@ -968,64 +1311,65 @@ __device__ __forceinline__ void add_source(const Params &P, int cell, int node, 
 
 template <int DIM, int N, int PHYS>
 __device__ __forceinline__ void inner_body(const Params &P, const Bufs &B, int blk) {
-    using C = Cfg<DIM, N, PHYS>;
+    using C = CfgW<DIM, N, PHYS>;
     constexpr int M = C::M, NN = C::NN, NTR = C::NTR, FPT = C::FPT;
     __shared__ Smem<C> S;
-    const int lc = threadIdx.x / NN, node = threadIdx.x - lc * NN;
+    __shared__ BlockTab<C> Tb;
+    int lc, node;
+    place<C>(lc, node);
     const int cell = blk * C::NCB + lc;
     const bool active = cell < P.ncell;
     const bool own = active && owned(P, cell) && !solid_cell(P, cell);  // counts in the flag and statistics
-    double un[M], cur[M], acc[M], gh[MAXS][M];
+    fill_tab<C>(P, Tb);
+    double un[M], cur[M], acc[M], gh[MAXS][M];  // gh is indexed by the stage loop: local memory, in L1
     load_node<DIM, N, PHYS>(P, B.un, cell, node, active, un);
 #pragma unroll
     for (int c = 0; c < M; ++c) cur[c] = acc[c] = un[c];
-#pragma unroll
-    for (int i = 0; i < MAXS; ++i) {
-        if (i >= P.s) break;
+    __syncthreads();
+    // not unrolled: four copies of a stage would not fit the instruction cache
+#pragma unroll 1
+    for (int i = 0; i < P.s; ++i) {
         if (i > 0) {
 #pragma unroll
-            for (int c = 0; c < M; ++c) {
-                double v = un[c];
+            for (int c = 0; c < M; ++c) cur[c] = un[c];
+#pragma unroll 1
+            for (int j = 0; j < i; ++j)
+                if (nonzero_bits(P.A[i][j]))
 #pragma unroll
-                for (int j = 0; j < i; ++j)
-                    if (nonzero_bits(P.A[i][j])) v = fma(P.dt * P.A[i][j], gh[j][c], v);
-                cur[c] = v;
-            }
+                    for (int c = 0; c < M; ++c) cur[c] = fma(Tb.dtA[i][j], gh[j][c], cur[c]);
             if (P.pk) project_pk<C>(S, lc, node, cur);
             double pts[C::PPT][M];
             limit_block(P, B, S, lc, node, own, cur, pts, true, true, false);
         }
-        double trs[FPT][M];
-        const bool keep_faces = P.slot[i] >= 0 && B.tfs != nullptr;
-        eval_G(P, S, lc, node, cur, gh[i], trs, keep_faces);
-        if (P.source && active) add_source<DIM, N, PHYS>(P, cell, node, i, gh[i]);
-        if (P.slot[i] >= 0) {  // cell average of the traced stage value (outflow exterior state)
-            const NodalTables &T = c_tab[N - 2];
-            cell_averages<C>(S.u[lc], node, [&](int c, double s) {
-                if (active) B.tavg[((size_t)P.slot[i] * M + c) * P.ncell + cell] = s;
-            });
-            __syncthreads();
-        }
+        double trs[FPT][M], tfl[FPT][M], tsp[FPT], g[M];
+        const int slot = P.slot[i];
+        const bool keep_faces = slot >= 0 && B.tfs != nullptr;
+        eval_G_fx<C>(P, S, Tb, lc, node, cur, g, trs, tfl, tsp, keep_faces, slot >= 0, [&](int c, double s) {
+            if (active) B.tavg[((size_t)slot * M + c) * P.ncell + cell] = s;  // outflow exterior state
+        });
+        if (P.source && active) add_source<DIM, N, PHYS>(P, cell, node, i, g);
+#pragma unroll
+        for (int c = 0; c < M; ++c) gh[i][c] = g[c];
         if (P.mode == MODE_OP_G) {
 #pragma unroll
-            for (int c = 0; c < M; ++c) acc[c] = gh[i][c];
+            for (int c = 0; c < M; ++c) acc[c] = g[c];
         } else if (nonzero_bits(P.b[i])) {
 #pragma unroll
-            for (int c = 0; c < M; ++c) acc[c] = fma(P.dt * P.b[i], gh[i][c], acc[c]);
+            for (int c = 0; c < M; ++c) acc[c] = fma(Tb.dtb[i], g[c], acc[c]);
         }
-        if (P.slot[i] >= 0 && active) {
-            double *dst = B.tr + (size_t)P.slot[i] * M * P.ncell * NTR;
-            double *dfs = keep_faces ? B.tfs + (size_t)P.slot[i] * (M + 1) * P.ncell * NTR : nullptr;
+        if (slot >= 0 && active) {
+            double *dst = B.tr + (size_t)slot * M * P.ncell * NTR;
+            double *dfs = keep_faces ? B.tfs + (size_t)slot * (M + 1) * P.ncell * NTR : nullptr;
 #pragma unroll
             for (int j = 0; j < FPT; ++j) {
                 int fp = node + j * NN;
                 if (fp < NTR) {
 #pragma unroll
                     for (int c = 0; c < M; ++c) dst[((size_t)c * P.ncell + cell) * NTR + fp] = trs[j][c];
-                    if (keep_faces) {  // this thread's own entries of S.tf and S.ts
+                    if (keep_faces) {
 #pragma unroll
-                        for (int c = 0; c < M; ++c) dfs[((size_t)c * P.ncell + cell) * NTR + fp] = S.tf[lc][fp][c];
-                        dfs[((size_t)M * P.ncell + cell) * NTR + fp] = S.ts[lc][fp];
+                        for (int c = 0; c < M; ++c) dfs[((size_t)c * P.ncell + cell) * NTR + fp] = tfl[j][c];
+                        dfs[((size_t)M * P.ncell + cell) * NTR + fp] = tsp[j];
                     }
                 }
             }
@@ -1039,7 +1383,7 @@ __device__ __forceinline__ void inner_body(const Params &P, const Bufs &B, int b
 }
 
 template <int DIM, int N, int PHYS>
-__global__ void __launch_bounds__(Cfg<DIM, N, PHYS>::NT) k_inner(Params P, Bufs B) {
+__global__ void __launch_bounds__(kWarpThreads, 4) k_inner(Params P, Bufs B) {
     inner_body<DIM, N, PHYS>(P, B, blockIdx.x);
 }
 
@@ -1049,11 +1393,12 @@ __global__ void __launch_bounds__(Cfg<DIM, N, PHYS>::NT) k_inner(Params P, Bufs 
 // sharing the face, so the update is conservative to round-off.
 template <int DIM, int N, int PHYS, bool STORED = false>
 __device__ __forceinline__ void final_body(const Params &P, const Bufs &B, int blk) {
-    using C = Cfg<DIM, N, PHYS>;
+    using C = CfgW<DIM, N, PHYS>;
     constexpr int M = C::M, NN = C::NN, NF = C::NF, NTR = C::NTR, FPT = C::FPT;
     __shared__ Smem<C> S;
     const NodalTables &T = c_tab[N - 2];
-    const int lc = threadIdx.x / NN, node = threadIdx.x - lc * NN;
+    int lc, node;
+    place<C>(lc, node);
     const int cell = blk * C::NCB + lc;
     const bool active = cell < P.ncell;
     const bool own = active && owned(P, cell) && !solid_cell(P, cell);  // counts in the flag, statistics and rate
@@ -1115,12 +1460,12 @@ __device__ __forceinline__ void final_body(const Params &P, const Bufs &B, int b
                     sI = speed_dir_ri<PHYS, DIM>(P, ui[j], dir, riI[j]);
                     sE = speed_dir_ri<PHYS, DIM>(P, ue[j], dir, riE[j]);
                 }
-                S.al[lc][fp] = fmax_nonneg(sI, sE);
+                S.c[lc].al[fp] = fmax_nonneg(sI, sE);
             } else if (fp < NTR) {
-                S.al[lc][fp] = 0.0;
+                S.c[lc].al[fp] = 0.0;
             }
         }
-        __syncthreads();
+        cell_sync<C>();
 #pragma unroll
         for (int j = 0; j < FPT; ++j) {
             int fp = node + j * NN;
@@ -1129,7 +1474,7 @@ __device__ __forceinline__ void final_body(const Params &P, const Bufs &B, int b
                 int dir = face >> 1;
                 double alpha = 0.0;  // per-edge LF viscosity: max over the edge's points
 #pragma unroll
-                for (int q = 0; q < NF; ++q) alpha = fmax_nonneg(alpha, S.al[lc][face * NF + q]);
+                for (int q = 0; q < NF; ++q) alpha = fmax_nonneg(alpha, S.c[lc].al[face * NF + q]);
                 double fI[M], fE[M];
                 const int nb = nbr[j];
                 if constexpr (STORED) {
@@ -1156,22 +1501,22 @@ __device__ __forceinline__ void final_body(const Params &P, const Bufs &B, int b
                 }
             }
         }
-        __syncthreads();
+        cell_sync<C>();
     }
 #pragma unroll
     for (int j = 0; j < FPT; ++j) {
         int fp = node + j * NN;
         if (fp < NTR)
 #pragma unroll
-            for (int c = 0; c < M; ++c) S.tf[lc][fp][c] = dc[j][c];
+            for (int c = 0; c < M; ++c) S.c[lc].tf[fp][c] = dc[j][c];
     }
-    __syncthreads();
+    cell_sync<C>();
 #pragma unroll
     for (int c = 0; c < M; ++c) {
-        double cx = -T.liftp[a] * S.tf[lc][NF + b][c] + T.liftm[a] * S.tf[lc][b][c];
+        double cx = -T.liftp[a] * S.c[lc].tf[NF + b][c] + T.liftm[a] * S.c[lc].tf[b][c];
         double corr = P.rhx * cx;
         if constexpr (DIM == 2) {
-            double cy = -T.liftp[b] * S.tf[lc][3 * NF + a][c] + T.liftm[b] * S.tf[lc][2 * NF + a][c];
+            double cy = -T.liftp[b] * S.c[lc].tf[3 * NF + a][c] + T.liftm[b] * S.c[lc].tf[2 * NF + a][c];
             corr = fma(P.rhy, cy, corr);
         }
         u[c] = fma(P.dt, corr, u[c]);
@@ -1186,14 +1531,14 @@ __device__ __forceinline__ void final_body(const Params &P, const Bufs &B, int b
     }
     if (P.defer_limit) {  // averages and their admissibility here; limiters in k_trouble
 #pragma unroll
-        for (int c = 0; c < M; ++c) S.u[lc][c][node] = u[c];
-        __syncthreads();
-        cell_averages<C>(S.u[lc], node, [&](int c, double s) {
-            S.avg[lc][c] = s;
+        for (int c = 0; c < M; ++c) S.c[lc].u[c][node] = u[c];
+        cell_sync<C>();
+        cell_averages<C>(S.c[lc].u, node, [&](int c, double s) {
+            S.c[lc].avg[c] = s;
             if (active) B.aux[(size_t)cell * M + c] = s;
         });
-        __syncthreads();
-        if (node == 0 && own && !admissible<PHYS, DIM>(P, S.avg[lc])) atomicOr(B.flag, 1);
+        cell_sync<C>();
+        if (node == 0 && own && !admissible<PHYS, DIM>(P, S.c[lc].avg)) atomicOr(B.flag, 1);
         store_node<DIM, N, PHYS>(P, B.unew, cell, node, active, u);
         return;
     }
@@ -1218,13 +1563,10 @@ __device__ __forceinline__ void final_body(const Params &P, const Bufs &B, int b
 // 2D Q^2 blocks (288 threads), five of the 128-thread ones.  Unbounded, the owned-box test of
 // the domain decomposition took the Q^2 kernel from 96 to 126 registers, one resident block,
 // and the 1024^2 Q^2 launch from 4.78 to 6.33 ms.
-template <class C>
-constexpr int fp64_final_min_blocks() {
-    return C::NT > 128 ? 2 : 5;
-}
+constexpr int fp64_final_min_blocks() { return 5; }
 
 template <int DIM, int N, int PHYS, bool STORED>
-__global__ void __launch_bounds__(Cfg<DIM, N, PHYS>::NT, fp64_final_min_blocks<Cfg<DIM, N, PHYS>>())
+__global__ void __launch_bounds__(kWarpThreads, fp64_final_min_blocks())
     k_final(Params P, Bufs B) {
     final_body<DIM, N, PHYS, STORED>(P, B, blockIdx.x);
 }
@@ -1234,10 +1576,11 @@ __global__ void __launch_bounds__(Cfg<DIM, N, PHYS>::NT, fp64_final_min_blocks<C
 // limiter leaves this thread's S_K values of the final nodal values in pts, the
 // same interpolation of the same values that the scan kernel would take.
 template <int DIM, int N, int PHYS>
-__global__ void __launch_bounds__(Cfg<DIM, N, PHYS>::NT) k_limit(Params P, Bufs B) {
-    using C = Cfg<DIM, N, PHYS>;
+__global__ void __launch_bounds__(kWarpThreads) k_limit(Params P, Bufs B) {
+    using C = CfgW<DIM, N, PHYS>;
     __shared__ Smem<C> S;
-    const int lc = threadIdx.x / C::NN, node = threadIdx.x - lc * C::NN;
+    int lc, node;
+    place<C>(lc, node);
     const int cell = blockIdx.x * C::NCB + lc;
     const bool active = cell < P.ncell;
     const bool own = active && owned(P, cell) && !solid_cell(P, cell);
@@ -1265,19 +1608,20 @@ __global__ void __launch_bounds__(Cfg<DIM, N, PHYS>::NT) k_limit(Params P, Bufs 
 
 // a0 over the S_K points of un, and the two smallest bound margins.
 template <int DIM, int N, int PHYS>
-__global__ void __launch_bounds__(Cfg<DIM, N, PHYS>::NT) k_scan(Params P, Bufs B) {
-    using C = Cfg<DIM, N, PHYS>;
+__global__ void __launch_bounds__(kWarpThreads) k_scan(Params P, Bufs B) {
+    using C = CfgW<DIM, N, PHYS>;
     constexpr int M = C::M, NN = C::NN;
     __shared__ Smem<C> S;
-    const int lc = threadIdx.x / NN, node = threadIdx.x - lc * NN;
+    int lc, node;
+    place<C>(lc, node);
     const int cell = blockIdx.x * C::NCB + lc;
     const bool active = cell < P.ncell;
     const bool own = active && owned(P, cell) && !solid_cell(P, cell);
     double u[M];
     load_node<DIM, N, PHYS>(P, B.un, cell, node, active, u);
 #pragma unroll
-    for (int c = 0; c < M; ++c) S.u[lc][c][node] = u[c];
-    __syncthreads();
+    for (int c = 0; c < M; ++c) S.c[lc].u[c][node] = u[c];
+    cell_sync<C>();
     double amax = 0.0, m0 = INFINITY, m1 = INFINITY;
     const bool margins = P.mode != MODE_RATE;
 #pragma unroll
@@ -1285,7 +1629,7 @@ __global__ void __launch_bounds__(Cfg<DIM, N, PHYS>::NT) k_scan(Params P, Bufs B
         int p = node + j * NN;
         if (p < C::NSK && own) {
             double v[M];
-            sk_eval<DIM, N, M, NN>(S.u[lc], p, v);
+            sk_eval<DIM, N, M, NN>(S.c[lc].u, p, v);
             amax = fmax(amax, sk_rate<PHYS, DIM>(P, v));
             if (!margins) continue;
             double a0m, a1m;
@@ -1384,22 +1728,23 @@ __device__ __forceinline__ double nb_average(const Params &P, const double *aux,
 // first Legendre moments.  Reads unew and the averages in aux; writes unew.
 template <int DIM, int N, int PHYS>
 __device__ __forceinline__ void trouble_body(const Params &P, const Bufs &B, int blk) {
-    using C = Cfg<DIM, N, PHYS>;
+    using C = CfgW<DIM, N, PHYS>;
     constexpr int M = C::M, NN = C::NN;
     __shared__ Smem<C> S;
     __shared__ double sP1[C::NCB][2][M];
     __shared__ int sTr[C::NCB];
     const NodalTables &T = c_tab[N - 2];
-    const int lc = threadIdx.x / NN, node = threadIdx.x - lc * NN;
+    int lc, node;
+    place<C>(lc, node);
     const int cell = blk * C::NCB + lc;
     const bool active = cell < P.ncell;
     const int a = node % N, b = DIM == 2 ? node / N : 0;
     double u[M];
     load_node<DIM, N, PHYS>(P, B.unew, cell, node, active, u);
 #pragma unroll
-    for (int c = 0; c < M; ++c) S.u[lc][c][node] = u[c];
+    for (int c = 0; c < M; ++c) S.c[lc].u[c][node] = u[c];
     if (node == 0) sTr[lc] = 0;
-    __syncthreads();
+    cell_sync<C>();
     // the (direction, component) pairs are spread over the cell's threads: each takes the
     // decision and the limited first moment of its pairs
     for (int j = node; j < DIM * M && active; j += NN) {
@@ -1410,7 +1755,7 @@ __device__ __forceinline__ void trouble_body(const Params &P, const Bufs &B, int
         const double hi = nb_average<PHYS, DIM>(P, B.aux, cell, 2 * d + 1, c);
         double fr = 0.0, fl = 0.0, p1 = 0.0;
         for (int q = 0; q < NN; ++q) {
-            double v = S.u[lc][c][q];
+            double v = S.c[lc].u[c][q];
             if constexpr (DIM == 2) {
                 fr = fma(T.trw2[d][0][q], v, fr);
                 fl = fma(T.trw2[d][1][q], v, fl);
@@ -1427,7 +1772,7 @@ __device__ __forceinline__ void trouble_body(const Params &P, const Bufs &B, int
         if (tvb_changes(utR, dp, dm, thr, thr_ok) || tvb_changes(utL, dp, dm, thr, thr_ok)) atomicOr(&sTr[lc], 1);
         sP1[lc][d][c] = minmod3_bits(p1, dp, dm);
     }
-    __syncthreads();
+    cell_sync<C>();
     bool troubled = active && (P.ind_stage >= 2 ? B.tflags[cell] != 0 : sTr[lc] != 0);
     if (P.ind_stage == 3 && active) {  // learned flags: p > 0.6 troubled, p < 0.4 smooth, else the plain flag
         const float pr = B.prob[cell];
@@ -1461,7 +1806,7 @@ __device__ __forceinline__ void trouble_body(const Params &P, const Bufs &B, int
 }
 
 template <int DIM, int N, int PHYS>
-__global__ void __launch_bounds__(Cfg<DIM, N, PHYS>::NT) k_trouble(Params P, Bufs B) {
+__global__ void __launch_bounds__(kWarpThreads) k_trouble(Params P, Bufs B) {
     trouble_body<DIM, N, PHYS>(P, B, blockIdx.x);
 }
 
@@ -1594,8 +1939,9 @@ __global__ void k_features(Params P, Bufs B) {
 }
 
 template <int DIM, int N, int PHYS>
-cudaError_t launch_one(int kernel, int nblocks, cudaStream_t st, const Params &P, const Bufs &B) {
-    using C = Cfg<DIM, N, PHYS>;
+cudaError_t launch_one(int kernel, cudaStream_t st, const Params &P, const Bufs &B) {
+    using C = CfgW<DIM, N, PHYS>;
+    const int nblocks = (P.ncell + C::NCB - 1) / C::NCB;
     switch (kernel) {
     case K_INNER: k_inner<DIM, N, PHYS><<<nblocks, C::NT, 0, st>>>(P, B); break;
     case K_FINAL:
@@ -1620,10 +1966,9 @@ cudaError_t launch_one(int kernel, int nblocks, cudaStream_t st, const Params &P
 }
 
 template <int DIM>
-cudaError_t launch_dim(int kernel, int n, int phys, int nblocks, cudaStream_t st, const Params &P,
-                       const Bufs &B) {
+cudaError_t launch_dim(int kernel, int n, int phys, cudaStream_t st, const Params &P, const Bufs &B) {
 #define CRKDG_CASE(NV, PV) \
-    if (n == NV && phys == PV) return launch_one<DIM, NV, PV>(kernel, nblocks, st, P, B);
+    if (n == NV && phys == PV) return launch_one<DIM, NV, PV>(kernel, st, P, B);
     CRKDG_CASE(2, PH_ADV) CRKDG_CASE(2, PH_BURG) CRKDG_CASE(2, PH_EULER)
     CRKDG_CASE(3, PH_ADV) CRKDG_CASE(3, PH_BURG) CRKDG_CASE(3, PH_EULER)
     CRKDG_CASE(4, PH_ADV) CRKDG_CASE(4, PH_BURG) CRKDG_CASE(4, PH_EULER)

@@ -30,7 +30,7 @@ int crkdg_ens_occupancy(int kind, int n) {
 
 int crkdg_ens_cells_per_block(int kind, int n) {
     if (kind == ENS_FEATURES) return 128;
-    return n == 3 ? Cfg<2, 3, PH_EULER>::NCB : Cfg<2, 4, PH_EULER>::NCB;
+    return n == 3 ? CfgW<2, 3, PH_EULER>::NCB : CfgW<2, 4, PH_EULER>::NCB;
 }
 
 cudaError_t crkdg_ens_control(int which, cudaStream_t st, EnsProblem *E, int np, EnsCtl *ctl, int arg) {

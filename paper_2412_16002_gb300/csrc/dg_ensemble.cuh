@@ -50,13 +50,13 @@ __device__ __forceinline__ void ens_body(const Params &P, const Bufs &B, int blk
 
 template <int N, int KIND>
 constexpr int ens_threads() {
-    return KIND == ENS_FEATURES ? 128 : Cfg<2, N, PH_EULER>::NT;
+    return KIND == ENS_FEATURES ? 128 : kWarpThreads;
 }
 
 // Persistent launch over the work items of one degree.  stage: the troubled-cell
 // kernel's ind_stage (ENS_TROUBLE only).
 template <int N, int KIND>
-__global__ void __launch_bounds__(ens_threads<N, KIND>()) k_ens(EnsProblem *E, const EnsItem *items, int nitems,
+__global__ void __launch_bounds__(ens_threads<N, KIND>(), KIND == ENS_FEATURES ? 1 : KIND == ENS_FINAL ? 5 : 4) k_ens(EnsProblem *E, const EnsItem *items, int nitems,
                                                                 EnsCtl *ctl, int counter, int stage) {
     __shared__ Params sP;
     __shared__ Bufs sB;

@@ -27,6 +27,7 @@ struct RunCfg1D {
     static constexpr int L = nlob(N);
     static constexpr int NSK = L;
     static constexpr int NCB = NCBV;  // cells per chunk including the two halo cells
+    static constexpr bool WARP = false;
     static constexpr int NT = NCB * NN;
     static constexpr int PPT = (NSK + NN - 1) / NN;
     static constexpr int FPT = (NTR + NN - 1) / NN;
@@ -154,15 +155,15 @@ __global__ void __launch_bounds__(RunCfg1D<N, PHYS, NCBV>::NT) k_run1d(Params P,
 #pragma unroll
                     for (int c = 0; c < M; ++c) {
                         sTr[P.slot[i]][lc][node][c] = trs[0][c];
-                        sTf[P.slot[i]][lc][node][c] = S.tf[lc][node][c];  // written by this thread
+                        sTf[P.slot[i]][lc][node][c] = S.c[lc].tf[node][c];  // written by this thread
                     }
-                    sSp[P.slot[i]][lc][node] = S.ts[lc][node];
+                    sSp[P.slot[i]][lc][node] = S.c[lc].ts[node];
                 }
                 if (P.slot[i] >= 0) {  // S.u holds the stage values until the next stage's limiter
                     for (int c = node; c < M; c += NN) {
                         double s = 0.0;
 #pragma unroll
-                        for (int q = 0; q < NN; ++q) s = fma(T.w1[q], S.u[lc][c][q], s);
+                        for (int q = 0; q < NN; ++q) s = fma(T.w1[q], S.c[lc].u[c][q], s);
                         sAv[P.slot[i]][lc][c] = s;
                     }
                     __syncthreads();

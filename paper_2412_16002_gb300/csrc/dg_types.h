@@ -7,6 +7,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include "dg_fixed.h"
+
 namespace crkdg {
 
 constexpr int MAXN = 4;  // nodes per direction (k <= 3)
@@ -38,6 +40,10 @@ __host__ __device__ constexpr int cells_per_block(int dim, int n) {
            (warp_cells(dim == 2 ? n * n : n) >= 128 ? 1 : 128 / warp_cells(dim == 2 ? n * n : n));
 }
 
+// The FP64 kernels instead keep whole cells per warp (32 / nn of them, see CfgW).
+constexpr int kWarpThreads = 128;
+__host__ __device__ constexpr int warp_cells_per_block(int nn) { return (32 / nn) * (kWarpThreads / 32); }
+
 // One-dimensional nodal tables for n = k+1 Gauss points on [-1, 1].
 struct NodalTables {
     double xg[MAXN], wg[MAXN];  // Gauss--Legendre nodes / weights (sum 2)
@@ -62,6 +68,21 @@ struct NodalTables {
     // from node q, sum over the Legendre modes i + j <= k of L_i(x_a) L_j(x_b) times the
     // Gauss-rule coefficient of that mode at node q
     double pk[MAXN * MAXN][MAXN * MAXN];
+    // fixed-point copies (dg_fixed.h): l_a(-1), l_a(+1) scaled by 2^kFxTrace, the average weights
+    // by 2^kFxAvg
+    Fx tlx[2][MAXN], w1x[MAXN], w2x[MAXN * MAXN];
+};
+constexpr int kFxTrace = 56;  // sum_a |l_a(+-1)| < 4
+constexpr int kFxAvg = 57;    // the weights sum to 1
+
+// Fixed-point coefficients of G scaled by 2^k: row a of the x term, 2/h_x Dhat[a][q] against the
+// x-fluxes of the node's row and -+ 2/h_x l_a(+-1)/w_a against its two x-face fluxes, and the y
+// term likewise; k makes the largest row sum of magnitudes at most 2^58.  on = 0: the scales
+// are outside the range of the fixed-point path (the FP64 form runs).
+struct FxOp {
+    Fx cx[MAXN][MAXN], cy[MAXN][MAXN];
+    Fx lx[MAXN][2], ly[MAXN][2];  // [0] the lower face, [1] the upper one
+    int k, on;
 };
 
 // FP32 copies of the parameters for the split-precision kernels, rounded once by
@@ -122,6 +143,7 @@ struct Params {
     // bits 4s..4s+3 the boundary kind of side s (GEO_*), GEO_SOLID a cell outside the domain.
     // Solid cells keep u^n (their operators are zero) and count in no test, statistic or rate.
     const unsigned *geo;
+    FxOp fx;  // set by fx_operator
     double gstate[2][MAXM];          // the fixed states A and B of the GEO_STATE_* / GEO_SHOCK kinds
     double shock_x0, shock_speed;    // GEO_SHOCK: state A where x < shock_x0 + shock_speed t
 };
@@ -150,6 +172,36 @@ inline void tvb_thresholds(Params &P) {
     P.thr[0] = P.tvb_M * hx * hx;
     P.thr[1] = P.tvb_M * hy * hy;
     P.thr_feat = P.tvb_M * (2.0 / P.rhx) * (2.0 / P.rhy);
+}
+
+// The fixed-point coefficients of G from rhx, rhy and the tables of the degree (host side).
+inline void fx_operator(Params &P, const NodalTables &T, int dim, int n) {
+    FxOp &F = P.fx;
+    memset(&F, 0, sizeof(F));
+    double sx = 0.0, sy = 0.0;  // largest row sums
+    for (int a = 0; a < n; ++a) {
+        double s = fabs(T.liftm[a]) + fabs(T.liftp[a]);
+        for (int q = 0; q < n; ++q) s += fabs(T.Dhat[a][q]);
+        sx = fmax(sx, fabs(P.rhx) * s);
+        if (dim == 2) sy = fmax(sy, fabs(P.rhy) * s);
+    }
+    auto moderate = [](double x) { return x == 0.0 || (fabs(x) > 0x1p-100 && fabs(x) < 0x1p100); };
+    const double s = sx + sy;
+    F.on = isfinite(s) && s > 0x1p-100 && s < 0x1p100 && moderate(P.gamma) && moderate(P.velx) && moderate(P.vely);
+    if (!F.on) return;
+    int e;
+    frexp(s, &e);  // s < 2^e
+    F.k = 58 - e;
+    for (int a = 0; a < n; ++a) {
+        for (int q = 0; q < n; ++q) {
+            F.cx[a][q] = fx_coef(P.rhx * T.Dhat[a][q], F.k);
+            F.cy[a][q] = dim == 2 ? fx_coef(P.rhy * T.Dhat[a][q], F.k) : Fx{0, 0};
+        }
+        F.lx[a][0] = fx_coef(P.rhx * T.liftm[a], F.k);
+        F.lx[a][1] = fx_coef(-P.rhx * T.liftp[a], F.k);
+        F.ly[a][0] = dim == 2 ? fx_coef(P.rhy * T.liftm[a], F.k) : Fx{0, 0};
+        F.ly[a][1] = dim == 2 ? fx_coef(-P.rhy * T.liftp[a], F.k) : Fx{0, 0};
+    }
 }
 
 // The FP32 bounds of the FP64 limiter's screen (host side): floats on the safe side of
@@ -305,10 +357,10 @@ enum RunStatus { RUN_OK = 0, RUN_BOUNDS = 4, RUN_TIMEOUT = 5 };
 extern "C++" {
 cudaError_t crkdg_upload_tables_1d(const crkdg::NodalTables *t);
 cudaError_t crkdg_upload_tables_2d(const crkdg::NodalTables *t);
-cudaError_t crkdg_launch_1d(int kernel, int n, int phys, int nblocks, cudaStream_t st,
-                            const crkdg::Params &P, const crkdg::Bufs &B);
-cudaError_t crkdg_launch_2d(int kernel, int n, int phys, int nblocks, cudaStream_t st,
-                            const crkdg::Params &P, const crkdg::Bufs &B);
+cudaError_t crkdg_launch_1d(int kernel, int n, int phys, cudaStream_t st, const crkdg::Params &P,
+                            const crkdg::Bufs &B);
+cudaError_t crkdg_launch_2d(int kernel, int n, int phys, cudaStream_t st, const crkdg::Params &P,
+                            const crkdg::Bufs &B);
 cudaError_t crkdg_launch_mx_1d(int kernel, int n, int phys, int nblocks, cudaStream_t st,
                                const crkdg::Params &P, const crkdg::MixBufs &B);
 cudaError_t crkdg_launch_mx_2d(int kernel, int n, int phys, int nblocks, cudaStream_t st,
@@ -326,6 +378,8 @@ cudaError_t crkdg_ens_control(int which, cudaStream_t st, crkdg::EnsProblem *E, 
 cudaError_t crkdg_launch_inner_tc(cudaStream_t st, const crkdg::Params &P, const crkdg::MixBufs &X);
 // Closed-form nodal tables for n = 2, 3, 4 (defined in crkdg_api.cu).
 void crkdg_build_tables(crkdg::NodalTables *tab);
+// The same tables, built once per process (host memory).
+const crkdg::NodalTables *crkdg_host_tables();
 // Persistent 1D step loop (cooperative launch); chunk: own cells per block chunk (0: fill
 // every block slot of the GPU); *nblocks receives the grid used.
 cudaError_t crkdg_run_1d(int n, int phys, cudaStream_t st, const crkdg::Params &P, double *u0, double *u1,
