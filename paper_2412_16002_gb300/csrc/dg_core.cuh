@@ -75,6 +75,17 @@ __device__ __forceinline__ double fmax_nonneg(double a, double b) {
     return bitsd(umax64(dbits(a), dbits(b)));
 }
 
+// x truncated towards zero to FP32 on the integer units (a conversion instruction takes the FP64
+// pipe 64 cycles): below 2^-126 it is zero, beyond the FP32 range infinite (NaN included).
+__device__ __forceinline__ float trunc_f(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned mag = hi & 0x7fffffffu;
+    unsigned f = __funnelshift_l(lo, mag - (896u << 20), 3);
+    if (mag < (897u << 20)) f = 0u;
+    if (mag >= (1151u << 20)) f = 0x7f800000u;
+    return __uint_as_float(f | (hi & 0x80000000u));
+}
+
 // 1/x by the Newton-Raphson iteration r <- r + r (1 - x r) (quadratic convergence) from
 // the hardware's approximate reciprocal (rcp.approx.ftz.f64); two steps reach double
 // precision (within an ulp of the rounded quotient).  Arguments outside [2^-1000,
@@ -155,18 +166,18 @@ __device__ __forceinline__ void flux_xy(const Params &P, const double *u, double
     } else if constexpr (PHYS == PH_BURG) {
         fx[0] = fy[0] = 0.5 * u[0] * u[0];
     } else {
-        double ri = recip_nr(u[0]);
-        double wx = u[1] * ri, wy = u[2] * ri;
-        double p = (P.gamma - 1.0) * (u[3] - 0.5 * (u[1] * wx + u[2] * wy));
-        double ep = u[3] + p;
+        const double ri = recip_nr(u[0]);
+        const double wx = __dmul_rn(u[1], ri), wy = __dmul_rn(u[2], ri);
+        const double p = __dmul_rn(P.gamma - 1.0, fma(-0.5, fma(u[1], wx, __dmul_rn(u[2], wy)), u[3]));
+        const double ep = __dadd_rn(u[3], p);
         fx[0] = u[1];
-        fx[1] = u[1] * wx + p;
-        fx[2] = u[2] * wx;
-        fx[3] = ep * wx;
+        fx[1] = fma(u[1], wx, p);
+        fx[2] = __dmul_rn(u[2], wx);
+        fx[3] = __dmul_rn(ep, wx);
         fy[0] = u[2];
-        fy[1] = u[1] * wy;
-        fy[2] = u[2] * wy + p;
-        fy[3] = ep * wy;
+        fy[1] = __dmul_rn(u[1], wy);
+        fy[2] = fma(u[2], wy, p);
+        fy[3] = __dmul_rn(ep, wy);
     }
 }
 
@@ -216,18 +227,18 @@ __device__ __forceinline__ double flux_speed_dir(const Params &P, const double *
 
 // Trial-step rate at one point: sum over directions of lambda_d / h_d, so that
 // dt = CFL / max rate (eq. numerical_experiment:CFL, directional radii summed in 2D).
-// The Euler form shares the reciprocal and the sound speed between the directions
-// (the same values as speed_dir per direction).
+// The Euler form shares the reciprocal and the sound speed between the directions.
+// Explicit roundings, as in euler_flux_ri: every kernel that takes a rate gets the same bits.
 template <int PHYS, int DIM>
 __device__ __forceinline__ double sk_rate(const Params &P, const double *u) {
     if constexpr (PHYS == PH_EULER) {
-        double ri = recip_nr(u[0]);
-        double kin = DIM == 1 ? u[1] * u[1] : u[1] * u[1] + u[2] * u[2];
-        double p = (P.gamma - 1.0) * (u[DIM + 1] - 0.5 * kin * ri);
-        double c2 = P.gamma * p * ri;
-        double c = positive_bits(c2) ? sqrt(c2) : 0.0;
-        double r = (fabs(u[1] * ri) + c) * (0.5 * P.rhx);
-        if constexpr (DIM == 2) r = fma(fabs(u[2] * ri) + c, 0.5 * P.rhy, r);
+        const double ri = recip_nr(u[0]);
+        const double kin = DIM == 1 ? __dmul_rn(u[1], u[1]) : fma(u[1], u[1], __dmul_rn(u[2], u[2]));
+        const double p = __dmul_rn(P.gamma - 1.0, fma(-0.5 * kin, ri, u[DIM + 1]));
+        const double c2 = __dmul_rn(__dmul_rn(P.gamma, p), ri);
+        const double c = positive_bits(c2) ? sqrt(c2) : 0.0;
+        double r = __dmul_rn(__dadd_rn(fabs(__dmul_rn(u[1], ri)), c), 0.5 * P.rhx);
+        if constexpr (DIM == 2) r = fma(__dadd_rn(fabs(__dmul_rn(u[2], ri)), c), 0.5 * P.rhy, r);
         return r;
     } else {
         double r = speed_dir<PHYS, DIM>(P, u, 0) * (0.5 * P.rhx);
@@ -239,8 +250,8 @@ __device__ __forceinline__ double sk_rate(const Params &P, const double *u) {
 // rho e = E - |m|^2 / (2 rho)   (eq. Euler-limiter2)
 template <int DIM>
 __device__ __forceinline__ double rho_e(const double *u) {
-    double kin = DIM == 1 ? u[1] * u[1] : u[1] * u[1] + u[2] * u[2];
-    return u[DIM + 1] - (0.5 * kin) * recip_nr(u[0]);
+    const double kin = DIM == 1 ? __dmul_rn(u[1], u[1]) : fma(u[1], u[1], __dmul_rn(u[2], u[2]));
+    return fma(-0.5 * kin, recip_nr(u[0]), u[DIM + 1]);
 }
 
 // The exact theta_2 of one S_K point (the alternative to eq. Euler-limiter2's concavity ratio):
@@ -574,6 +585,33 @@ __device__ __forceinline__ bool screen_point(const Params &P, const float *v, co
     }
 }
 
+// An upper bound of sk_rate's FP64 value at a point whose FP64 components lie within e of v and
+// that screen_point has cleared (Euler): the density from below, momenta, and pressure from above,
+// and 2^-18 for the roundings of this bound and of the FP64 form.  Infinity or NaN where the
+// bound fails; the callers then evaluate the point.
+template <int PHYS, int DIM>
+__device__ __forceinline__ float rate_bound(const Params &P, const float *v, const float *e) {
+    if constexpr (PHYS == PH_EULER) {
+        const float up = 1.0f + 3.814697265625e-06f;
+        const float ri = __frcp_rn(v[0] - e[0]), rj = __frcp_rn(v[0] + e[0]);
+        float kin = 0.0f, adv = 0.0f;
+        const float hr[2] = {0.5f * P.scr_rh[0], 0.5f * P.scr_rh[1]};
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) {
+            const float lo = fmaxf(fabsf(v[1 + d]) - e[1 + d], 0.0f);
+            kin = fmaf(lo, lo, kin);
+            adv = fmaf(fabsf(v[1 + d]) + e[1 + d], hr[d], adv);
+        }
+        const float el = v[DIM + 1] + e[DIM + 1];
+        // el - kin rj / 2 with its own rounding covered by 2^-20 of both terms
+        const float re = fmaxf((el - 0.5f * kin * rj) + 9.5367431640625e-07f * (el + 0.5f * kin * rj), 0.0f);
+        const float c = sqrtf(P.scr_gg * re * ri);
+        return fmaf(adv, ri, c * (DIM == 2 ? hr[0] + hr[1] : hr[0])) * up;
+    } else {
+        return INFINITY;
+    }
+}
+
 // S_K bound predicate used by the limiter's verification and by the margins
 template <int PHYS, int DIM>
 __device__ __forceinline__ bool point_ok(const Params &P, const double *v) {
@@ -634,29 +672,32 @@ __device__ __forceinline__ double retry_factor(int attempt) {
 // admissibility of the cell average sets *B.flag (Sec. 4.1 restart test).
 //
 // Most cells need no limiting.  An FP32 screen (screen_point, with a bound on its
-// distance to the FP64 values) first tests every S_K point and the average; when it
-// clears every cell of the block, the FP64 limiter would leave all of them unchanged
-// (theta = 1, no flag), and it is skipped: the results are those of the FP64 path.
+// distance to the FP64 values) first tests every S_K point; when it clears every cell of
+// the block (or warp), the FP64 limiter would leave all of them unchanged (theta = 1) and
+// it is skipped: the results are those of the FP64 path.  The averages need no test of
+// their own then: an average is a convex combination of the S_K values (Prop. 2.2), rho e is
+// concave, and the screen leaves 2^-20 of |E| and |m|^2 / 2 rho (and 2^-22 of the nodes'
+// magnitudes), far above the FP64 rounding of the average.  Returns true when it was
+// skipped; pts is then not set, and with want_rate rhi bounds this thread's point rates.
 template <class C>
-__device__ void limit_block(const Params &P, const Bufs &B, Smem<C> &S, int lc, int node, bool active,
-                            double *u, double (&pts)[C::PPT][C::M], bool check_avg, bool stats,
-                            bool need_pts = true) {
+__device__ bool limit_block(const Params &P, const Bufs &B, Smem<C> &S, int lc, int node, bool active,
+                            double *u, double (&pts)[C::PPT][C::M], bool check_avg, bool stats, bool want_rate,
+                            float &rhi) {
     constexpr int DIM = C::D, N = C::NP, PHYS = C::PH;
     constexpr int M = C::M, NN = C::NN, NSK = C::NSK, PPT = C::PPT;
-    const NodalTables &T = c_tab[N - 2];
 
-    // 1. publish node values (and FP32 copies for the screen)
+    // 1. publish node values (and FP32 copies for the screen: truncated, 2^-23 of the value,
+    //    which the bound of sk_eval_screen covers)
     cell_sync<C>();  // earlier readers of the cell's arrays are done
 #pragma unroll
     for (int c = 0; c < M; ++c) {
         S.c[lc].u[c][node] = u[c];
-        S.c[lc].uf[c][node] = (float)u[c];
+        S.c[lc].uf[c][node] = PHYS == PH_EULER ? trunc_f(u[c]) : (float)u[c];
     }
     cell_sync<C>();
-    // 2. cell averages (Gauss weights; the mass matrix is exact); FP32 screen of this
-    //    thread's S_K points
-    cell_averages<C>(S.c[lc].u, node, [&](int c, double s) { S.c[lc].avg[c] = s; });
+    // 2. FP32 screen of this thread's S_K points
     bool unsafe = false;
+    rhi = 0.0f;
 #pragma unroll
     for (int j = 0; j < PPT; ++j) {
         int p = node + j * NN;
@@ -664,28 +705,15 @@ __device__ void limit_block(const Params &P, const Bufs &B, Smem<C> &S, int lc, 
             float v[M], e[M];
             sk_eval_screen<DIM, N, M, NN>(S.c[lc].uf, p, v, e);
             if (!screen_point<PHYS, DIM>(P, v, e)) unsafe = true;
-        }
-    }
-    cell_sync<C>();
-    if (node == 0) {  // the average (FP32 rounding of the FP64 value: 2^-22 of it)
-        float v[M], e[M];
-#pragma unroll
-        for (int c = 0; c < M; ++c) {
-            v[c] = (float)S.c[lc].avg[c];
-            e[c] = 2.384185791015625e-07f * fabsf(v[c]);
-        }
-        if (!screen_point<PHYS, DIM>(P, v, e)) unsafe = true;
-    }
-    if (!cell_sync_or<C>(unsafe)) {  // every cell of the block cleared
-        if (need_pts) {
-#pragma unroll
-            for (int j = 0; j < PPT; ++j) {
-                int p = node + j * NN;
-                if (p < NSK) sk_eval<DIM, N, M, NN>(S.c[lc].u, p, pts[j]);
+            if (want_rate) {
+                const float r = rate_bound<PHYS, DIM>(P, v, e);
+                rhi = r <= rhi ? rhi : r;  // a NaN stays
             }
         }
-        return;
     }
+    if (!cell_sync_or<C>(unsafe)) return true;  // every cell cleared
+    cell_averages<C>(S.c[lc].u, node, [&](int c, double s) { S.c[lc].avg[c] = s; });
+    cell_sync<C>();
     // 3. values at S_K and this thread's extremes (order-preserving integer keys)
     unsigned long long kmin = kKeyPosInf, kmax = kKeyNegInf;
 #pragma unroll
@@ -826,6 +854,42 @@ __device__ void limit_block(const Params &P, const Bufs &B, Smem<C> &S, int lc, 
         double tr = PHYS == PH_EULER ? fmin(th1, tfin) : th1 * tfin;
         atomicAdd(B.nlim, 1ull);
         atomicMin(B.thmin, dbits(tr > 0.0 ? tr : 0.0));
+    }
+    cell_sync<C>();
+    return false;
+}
+
+// Posts the largest trial-step rate over the S_K points of the limited state (limit_block's
+// cleared, rhi and pts).  A warp whose FP32 bounds stay at or below the rate already posted by
+// others cannot raise the maximum and skips the FP64 interpolation and rates (114 FP64
+// instructions per warp in Q^3): the posted maximum is the same.
+template <class C>
+__device__ __forceinline__ void post_rate(const Params &P, const Bufs &B, const Smem<C> &S, int lc, int node, bool own,
+                                          bool cleared, float rhi, double (&pts)[C::PPT][C::M]) {
+    constexpr int DIM = C::D, N = C::NP, PHYS = C::PH;
+    constexpr int M = C::M, NN = C::NN;
+    bool need = own;
+    if constexpr (PHYS == PH_EULER) {
+        if (cleared) {
+            const double now = bitsd(*(const volatile unsigned long long *)B.a0);
+            need = own && !(rhi <= fminf(trunc_f(now), 3.0e38f));
+        }
+    }
+    if (__any_sync(0xffffffffu, need)) {
+        double amax = 0.0;
+#pragma unroll
+        for (int j = 0; j < C::PPT; ++j) {
+            int p = node + j * NN;
+            if (p < C::NSK && own) {
+                if (cleared) sk_eval<DIM, N, M, NN>(S.c[lc].u, p, pts[j]);
+                amax = fmax_nonneg(amax, sk_rate<PHYS, DIM>(P, pts[j]));
+            }
+        }
+        __syncwarp();
+        unsigned long long abits = dbits(amax);  // non-negative: the bits order as the values
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) abits = umax64(abits, __shfl_xor_sync(0xffffffffu, abits, o));
+        if ((threadIdx.x & 31) == 0 && abits > 0ull) atomicMax(B.a0, abits);
     }
 }
 
@@ -998,6 +1062,14 @@ __device__ __forceinline__ unsigned cell_max_halves(unsigned w, int node) {
     return w;
 }
 
+// Whether x holds for any thread of this thread's cell.
+template <class C>
+__device__ __forceinline__ bool cell_any(bool x, int node) {
+    int l = threadIdx.x & 31;
+    if (l >= C::CPW * C::NN) l = C::CPW * C::NN - 1;
+    return ((__ballot_sync(0xffffffffu, x) >> (l - node)) & ((1u << C::NN) - 1u)) != 0u;
+}
+
 // Exponents outside this range (u's components; zero is fine) take the FP64 form: products of
 // three such values and their differences stay far from overflow and underflow.
 constexpr int kFxExpLo = 1023 - 150, kFxExpHi = 1023 + 150;
@@ -1010,7 +1082,8 @@ constexpr int kFxExpLo = 1023 - 150, kFxExpHi = 1023 + 150;
 // called once per cell and component with want_avg.  Warp collective.
 //
 // Near vacuum (a density at a node or a trace 2^-20 below the cell's largest, or not positive)
-// and for values outside the exponent range the whole warp takes the FP64 form.
+// and for values outside the exponent range the cell takes the FP64 form: a rule of the cell's
+// own values, so a cell's result does not depend on the cells it shares a warp with.
 //
 // Bound by the FP64 fluxes that remain (about 70 FP64 instructions per warp and stage in Q^3 against
 // 145 with FP64 maps).  Set state, steps, get state: 513^2 Q^3, 2 RK4 steps 15.9 -> 11.8 ms; 1024^2
@@ -1083,29 +1156,6 @@ __device__ __forceinline__ void eval_G_fx(const Params &P, Smem<C> &S, const Blo
                 if (!positive_bits(trs[j][0]) || fx_exp(trs[j][0]) < field(eu, 0) - 20) bad = true;
             }
         }
-    }
-    if (__any_sync(0xffffffffu, bad)) {  // the FP64 form, for the whole warp
-        double uu[M], gg[M], tt[FPT][M];
-#pragma unroll
-        for (int c = 0; c < M; ++c) uu[c] = u[c];
-        eval_G_slow<C>(P, S, lc, node, uu, gg, tt, want_speed);
-#pragma unroll
-        for (int c = 0; c < M; ++c) g[c] = gg[c];
-#pragma unroll
-        for (int j = 0; j < FPT; ++j) {
-            const int fp = node + j * NN;
-            if (fp < NTR) {
-#pragma unroll
-                for (int c = 0; c < M; ++c) {
-                    trs[j][c] = tt[j][c];
-                    tfl[j][c] = D.tf[fp][c];
-                }
-                if (want_speed) tsp[j] = D.ts[fp];
-            }
-        }
-        if (want_avg) cell_averages<C>(D.u, node, avg);
-        cell_sync<C>();
-        return;
     }
 #pragma unroll
     for (int j = 0; j < FPT; ++j) {
@@ -1193,6 +1243,35 @@ __device__ __forceinline__ void eval_G_fx(const Params &P, Smem<C> &S, const Blo
                 avg(c, fx_double(fx_sum(s), fx_shift(field(eu, c), kFxAvg)));
             }
         }
+    }
+    if (__any_sync(0xffffffffu, bad)) {  // a cell of the warp takes the FP64 form instead
+        const bool mine = cell_any<C>(bad, node);
+        double uu[M], gg[M], tt[FPT][M];
+#pragma unroll
+        for (int c = 0; c < M; ++c) uu[c] = u[c];
+        eval_G_slow<C>(P, S, lc, node, uu, gg, tt, want_speed);
+        cell_sync<C>();
+        if (mine) {
+#pragma unroll
+            for (int c = 0; c < M; ++c) g[c] = gg[c];
+#pragma unroll
+            for (int j = 0; j < FPT; ++j) {
+                const int fp = node + j * NN;
+                if (fp < NTR) {
+#pragma unroll
+                    for (int c = 0; c < M; ++c) {
+                        trs[j][c] = tt[j][c];
+                        tfl[j][c] = D.tf[fp][c];
+                    }
+                    if (want_speed) tsp[j] = D.ts[fp];
+                }
+            }
+        }
+        if (want_avg)
+            cell_averages<C>(D.u, node, [&](int c, double v) {
+                if (mine) avg(c, v);
+            });
+        cell_sync<C>();
     }
 }
 
@@ -1339,7 +1418,8 @@ __device__ __forceinline__ void inner_body(const Params &P, const Bufs &B, int b
                     for (int c = 0; c < M; ++c) cur[c] = fma(Tb.dtA[i][j], gh[j][c], cur[c]);
             if (P.pk) project_pk<C>(S, lc, node, cur);
             double pts[C::PPT][M];
-            limit_block(P, B, S, lc, node, own, cur, pts, true, true, false);
+            float rhi;
+            limit_block(P, B, S, lc, node, own, cur, pts, true, true, false, rhi);
         }
         double trs[FPT][M], tfl[FPT][M], tsp[FPT], g[M];
         const int slot = P.slot[i];
@@ -1383,20 +1463,99 @@ __device__ __forceinline__ void inner_body(const Params &P, const Bufs &B, int b
 }
 
 template <int DIM, int N, int PHYS>
-__global__ void __launch_bounds__(kWarpThreads, 4) k_inner(Params P, Bufs B) {
+__global__ void __launch_bounds__(kWarpThreads, 4) k_inner(const __grid_constant__ Params P, const __grid_constant__ Bufs B) {
     inner_body<DIM, N, PHYS>(P, B, blockIdx.x);
+}
+
+// u += dt lift(dc) at this thread's node, dc the corrections of this thread's face points (a cell
+// collective): the four products per component in fixed point with one exponent per cell and
+// component (dg_fixed.h), as in eval_G_fx; corrections outside its range take the FP64 form.
+template <class C>
+__device__ __forceinline__ void lift_faces(const Params &P, CellData<C> &D, int node, int a, int b,
+                                           const double (&dc)[C::FPT][C::M], double *u) {
+    constexpr int DIM = C::D, N = C::NP, M = C::M, NN = C::NN, NF = C::NF, NTR = C::NTR, FPT = C::FPT;
+    constexpr int W = (M + 1) / 2;
+    unsigned ef[W];
+    bool bad = P.fx.on == 0;
+#pragma unroll
+    for (int k = 0; k < W; ++k) ef[k] = 0u;
+#pragma unroll
+    for (int c = 0; c < M; ++c) {
+        int e = 0;
+#pragma unroll
+        for (int j = 0; j < FPT; ++j)
+            if (node + j * NN < NTR) {
+                const int ej = fx_exp(dc[j][c]);
+                if (ej == 0 ? nonzero_bits(dc[j][c]) : (ej < 1023 - 600 || ej > 1023 + 600)) bad = true;
+                e = max(e, ej);
+            }
+        ef[c >> 1] |= (unsigned)e << (16 * (c & 1));
+    }
+    double corr[M];
+    const bool any_bad = __any_sync(0xffffffffu, bad);
+    if (any_bad) {  // a cell of the warp takes the FP64 form instead
+        const NodalTables &T = c_tab[N - 2];
+#pragma unroll
+        for (int j = 0; j < FPT; ++j) {
+            const int fp = node + j * NN;
+            if (fp < NTR)
+#pragma unroll
+                for (int c = 0; c < M; ++c) D.tf[fp][c] = dc[j][c];
+        }
+        cell_sync<C>();
+#pragma unroll
+        for (int c = 0; c < M; ++c) {
+            double cx = -T.liftp[a] * D.tf[NF + b][c] + T.liftm[a] * D.tf[b][c];
+            corr[c] = P.rhx * cx;
+            if constexpr (DIM == 2) {
+                double cy = -T.liftp[b] * D.tf[3 * NF + a][c] + T.liftm[b] * D.tf[2 * NF + a][c];
+                corr[c] = fma(P.rhy, cy, corr[c]);
+            }
+        }
+        bad = cell_any<C>(bad, node);
+        cell_sync<C>();
+    }
+    Fx(&ft)[M][NTR] = reinterpret_cast<Fx(&)[M][NTR]>(D.tf);
+#pragma unroll
+    for (int k = 0; k < W; ++k) ef[k] = cell_max_halves<C>(ef[k], node);
+#pragma unroll
+    for (int c = 0; c < M; ++c) {
+        const int E = (int)((ef[c >> 1] >> (16 * (c & 1))) & 0xffffu);
+#pragma unroll
+        for (int j = 0; j < FPT; ++j) {
+            const int fp = node + j * NN;
+            if (fp < NTR) ft[c][fp] = fx_of(dc[j][c], E);
+        }
+    }
+    const Fx x0 = P.fx.lx[a][0], x1 = P.fx.lx[a][1], y0 = P.fx.ly[b][0], y1 = P.fx.ly[b][1];
+    cell_sync<C>();
+#pragma unroll
+    for (int c = 0; c < M; ++c) {
+        const int E = (int)((ef[c >> 1] >> (16 * (c & 1))) & 0xffffu);
+        FxSum s{0, 0};
+        fx_mac(s, ft[c][b], x0);
+        fx_mac(s, ft[c][NF + b], x1);
+        if constexpr (DIM == 2) {
+            fx_mac(s, ft[c][2 * NF + a], y0);
+            fx_mac(s, ft[c][3 * NF + a], y1);
+        }
+        const double v = fx_double(fx_sum(s), fx_shift(E, P.fx.k));
+        u[c] = fma(P.dt, bad ? corr[c] : v, u[c]);
+    }
 }
 
 // Final stage: u^{n+1} = u* + dt lift( sum_i b_i (fhat^(i) - f(u_int^(i))) ), then the
 // limiter, the admissibility test and a0 of the new state.  Each face flux is
-// evaluated from the same ordered pair (lower side, upper side) by both cells
-// sharing the face, so the update is conservative to round-off.
+// evaluated from the same differences by both cells sharing the face, so the update is
+// conservative to round-off.  Bound by the FP64 pipe: 17 FP64 instructions per face point
+// and traced stage are left of 28, the lift runs in fixed point, and the rate is taken only by
+// warps that can raise it (513^2 Q^3, 2 RK4 steps with set and get 11.8 -> 8.3 ms; 1024^2 Q^2,
+// 3 Heun steps 40.0 -> 29.0 ms).
 template <int DIM, int N, int PHYS, bool STORED = false>
 __device__ __forceinline__ void final_body(const Params &P, const Bufs &B, int blk) {
     using C = CfgW<DIM, N, PHYS>;
     constexpr int M = C::M, NN = C::NN, NF = C::NF, NTR = C::NTR, FPT = C::FPT;
     __shared__ Smem<C> S;
-    const NodalTables &T = c_tab[N - 2];
     int lc, node;
     place<C>(lc, node);
     const int cell = blk * C::NCB + lc;
@@ -1491,36 +1650,20 @@ __device__ __forceinline__ void final_body(const Params &P, const Bufs &B, int b
                     flux_dir_ri<PHYS, DIM>(P, ui[j], dir, riI[j], fI);
                     flux_dir_ri<PHYS, DIM>(P, ue[j], dir, riE[j], fE);
                 }
-                bool upper = face & 1;  // R or T: the cell is on the lower side of the face
+                // fhat - f_int = (f_ext - f_int) / 2 -+ alpha (u_ext - u_int) / 2, the sign of the
+                // side: both cells of a face form the same differences
+                const double ba = (face & 1) ? -0.5 * P.b[i] * alpha : 0.5 * P.b[i] * alpha;
+                const double bh = 0.5 * P.b[i];
 #pragma unroll
                 for (int c = 0; c < M; ++c) {
-                    const double uLc = upper ? ui[j][c] : ue[j][c], uRc = upper ? ue[j][c] : ui[j][c];
-                    const double fLc = upper ? fI[c] : fE[c], fRc = upper ? fE[c] : fI[c];
-                    double fhat = 0.5 * (fLc + fRc) - 0.5 * alpha * (uRc - uLc);
-                    dc[j][c] = fma(P.b[i], fhat - fI[c], dc[j][c]);
+                    dc[j][c] = fma(bh, fE[c] - fI[c], dc[j][c]);
+                    dc[j][c] = fma(ba, ue[j][c] - ui[j][c], dc[j][c]);
                 }
             }
         }
         cell_sync<C>();
     }
-#pragma unroll
-    for (int j = 0; j < FPT; ++j) {
-        int fp = node + j * NN;
-        if (fp < NTR)
-#pragma unroll
-            for (int c = 0; c < M; ++c) S.c[lc].tf[fp][c] = dc[j][c];
-    }
-    cell_sync<C>();
-#pragma unroll
-    for (int c = 0; c < M; ++c) {
-        double cx = -T.liftp[a] * S.c[lc].tf[NF + b][c] + T.liftm[a] * S.c[lc].tf[b][c];
-        double corr = P.rhx * cx;
-        if constexpr (DIM == 2) {
-            double cy = -T.liftp[b] * S.c[lc].tf[3 * NF + a][c] + T.liftm[b] * S.c[lc].tf[2 * NF + a][c];
-            corr = fma(P.rhy, cy, corr);
-        }
-        u[c] = fma(P.dt, corr, u[c]);
-    }
+    lift_faces<C>(P, S.c[lc], node, a, b, dc, u);
     if (P.pk) project_pk<C>(S, lc, node, u);
     if (P.mode == MODE_OP_F) {
         if (active && solid_cell(P, cell))  // outside the domain: no operator
@@ -1538,31 +1681,30 @@ __device__ __forceinline__ void final_body(const Params &P, const Bufs &B, int b
             if (active) B.aux[(size_t)cell * M + c] = s;
         });
         cell_sync<C>();
-        if (node == 0 && own && !admissible<PHYS, DIM>(P, S.c[lc].avg)) atomicOr(B.flag, 1);
+        bool check = node == 0 && own;
+        if (check) {  // the FP32 screen of the average (truncated: 2^-22 of it) clears most cells
+            float v[M], e[M];
+#pragma unroll
+            for (int c = 0; c < M; ++c) {
+                v[c] = PHYS == PH_EULER ? trunc_f(S.c[lc].avg[c]) : (float)S.c[lc].avg[c];
+                e[c] = 2.384185791015625e-07f * fabsf(v[c]);
+            }
+            check = !screen_point<PHYS, DIM>(P, v, e);
+        }
+        if (check && !admissible<PHYS, DIM>(P, S.c[lc].avg)) atomicOr(B.flag, 1);
         store_node<DIM, N, PHYS>(P, B.unew, cell, node, active, u);
         return;
     }
     double pts[C::PPT][M];
-    limit_block(P, B, S, lc, node, own, u, pts, true, true);
+    float rhi;
+    const bool cleared = limit_block(P, B, S, lc, node, own, u, pts, true, true, true, rhi);
     // wave-speed rate of the new state over its S_K points (next trial step)
-    double amax = 0.0;
-#pragma unroll
-    for (int j = 0; j < C::PPT; ++j) {
-        int p = node + j * NN;
-        if (p < C::NSK && own) amax = fmax_nonneg(amax, sk_rate<PHYS, DIM>(P, pts[j]));
-    }
-    unsigned long long abits = dbits(amax);  // non-negative: the bits order as the values
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) abits = umax64(abits, __shfl_xor_sync(0xffffffffu, abits, o));
-    if ((threadIdx.x & 31) == 0 && abits > 0ull) atomicMax(B.a0, abits);
+    post_rate<C>(P, B, S, lc, node, own, cleared, rhi, pts);
     if (active && solid_cell(P, cell)) load_node<DIM, N, PHYS>(P, B.un, cell, node, true, u);  // keeps u^n
     store_node<DIM, N, PHYS>(P, B.unew, cell, node, active, u);
 }
 
-// Resident blocks per SM the FP64 final kernel's register budget is sized for: two of the
-// 2D Q^2 blocks (288 threads), five of the 128-thread ones.  Unbounded, the owned-box test of
-// the domain decomposition took the Q^2 kernel from 96 to 126 registers, one resident block,
-// and the 1024^2 Q^2 launch from 4.78 to 6.33 ms.
+// Resident blocks per SM the FP64 final kernel's register budget is sized for (96 registers).
 constexpr int fp64_final_min_blocks() { return 5; }
 
 template <int DIM, int N, int PHYS, bool STORED>
@@ -1572,8 +1714,7 @@ __global__ void __launch_bounds__(kWarpThreads, fp64_final_min_blocks())
 }
 
 // Limiter applied to a state (set-up projection, operator checks): un -> unew.  In
-// MODE_RATE it also posts the wave-speed rate of the limited state to B.a0: the
-// limiter leaves this thread's S_K values of the final nodal values in pts, the
+// MODE_RATE it also posts the wave-speed rate of the limited state to B.a0, from the
 // same interpolation of the same values that the scan kernel would take.
 template <int DIM, int N, int PHYS>
 __global__ void __launch_bounds__(kWarpThreads) k_limit(Params P, Bufs B) {
@@ -1589,19 +1730,9 @@ __global__ void __launch_bounds__(kWarpThreads) k_limit(Params P, Bufs B) {
     double u[C::M], pts[C::PPT][C::M];
     load_node<DIM, N, PHYS>(P, B.un, cell, node, active, u);
     if (P.pk) project_pk<C>(S, lc, node, u);  // a state set in P^k: its L2 projection first
-    limit_block(P, B, S, lc, node, own, u, pts, check, check, rate);
-    if (rate) {
-        double amax = 0.0;
-#pragma unroll
-        for (int j = 0; j < C::PPT; ++j) {
-            int p = node + j * C::NN;
-            if (p < C::NSK && own) amax = fmax(amax, sk_rate<PHYS, DIM>(P, pts[j]));
-        }
-        unsigned long long abits = dbits(amax);  // non-negative: the bits order as the values
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) abits = umax64(abits, __shfl_xor_sync(0xffffffffu, abits, o));
-        if ((threadIdx.x & 31) == 0 && abits > 0ull) atomicMax(B.a0, abits);
-    }
+    float rhi;
+    const bool cleared = limit_block(P, B, S, lc, node, own, u, pts, check, check, rate, rhi);
+    if (rate) post_rate<C>(P, B, S, lc, node, own, cleared, rhi, pts);
     if (active && solid_cell(P, cell)) load_node<DIM, N, PHYS>(P, B.un, cell, node, true, u);  // not limited
     store_node<DIM, N, PHYS>(P, B.unew, cell, node, active, u);
 }
@@ -1791,17 +1922,9 @@ __device__ __forceinline__ void trouble_body(const Params &P, const Bufs &B, int
         if (troubled) atomicAdd(B.ntrb, 1ull);
     }
     double pts[C::PPT][M];
-    limit_block(P, B, S, lc, node, active, u, pts, false, true);
-    double amax = 0.0;
-#pragma unroll
-    for (int j = 0; j < C::PPT; ++j) {
-        int p = node + j * NN;
-        if (p < C::NSK && active) amax = fmax_nonneg(amax, sk_rate<PHYS, DIM>(P, pts[j]));
-    }
-    unsigned long long abits = dbits(amax);  // non-negative: the bits order as the values
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) abits = umax64(abits, __shfl_xor_sync(0xffffffffu, abits, o));
-    if ((threadIdx.x & 31) == 0 && abits > 0ull) atomicMax(B.a0, abits);
+    float rhi;
+    const bool cleared = limit_block(P, B, S, lc, node, active, u, pts, false, true, true, rhi);
+    post_rate<C>(P, B, S, lc, node, active, cleared, rhi, pts);
     store_node<DIM, N, PHYS>(P, B.unew, cell, node, active, u);
 }
 

@@ -142,7 +142,8 @@ __global__ void __launch_bounds__(RunCfg1D<N, PHYS, NCBV>::NT) k_run1d(Params P,
                         cur_u[c] = v;
                     }
                     double pts[C::PPT][M];
-                    limit_block(P, B, S, lc, node, own, cur_u, pts, true, true, false);
+                    float rhi;
+                    limit_block(P, B, S, lc, node, own, cur_u, pts, true, true, false, rhi);
                 }
                 double trs[C::FPT][M];
                 const bool traced = P.slot[i] >= 0;
@@ -252,17 +253,9 @@ __global__ void __launch_bounds__(RunCfg1D<N, PHYS, NCBV>::NT) k_run1d(Params P,
                 for (int c = 0; c < M; ++c) u[c] = acc[c];
             }
             double pts[C::PPT][M];
-            limit_block(P, B, S, lc, node, own, u, pts, true, true);
-            double amax = 0.0;
-#pragma unroll
-            for (int j = 0; j < C::PPT; ++j) {
-                int p = node + j * NN;
-                if (p < C::NSK && own) amax = fmax_nonneg(amax, sk_rate<PHYS, 1>(P, pts[j]));
-            }
-            unsigned long long abits = dbits(amax);  // non-negative: the bits order as the values
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) abits = umax64(abits, __shfl_xor_sync(0xffffffffu, abits, o));
-            if ((threadIdx.x & 31) == 0 && abits > 0ull) atomicMax(B.a0, abits);
+            float rhi;
+            const bool cleared = limit_block(P, B, S, lc, node, own, u, pts, true, true, true, rhi);
+            post_rate<C>(P, B, S, lc, node, own, cleared, rhi, pts);
             if (own) store_node<1, N, PHYS>(P, unew, gc, node, true, u);
             __syncthreads();
         }

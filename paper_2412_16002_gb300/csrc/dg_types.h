@@ -119,6 +119,7 @@ struct Params {
     // hi rounded down (scr_on = 0: the screen clears nothing)
     int scr_on;
     float scr_eps, scr_lo, scr_hi;
+    float scr_rh[2], scr_gg;  // rate_bound: 2/h_x, 2/h_y and gamma (gamma - 1), rounded up
     int ind_stage;    // troubled-cell kernel: 0 decide and limit, 2 limit the given flags (the feature
                       // kernel decided), 3 combine the given plain flags with the learned
                       // probabilities, then limit; 4 (split path) decide, combine with the
@@ -223,6 +224,9 @@ inline void screen_bounds(Params &P) {
     P.scr_lo = P.scr_lo + in * fabsf(P.scr_lo);
     P.scr_hi = float_at_most(P.hi);
     P.scr_hi = P.scr_hi - in * fabsf(P.scr_hi);
+    P.scr_rh[0] = float_at_least(P.rhx);
+    P.scr_rh[1] = float_at_least(P.rhy);
+    P.scr_gg = float_at_least(P.gamma * (P.gamma - 1.0));
     P.scr_on = 1;
 }
 
