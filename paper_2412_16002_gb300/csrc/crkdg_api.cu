@@ -312,7 +312,7 @@ Params base_params(const crkdg_ctx *h) {
     P.gamma = h->flux.gamma;
     P.velx = h->flux.velocity[0];
     P.vely = h->flux.velocity[1];
-    fx_operator(P, crkdg_host_tables()[h->n - 2], h->dim, h->n);
+    fx_operator(P, crkdg_host_tables()[h->n - 2], h->dim, h->n, h->phys);
     P.lo = h->bounds.lo;
     P.hi = h->bounds.hi;
     P.eps = h->bounds.eps;
@@ -347,7 +347,8 @@ Bufs base_bufs(const crkdg_ctx *h) {
     B.unew = h->unew;
     B.tr = h->tr;
     B.tavg = h->tr ? h->tr + (size_t)h->tr_slots * h->m * h->ncell * h->ntr : nullptr;
-    B.tfs = h->tr ? h->tr + (size_t)h->tr_slots * h->m * h->ncell * (h->ntr + 1) : nullptr;
+    B.tsum = h->tr ? h->tr + (size_t)h->tr_slots * h->m * h->ncell * (h->ntr + 1) : nullptr;
+    B.tsp = h->tr ? B.tsum + (size_t)h->m * h->ncell * h->ntr : nullptr;
     B.flag = &h->scal->flag;
     B.nlim = &h->scal->nlim;
     B.thmin = &h->scal->thmin;
@@ -522,9 +523,11 @@ crkdg_status ensure_traces(crkdg_ctx *h, int slots) {
     if (h->tr) cudaFree(h->tr);
     h->tr = nullptr;
     h->tr_slots = 0;
-    // traces [slot][m][cell][face point], the traced stages' cell averages [slot][m][cell],
-    // then the traces' normal fluxes and spectral radii [slot][m + 1][cell][face point]
-    size_t bytes = ((size_t)slots * h->m * h->ncell * (h->ntr + 1) + (size_t)slots * (h->m + 1) * h->ncell * h->ntr) *
+    // traces [slot][m][cell][face point], the traced stages' cell averages [slot][m][cell], then
+    // the weighted sum of the traces' normal fluxes [m][cell][face point] and each stage's
+    // largest radius per face [slot][cell][face]
+    size_t bytes = ((size_t)slots * h->m * h->ncell * (h->ntr + 1) + (size_t)h->m * h->ncell * h->ntr +
+                    (size_t)slots * h->ncell * 2 * h->dim) *
                    sizeof(double);
     CK(h, cudaMalloc(&h->tr, bytes));
     h->tr_slots = slots;

@@ -421,7 +421,7 @@ crkdg_status crkdg_ensemble_create(int count, const crkdg_ens_problem *problems,
         P.gamma = flux->gamma;
         P.velx = flux->velocity[0];
         P.vely = flux->velocity[1];
-        fx_operator(P, crkdg_host_tables()[q.k - 1], 2, q.k + 1);
+        fx_operator(P, crkdg_host_tables()[q.k - 1], 2, q.k + 1, PH_EULER);
         P.lo = bounds->lo;
         P.hi = bounds->hi;
         P.eps = bounds->eps;

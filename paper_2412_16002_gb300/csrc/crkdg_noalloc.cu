@@ -101,7 +101,7 @@ extern "C" crkdg_status crkdg_apply_F_noalloc(const crkdg_mesh *mesh, int k, int
         P.bc[side] = (mesh->dim == 1 && side >= 2) ? BC_OUTFLOW : mesh->bc[side];
         for (int c = 0; c < MAXM; ++c) P.bcs[side][c] = mesh->bc_state[side][c];
     }
-    fx_operator(P, crkdg_host_tables()[n - 2], mesh->dim, n);
+    fx_operator(P, crkdg_host_tables()[n - 2], mesh->dim, n, flux->kind);
     for (int i = 0; i < MAXS; ++i) P.slot[i] = -1;
     P.s = 1;
     P.dt = 1.0;

@@ -75,6 +75,12 @@ __device__ __forceinline__ double fmax_nonneg(double a, double b) {
     return bitsd(umax64(dbits(a), dbits(b)));
 }
 
+// x / 2 on the integer units
+__device__ __forceinline__ double half_of(double x) {
+    const unsigned e = (unsigned)(dbits(x) >> 52) & 0x7ffu;
+    return e > 1u && e < 0x7ffu ? bitsd(dbits(x) - (1ull << 52)) : 0.5 * x;
+}
+
 // x truncated towards zero to FP32 on the integer units (a conversion instruction takes the FP64
 // pipe 64 cycles): below 2^-126 it is zero, beyond the FP32 range infinite (NaN included).
 __device__ __forceinline__ float trunc_f(double x) {
@@ -223,6 +229,63 @@ __device__ __forceinline__ double flux_speed_dir(const Params &P, const double *
     double ri = recip_rho<PHYS>(u);
     flux_dir_ri<PHYS, DIM>(P, u, dir, ri, f);
     return speed_dir_ri<PHYS, DIM>(P, u, dir, ri);
+}
+
+// Exponents outside this range (a state's components; zero is fine) take the FP64 forms: products of
+// three such values and their differences stay far from overflow and underflow.
+constexpr int kFxExpLo = 1023 - 150, kFxExpHi = 1023 + 150;
+__device__ __forceinline__ bool fx_range(double x) {
+    const int e = fx_exp(x);
+    return e == 0 ? !nonzero_bits(x) : (e >= kFxExpLo && e <= kFxExpHi);
+}
+// an Euler state that fx_point takes
+template <int DIM>
+__device__ __forceinline__ bool fx_state(const double *u) {
+    bool ok = positive_bits(u[0]) && positive_bits(u[DIM + 1]);
+#pragma unroll
+    for (int c = 0; c < DIM + 2; ++c) ok = ok && fx_range(u[c]);
+    return ok;
+}
+
+// Normal flux (FP64) of direction dir from the shared parts of a state, and its spectral radius.
+template <int DIM>
+__device__ __forceinline__ void fx_face_flux(const FxPoint<DIM> &o, const double *u, int dir, double *f) {
+    f[0] = u[1 + dir];
+    if constexpr (DIM == 1) {
+        f[1] = fx_value(o.q[0] + o.p, o.X);
+        f[2] = fx_value(fx_energy_flux<DIM>(o, 0), o.X + o.xw[0] + 1);
+    } else {
+        const double n = fx_value((dir ? o.q[1] : o.q[0]) + o.p, o.X), t = fx_value(o.c, o.X);
+        f[1] = dir ? t : n;
+        f[2] = dir ? n : t;
+        f[3] = fx_value(fx_energy_flux<DIM>(o, dir), o.X + (dir ? o.xw[1] : o.xw[0]) + 1);
+    }
+}
+template <int DIM>
+__device__ __forceinline__ double fx_face_speed(const FxGas &gas, const FxPoint<DIM> &o, int dir) {
+    const int d = DIM == 2 ? dir : 0;
+    const long long w = DIM == 2 && d ? o.w[DIM - 1] : o.w[0];
+    const int xw = DIM == 2 && d ? o.xw[DIM - 1] : o.xw[0];
+    double c = 0.0;  // sound speed: c^2 = gamma p / rho
+    if (o.p > 0) c = sqrt(fx_value(fx_mul(fx_limb(fx_mul(fx_limb(o.p), fx_limb(o.r))), gas.g), o.X - o.xr + 2));
+    return __dadd_rn(fx_value(w < 0 ? -w : w, xw), c);
+}
+
+// Normal flux f and spectral radius (returned) of one state at a face point: on the integer
+// units (dg_fixed.h: about 2^-60 where FP64 rounds at 2^-53 per operation, and no FP64 pipe but for
+// the conversions and the root) where the state allows it, a rule of the state alone, so that every
+// kernel gets the same bits for the same state.
+template <int PHYS, int DIM>
+__device__ __forceinline__ double face_flux(const Params &P, const double *u, int dir, bool want_speed, double *f) {
+    if constexpr (PHYS == PH_EULER) {
+        if (P.fx.on && fx_state<DIM>(u)) {
+            FxPoint<DIM> o;
+            fx_point<DIM>(u, P.fx.gas, o);
+            fx_face_flux<DIM>(o, u, dir, f);
+            return want_speed ? fx_face_speed<DIM>(P.fx.gas, o, dir) : 0.0;
+        }
+    }
+    return flux_speed_dir<PHYS, DIM>(P, u, dir, f);
 }
 
 // Trial-step rate at one point: sum over directions of lambda_d / h_d, so that
@@ -956,11 +1019,10 @@ __device__ void eval_G(const Params &P, Smem<C> &S, int lc, int node, const doub
                 trs[j][c] = s;
             }
             double f[M];
-            const double ri = recip_rho<PHYS>(trs[j]);
-            flux_dir_ri<PHYS, DIM>(P, trs[j], face >> 1, ri, f);
+            const double sp = face_flux<PHYS, DIM>(P, trs[j], face >> 1, want_speed, f);
 #pragma unroll
             for (int c = 0; c < M; ++c) S.c[lc].tf[fp][c] = f[c];
-            if (want_speed) S.c[lc].ts[fp] = speed_dir_ri<PHYS, DIM>(P, trs[j], face >> 1, ri);
+            if (want_speed) S.c[lc].ts[fp] = sp;
         }
     }
     cell_sync<C>();
@@ -1033,17 +1095,17 @@ __device__ __forceinline__ void load_fx(const Fx *p, Fx (&v)[N]) {
 }
 
 // Largest of each 16-bit half over the threads of a cell.
+__device__ __forceinline__ unsigned vmax_u16x2(unsigned a, unsigned b) {
+    unsigned r;
+    asm("max.u16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
 template <class C>
 __device__ __forceinline__ unsigned cell_max_halves(unsigned w, int node) {
-    auto vmax = [](unsigned a, unsigned b) {
-        unsigned r;
-        asm("max.u16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
-        return r;
-    };
     constexpr int NN = C::NN;
     if constexpr ((NN & (NN - 1)) == 0) {
 #pragma unroll
-        for (int o = 1; o < NN; o <<= 1) w = vmax(w, __shfl_xor_sync(0xffffffffu, w, o));
+        for (int o = 1; o < NN; o <<= 1) w = vmax_u16x2(w, __shfl_xor_sync(0xffffffffu, w, o));
     } else {  // rotations within the cell's lanes: windows of 2, 4, ... nodes until all are covered
         int l = threadIdx.x & 31;
         if (l >= C::CPW * NN) l = C::CPW * NN - 1;
@@ -1054,12 +1116,31 @@ __device__ __forceinline__ unsigned cell_max_halves(unsigned w, int node) {
             const int k = have + o <= NN && o == have ? o : NN - have;
             int src = node + k;
             if (src >= NN) src -= NN;
-            w = vmax(w, __shfl_sync(0xffffffffu, w, base + src));
+            w = vmax_u16x2(w, __shfl_sync(0xffffffffu, w, base + src));
             have += k;
             if (have >= NN) break;
         }
     }
     return w;
+}
+
+// Largest x (non-negative) over the threads of a face's points (NF consecutive nodes).
+template <class C>
+__device__ __forceinline__ double face_max(double x, int node) {
+    constexpr int NF = C::NF;
+    unsigned long long k = dbits(x);
+    if constexpr (NF == 3) {
+        int l = threadIdx.x & 31;
+        if (l >= C::CPW * C::NN) l = C::CPW * C::NN - 1;
+        const int r = node % 3, base = l - r;
+        const unsigned long long k1 = __shfl_sync(0xffffffffu, k, base + (r == 2 ? 0 : r + 1));
+        const unsigned long long k2 = __shfl_sync(0xffffffffu, k, base + (r == 0 ? 2 : r - 1));
+        k = umax64(k, umax64(k1, k2));
+    } else {
+#pragma unroll
+        for (int o = 1; o < NF; o <<= 1) k = umax64(k, __shfl_xor_sync(0xffffffffu, k, o));
+    }
+    return bitsd(k);
 }
 
 // Whether x holds for any thread of this thread's cell.
@@ -1070,128 +1151,196 @@ __device__ __forceinline__ bool cell_any(bool x, int node) {
     return ((__ballot_sync(0xffffffffu, x) >> (l - node)) & ((1u << C::NN) - 1u)) != 0u;
 }
 
-// Exponents outside this range (u's components; zero is fine) take the FP64 form: products of
-// three such values and their differences stay far from overflow and underflow.
-constexpr int kFxExpLo = 1023 - 150, kFxExpHi = 1023 + 150;
+// A cell's exponents of G's fluxes: comp 0, the momentum components, the last one (scalar laws: the
+// first only), two 16-bit fields per word.
+struct FluxExp {
+    unsigned w0, w1;
+};
+__device__ __forceinline__ unsigned biased_exp(int x) { return (unsigned)max(x + 1023, 0); }
 
 // G(u) with its linear maps in fixed point (dg_fixed.h): the stage's node values, then the
 // node and trace fluxes, share one exponent per cell and component, and the volume term, both
-// lifts and their sum are one sum of 2 n + 4 products (2D) per node and component on the integer units,
-// as are the traces and the cell average.  Fluxes and radii are FP64 functions of FP64 states.
-// tfl, tsp: normal fluxes and (want_speed) radii of this thread's traces; avg(c, value) is
-// called once per cell and component with want_avg.  Warp collective.
+// lifts and their sum are one sum of 2 n + 4 products (2D) per node and component on the integer
+// units, as are the traces and the cell average.  Euler fluxes are evaluated there too (fx_point):
+// the FP64 pipe keeps the conversions to FP64, the root of the sound speed and the stage sums.
+// put(j, trace, flux, radius) is called once for every face point of this thread (the radius the
+// largest of its face), avg(c, value) once per cell and component with want_avg.  Warp collective.
 //
-// Near vacuum (a density at a node or a trace 2^-20 below the cell's largest, or not positive)
-// and for values outside the exponent range the cell takes the FP64 form: a rule of the cell's
-// own values, so a cell's result does not depend on the cells it shares a warp with.
+// Near vacuum (a density at a node or a trace 2^-20 below the cell's largest, or not positive),
+// for an energy that is not positive and for values outside the exponent range the cell takes the
+// FP64 form: a rule of the cell's own values, so a cell's result does not depend on the cells it
+// shares a warp with.
 //
-// Bound by the FP64 fluxes that remain (about 70 FP64 instructions per warp and stage in Q^3 against
-// 145 with FP64 maps).  Set state, steps, get state: 513^2 Q^3, 2 RK4 steps 15.9 -> 11.8 ms; 1024^2
-// Q^2, 3 Heun steps 49.7 -> 40.0 ms (with the warp-synchronous layout of CfgW).
-template <class C, class Fn>
+// Why: with FP64 maps and fluxes a warp issued about 145 FP64 instructions per Q^3 stage, 76 cycles
+// each; now about 40, with 2100 instructions on the other pipes beside them.  Set state, steps, get
+// state: 513^2 Q^3, 2 RK4 steps 15.9 -> 11.8 (maps) -> 5.8 ms (fluxes and the final stage); 1024^2
+// Q^2, 3 Heun steps 49.7 -> 40.0 -> 22.2 ms.
+template <class C, class Put, class Fn>
 __device__ __forceinline__ void eval_G_fx(const Params &P, Smem<C> &S, const BlockTab<C> &Tb, int lc, int node,
-                                          const double *u, double *g, double (&trs)[C::FPT][C::M],
-                                          double (&tfl)[C::FPT][C::M], double (&tsp)[C::FPT], bool want_speed,
-                                          bool want_avg, Fn avg) {
+                                          const double *u, double *g, bool want_speed, bool want_avg, Put put,
+                                          Fn avg) {
     constexpr int DIM = C::D, N = C::NP, PHYS = C::PH;
     constexpr int M = C::M, NN = C::NN, NF = C::NF, NTR = C::NTR, FPT = C::FPT;
-    constexpr int W = (M + 1) / 2;  // words of two 16-bit exponents
+    constexpr int W = (M + 1) / 2;
     const int a = node % N, b = DIM == 2 ? node / N : 0;
+    CellData<C> &D = S.c[lc];
+    Fx(&fu)[M][NN] = reinterpret_cast<Fx(&)[M][NN]>(D.u);
+    Fx(&ff)[C::D][M][NN] = reinterpret_cast<Fx(&)[C::D][M][NN]>(D.f);
+    Fx(&ft)[M][NTR] = reinterpret_cast<Fx(&)[M][NTR]>(D.tf);
     auto field = [](const unsigned (&w)[W], int c) { return (int)((w[c >> 1] >> (16 * (c & 1))) & 0xffffu); };
-    // 1. node values in fixed point; node fluxes
-    unsigned eu[W];
     bool bad = P.fx.on == 0;
+    // 1. node values in fixed point
+    unsigned eu[W];
 #pragma unroll
     for (int k = 0; k < W; ++k) eu[k] = 0u;
 #pragma unroll
     for (int c = 0; c < M; ++c) {
-        const int e = fx_exp(u[c]);
-        if (e == 0 ? nonzero_bits(u[c]) : (e < kFxExpLo || e > kFxExpHi)) bad = true;
-        eu[c >> 1] |= (unsigned)e << (16 * (c & 1));
+        if (!fx_range(u[c])) bad = true;
+        eu[c >> 1] |= (unsigned)fx_exp(u[c]) << (16 * (c & 1));
     }
     const int e0 = eu[0] & 0xffffu;  // this node's density
 #pragma unroll
     for (int k = 0; k < W; ++k) eu[k] = cell_max_halves<C>(eu[k], node);
     if constexpr (PHYS == PH_EULER) {
-        if (!positive_bits(u[0]) || e0 < field(eu, 0) - 20) bad = true;
+        if (!positive_bits(u[0]) || !positive_bits(u[M - 1]) || e0 < field(eu, 0) - 20) bad = true;
     }
-    CellData<C> &D = S.c[lc];
-    Fx(&fu)[M][NN] = reinterpret_cast<Fx(&)[M][NN]>(D.u);
-    Fx(&ff)[C::D][M][NN] = reinterpret_cast<Fx(&)[C::D][M][NN]>(D.f);
-    Fx(&ft)[M][NTR] = reinterpret_cast<Fx(&)[M][NTR]>(D.tf);
     cell_sync<C>();  // earlier readers of the cell's arrays are done
 #pragma unroll
     for (int c = 0; c < M; ++c) fu[c][node] = fx_of(u[c], field(eu, c));
-    double fx[M], fy[M];
-    if constexpr (DIM == 2) {
-        flux_xy<PHYS>(P, u, fx, fy);
-    } else {
-        flux_dir<PHYS, DIM>(P, u, 0, fx);
-    }
     cell_sync<C>();
-    // 2. traces of this thread's face points, their fluxes and radii
+    // 2. traces of this thread's face points and their fluxes
+    FluxExp e{0u, 0u};
+    long long tm[FPT][M];  // mantissas of the normal fluxes (Euler)
+    int tx[FPT][3];        // their exponents: component 0, the momenta, the last
+    double tf0[FPT];       // scalar laws: the flux itself
+    double t[FPT][M];
 #pragma unroll
     for (int j = 0; j < FPT; ++j) {
         const int fp = node + j * NN;
         if (fp < NTR) {
             const int face = fp / NF, pos = fp - face * NF;
-            const bool row = DIM == 1 || face < 2;
+            const int at = DIM == 1 || face < 2 ? pos * N : pos, step = DIM == 1 || face < 2 ? 1 : N;
             Fx l[N];
             load_fx<N>(Tb.tl[face & 1], l);
 #pragma unroll
             for (int c = 0; c < M; ++c) {
                 FxSum s{0, 0};
-                if (row) {
-                    Fx v[N];
-                    load_fx<N>(&fu[c][pos * N], v);
 #pragma unroll
-                    for (int q = 0; q < N; ++q) fx_mac(s, v[q], l[q]);
-                } else {
-#pragma unroll
-                    for (int q = 0; q < N; ++q) fx_mac(s, fu[c][q * N + pos], l[q]);
-                }
-                trs[j][c] = fx_double(fx_sum(s), fx_shift(field(eu, c), kFxTrace));
+                for (int q = 0; q < N; ++q) fx_mac(s, fu[c][at + q * step], l[q]);
+                t[j][c] = fx_double(fx_sum(s), fx_shift(field(eu, c), kFxTrace));
             }
             if constexpr (PHYS == PH_EULER) {
-                if (!positive_bits(trs[j][0]) || fx_exp(trs[j][0]) < field(eu, 0) - 20) bad = true;
+                if (!fx_state<DIM>(t[j]) || fx_exp(t[j][0]) < field(eu, 0) - 20) bad = true;
             }
         }
     }
+    const bool any_bad = __any_sync(0xffffffffu, bad);
+    const bool mine = any_bad && cell_any<C>(bad, node);  // this cell takes the FP64 form below
 #pragma unroll
     for (int j = 0; j < FPT; ++j) {
         const int fp = node + j * NN;
+        double f[M], sp = 0.0;
         if (fp < NTR) {
-            const int face = fp / NF;
-            const double ri = recip_rho<PHYS>(trs[j]);
-            flux_dir_ri<PHYS, DIM>(P, trs[j], face >> 1, ri, tfl[j]);
-            if (want_speed) tsp[j] = speed_dir_ri<PHYS, DIM>(P, trs[j], face >> 1, ri);
+            const int dir = fp / NF >> 1;
+            if constexpr (PHYS == PH_EULER) {
+                FxPoint<DIM> o;
+                fx_point<DIM>(t[j], P.fx.gas, o);
+                if (want_speed) {
+                    fx_face_flux<DIM>(o, t[j], dir, f);
+                    sp = fx_face_speed<DIM>(P.fx.gas, o, dir);
+                }
+                const bool y = DIM == 2 && dir == 1;
+                const long long nf = (y ? o.q[DIM - 1] : o.q[0]) + o.p;
+                tm[j][0] = y ? o.m[DIM - 1] : o.m[0];
+                tm[j][1] = y ? o.c : nf;
+                if constexpr (DIM == 2) tm[j][2] = y ? nf : o.c;
+                tm[j][M - 1] = fx_energy_flux<DIM>(o, dir);
+                tx[j][0] = y ? o.xm[DIM - 1] : o.xm[0];
+                tx[j][1] = o.X;
+                tx[j][2] = o.X + (y ? o.xw[DIM - 1] : o.xw[0]) + 1;
+                e.w0 = vmax_u16x2(e.w0, biased_exp(tx[j][0]) | biased_exp(o.X + 1) << 16);
+                e.w1 = max(e.w1, biased_exp(tx[j][2] + 1));
+            } else {
+                sp = flux_speed_dir<PHYS, DIM>(P, t[j], dir, f);
+                tf0[j] = f[0];
+                e.w0 = max(e.w0, (unsigned)fx_exp(f[0]));
+            }
         }
+        if (want_speed) sp = face_max<C>(sp, node);
+        if (fp < NTR && !mine) put(j, t[j], f, sp);
     }
-    // 3. the fluxes of the cell in fixed point
-    unsigned ef[W];
+    if (want_avg) {
+        if constexpr (DIM == 2 && NN == 16 && M == 4) {  // four lanes of four nodes per component
+            const int c = node >> 2, r = node & 3;
+            FxSum s{0, 0};
+            Fx v[4], w[4];
+            load_fx<4>(&fu[c][4 * r], v);
+            load_fx<4>(&Tb.w[4 * r], w);
 #pragma unroll
-    for (int k = 0; k < W; ++k) ef[k] = 0u;
+            for (int q = 0; q < 4; ++q) fx_mac(s, v[q], w[q]);
+            long long x = fx_sum(s);
+            x += __shfl_xor_sync(0xffffffffu, x, 1);
+            x += __shfl_xor_sync(0xffffffffu, x, 2);
+            const double m = fx_double(x, fx_shift(field(eu, c), kFxAvg));
+            if (r == 0) avg(c, m);
+        } else {
+            for (int c = node; c < M; c += NN) {
+                FxSum s{0, 0};
 #pragma unroll
-    for (int c = 0; c < M; ++c) {
-        int e = fx_exp(fx[c]);
-        if constexpr (DIM == 2) e = max(e, fx_exp(fy[c]));
-#pragma unroll
-        for (int j = 0; j < FPT; ++j)
-            if (node + j * NN < NTR) e = max(e, fx_exp(tfl[j][c]));
-        ef[c >> 1] |= (unsigned)e << (16 * (c & 1));
+                for (int q = 0; q < NN; ++q) fx_mac(s, fu[c][q], Tb.w[q]);
+                avg(c, fx_double(fx_sum(s), fx_shift(field(eu, c), kFxAvg)));
+            }
+        }
+        __syncwarp();
     }
+    // 3. node fluxes; every flux of the cell in fixed point
+    if constexpr (PHYS == PH_EULER) {
+        FxPoint<DIM> o;
+        fx_point<DIM>(u, P.fx.gas, o);
+        long long h[DIM];
+        int xh = kFxNone, x0 = kFxNone;
 #pragma unroll
-    for (int k = 0; k < W; ++k) ef[k] = cell_max_halves<C>(ef[k], node);
+        for (int d = 0; d < DIM; ++d) {
+            h[d] = fx_energy_flux<DIM>(o, d);
+            xh = max(xh, o.X + o.xw[d] + 2);  // one more for 63 bits
+            x0 = max(x0, o.xm[d]);
+        }
+        e.w0 = vmax_u16x2(e.w0, biased_exp(x0) | biased_exp(o.X + 1) << 16);
+        e.w1 = max(e.w1, biased_exp(xh));
+        e.w0 = cell_max_halves<C>(e.w0, node);
+        e.w1 = cell_max_halves<C>(e.w1, node);
+        const int E0 = e.w0 & 0xffffu, E1 = e.w0 >> 16, E2 = e.w1;
 #pragma unroll
-    for (int c = 0; c < M; ++c) {
-        const int E = field(ef, c);
-        ff[0][c][node] = fx_of(fx[c], E);
-        if constexpr (DIM == 2) ff[1][c][node] = fx_of(fy[c], E);
+        for (int d = 0; d < DIM; ++d) {
+            ff[d][0][node] = fx_limbs(o.m[d], o.xm[d], E0);
+            ff[d][1 + d][node] = fx_limbs(o.q[d] + o.p, o.X, E1);
+            ff[d][M - 1][node] = fx_limbs(h[d], o.X + o.xw[d] + 1, E2);
+        }
+        if constexpr (DIM == 2) ff[0][2][node] = ff[1][1][node] = fx_limbs(o.c, o.X, E1);
 #pragma unroll
         for (int j = 0; j < FPT; ++j) {
             const int fp = node + j * NN;
-            if (fp < NTR) ft[c][fp] = fx_of(tfl[j][c], E);
+            if (fp < NTR) {
+                ft[0][fp] = fx_limbs(tm[j][0], tx[j][0], E0);
+                ft[1][fp] = fx_limbs(tm[j][1], tx[j][1], E1);
+                if constexpr (DIM == 2) ft[2][fp] = fx_limbs(tm[j][2], tx[j][1], E1);
+                ft[M - 1][fp] = fx_limbs(tm[j][M - 1], tx[j][2], E2);
+            }
         }
+    } else {
+        double fx[1], fy[1];
+        if constexpr (DIM == 2) {
+            flux_xy<PHYS>(P, u, fx, fy);
+            e.w0 = max(e.w0, (unsigned)fx_exp(fy[0]));
+        } else {
+            flux_dir<PHYS, DIM>(P, u, 0, fx);
+        }
+        e.w0 = cell_max_halves<C>(max(e.w0, (unsigned)fx_exp(fx[0])), node);
+        ff[0][0][node] = fx_of(fx[0], (int)e.w0);
+        if constexpr (DIM == 2) ff[1][0][node] = fx_of(fy[0], (int)e.w0);
+#pragma unroll
+        for (int j = 0; j < FPT; ++j)
+            if (node + j * NN < NTR) ft[0][node + j * NN] = fx_of(tf0[j], (int)e.w0);
     }
     cell_sync<C>();
     // 4. G: the row, the column and the four lifted face fluxes
@@ -1218,34 +1367,11 @@ __device__ __forceinline__ void eval_G_fx(const Params &P, Smem<C> &S, const Blo
                 fx_mac(s, ft[c][2 * NF + a], ly[0]);
                 fx_mac(s, ft[c][3 * NF + a], ly[1]);
             }
-            g[c] = fx_double(fx_sum(s), fx_shift(field(ef, c), P.fx.k));
+            const int E = (int)(c == 0 ? e.w0 & 0xffffu : c == M - 1 ? e.w1 : e.w0 >> 16);
+            g[c] = fx_double(fx_sum(s), fx_shift(E, P.fx.k));
         }
     }
-    if (want_avg) {
-        if constexpr (DIM == 2 && NN == 16 && M == 4) {  // four lanes of four nodes per component
-            const int c = node >> 2, r = node & 3;
-            FxSum s{0, 0};
-            Fx v[4], w[4];
-            load_fx<4>(&fu[c][4 * r], v);
-            load_fx<4>(&Tb.w[4 * r], w);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) fx_mac(s, v[q], w[q]);
-            long long x = fx_sum(s);
-            x += __shfl_xor_sync(0xffffffffu, x, 1);
-            x += __shfl_xor_sync(0xffffffffu, x, 2);
-            const double m = fx_double(x, fx_shift(field(eu, c), kFxAvg));
-            if (r == 0) avg(c, m);
-        } else {
-            for (int c = node; c < M; c += NN) {
-                FxSum s{0, 0};
-#pragma unroll
-                for (int q = 0; q < NN; ++q) fx_mac(s, fu[c][q], Tb.w[q]);
-                avg(c, fx_double(fx_sum(s), fx_shift(field(eu, c), kFxAvg)));
-            }
-        }
-    }
-    if (__any_sync(0xffffffffu, bad)) {  // a cell of the warp takes the FP64 form instead
-        const bool mine = cell_any<C>(bad, node);
+    if (any_bad) {
         double uu[M], gg[M], tt[FPT][M];
 #pragma unroll
         for (int c = 0; c < M; ++c) uu[c] = u[c];
@@ -1258,12 +1384,10 @@ __device__ __forceinline__ void eval_G_fx(const Params &P, Smem<C> &S, const Blo
             for (int j = 0; j < FPT; ++j) {
                 const int fp = node + j * NN;
                 if (fp < NTR) {
-#pragma unroll
-                    for (int c = 0; c < M; ++c) {
-                        trs[j][c] = tt[j][c];
-                        tfl[j][c] = D.tf[fp][c];
-                    }
-                    if (want_speed) tsp[j] = D.ts[fp];
+                    double sp = 0.0;
+                    if (want_speed)
+                        for (int q = 0; q < NF; ++q) sp = fmax_nonneg(sp, D.ts[fp / NF * NF + q]);
+                    put(j, tt[j], D.tf[fp], sp);
                 }
             }
         }
@@ -1391,7 +1515,7 @@ __device__ __forceinline__ void add_source(const Params &P, int cell, int node, 
 template <int DIM, int N, int PHYS>
 __device__ __forceinline__ void inner_body(const Params &P, const Bufs &B, int blk) {
     using C = CfgW<DIM, N, PHYS>;
-    constexpr int M = C::M, NN = C::NN, NTR = C::NTR, FPT = C::FPT;
+    constexpr int M = C::M, NN = C::NN, NTR = C::NTR;
     __shared__ Smem<C> S;
     __shared__ BlockTab<C> Tb;
     int lc, node;
@@ -1405,6 +1529,12 @@ __device__ __forceinline__ void inner_body(const Params &P, const Bufs &B, int b
 #pragma unroll
     for (int c = 0; c < M; ++c) cur[c] = acc[c] = un[c];
     __syncthreads();
+    const size_t at = (size_t)cell * NTR + node, cstr = (size_t)P.ncell * NTR;
+    double fs[C::FPT][M];  // sum_i b_i f(u_int^(i)) at this thread's face points
+#pragma unroll
+    for (int j = 0; j < C::FPT; ++j)
+#pragma unroll
+        for (int c = 0; c < M; ++c) fs[j][c] = 0.0;
     // not unrolled: four copies of a stage would not fit the instruction cache
 #pragma unroll 1
     for (int i = 0; i < P.s; ++i) {
@@ -1421,12 +1551,28 @@ __device__ __forceinline__ void inner_body(const Params &P, const Bufs &B, int b
             float rhi;
             limit_block(P, B, S, lc, node, own, cur, pts, true, true, false, rhi);
         }
-        double trs[FPT][M], tfl[FPT][M], tsp[FPT], g[M];
+        double g[M];
         const int slot = P.slot[i];
-        const bool keep_faces = slot >= 0 && B.tfs != nullptr;
-        eval_G_fx<C>(P, S, Tb, lc, node, cur, g, trs, tfl, tsp, keep_faces, slot >= 0, [&](int c, double s) {
-            if (active) B.tavg[((size_t)slot * M + c) * P.ncell + cell] = s;  // outflow exterior state
-        });
+        const bool traced = slot >= 0 && active;
+        const bool keep_faces = slot >= 0 && B.tsum != nullptr;
+        double *dst = B.tr + (size_t)max(slot, 0) * M * P.ncell * NTR;
+        eval_G_fx<C>(
+            P, S, Tb, lc, node, cur, g, keep_faces, slot >= 0,
+            [&](int j, const double *t, const double *f, double sp) {
+                if (traced)
+#pragma unroll
+                    for (int c = 0; c < M; ++c) dst[at + j * NN + c * cstr] = t[c];
+                if (keep_faces) {
+#pragma unroll
+                    for (int c = 0; c < M; ++c) fs[j][c] = fma(P.b[i], f[c], fs[j][c]);
+                    const int fp = node + j * NN;
+                    if (active && fp % C::NF == 0)
+                        B.tsp[((size_t)slot * P.ncell + cell) * (2 * DIM) + fp / C::NF] = sp;
+                }
+            },
+            [&](int c, double v) {
+                if (active) B.tavg[((size_t)slot * M + c) * P.ncell + cell] = v;  // outflow exterior state
+            });
         if (P.source && active) add_source<DIM, N, PHYS>(P, cell, node, i, g);
 #pragma unroll
         for (int c = 0; c < M; ++c) gh[i][c] = g[c];
@@ -1437,24 +1583,13 @@ __device__ __forceinline__ void inner_body(const Params &P, const Bufs &B, int b
 #pragma unroll
             for (int c = 0; c < M; ++c) acc[c] = fma(Tb.dtb[i], g[c], acc[c]);
         }
-        if (slot >= 0 && active) {
-            double *dst = B.tr + (size_t)slot * M * P.ncell * NTR;
-            double *dfs = keep_faces ? B.tfs + (size_t)slot * (M + 1) * P.ncell * NTR : nullptr;
-#pragma unroll
-            for (int j = 0; j < FPT; ++j) {
-                int fp = node + j * NN;
-                if (fp < NTR) {
-#pragma unroll
-                    for (int c = 0; c < M; ++c) dst[((size_t)c * P.ncell + cell) * NTR + fp] = trs[j][c];
-                    if (keep_faces) {
-#pragma unroll
-                        for (int c = 0; c < M; ++c) dfs[((size_t)c * P.ncell + cell) * NTR + fp] = tfl[j][c];
-                        dfs[((size_t)M * P.ncell + cell) * NTR + fp] = tsp[j];
-                    }
-                }
-            }
-        }
     }
+    if (B.tsum != nullptr && active)
+#pragma unroll
+        for (int j = 0; j < C::FPT; ++j)
+            if (node + j * NN < NTR)
+#pragma unroll
+                for (int c = 0; c < M; ++c) B.tsum[at + j * NN + c * cstr] = fs[j][c];
     if (P.pk) project_pk<C>(S, lc, node, acc);
     if (active && solid_cell(P, cell))  // outside the domain: G = 0, u* = u^n
 #pragma unroll
@@ -1547,10 +1682,10 @@ __device__ __forceinline__ void lift_faces(const Params &P, CellData<C> &D, int 
 // Final stage: u^{n+1} = u* + dt lift( sum_i b_i (fhat^(i) - f(u_int^(i))) ), then the
 // limiter, the admissibility test and a0 of the new state.  Each face flux is
 // evaluated from the same differences by both cells sharing the face, so the update is
-// conservative to round-off.  Bound by the FP64 pipe: 17 FP64 instructions per face point
-// and traced stage are left of 28, the lift runs in fixed point, and the rate is taken only by
-// warps that can raise it (513^2 Q^3, 2 RK4 steps with set and get 11.8 -> 8.3 ms; 1024^2 Q^2,
-// 3 Heun steps 40.0 -> 29.0 ms).
+// conservative to round-off.  Bound by the FP64 pipe: 9 FP64 instructions per face point and
+// traced stage are left of 28 (the inner kernel leaves the weighted flux sums, one set for all
+// stages, and the faces' radii), the lift runs in fixed point, and the rate is taken only by
+// warps that can raise it (513^2 Q^3: 1.15 ms a launch with the fluxes of every stage read back).
 template <int DIM, int N, int PHYS, bool STORED = false>
 __device__ __forceinline__ void final_body(const Params &P, const Bufs &B, int blk) {
     using C = CfgW<DIM, N, PHYS>;
@@ -1565,104 +1700,96 @@ __device__ __forceinline__ void final_body(const Params &P, const Bufs &B, int b
     double u[M];
     load_node<DIM, N, PHYS>(P, B.ustar, cell, node, active, u);
 
+    // dc = sum_i b_i (fhat^(i) - f_int^(i)) = (F_ext - F_int) / 2 -+ sum_i b_i alpha^(i) (u_ext^(i) - u_int^(i)) / 2
+    // with F = sum_i b_i f^(i), the sign of the side: both cells of a face form the same
+    // differences.  F and the faces' radii as the inner kernel stored them (STORED), else
+    // recomputed here; the exterior state of a boundary face always here.
+    CellData<C> &D = S.c[lc];
+    double(&sI)[NTR][M] = D.tf;  // this thread's running sums F (own face points only)
+    double(&sE)[NTR][M] = reinterpret_cast<double(&)[NTR][M]>(D.f);
+    const size_t cstr = (size_t)P.ncell * NTR;
     double dc[FPT][M];
+    size_t noff[FPT];  // the partner point's offset within a component's block
+    int nbr[FPT];
 #pragma unroll
-    for (int j = 0; j < FPT; ++j)
+    for (int j = 0; j < FPT; ++j) {
+        const int fp = node + j * NN;
+        nbr[j] = -1;
+        noff[j] = 0;
+        if (fp < NTR && active) {
+            const int face = fp / NF, pos = fp - face * NF;
+            nbr[j] = neighbour_geo(P, cell, face);
+            if (nbr[j] >= 0) noff[j] = (size_t)nbr[j] * NTR + (face ^ 1) * NF + pos;
+        }
 #pragma unroll
-        for (int c = 0; c < M; ++c) dc[j][c] = 0.0;
-
+        for (int c = 0; c < M; ++c) {
+            dc[j][c] = 0.0;
+            if (fp < NTR) sE[fp][c] = sI[fp][c] = 0.0;
+        }
+    }
     for (int i = 0; i < P.s; ++i) {
         if (P.slot[i] < 0) continue;
-        const double *tr = B.tr + (size_t)P.slot[i] * M * P.ncell * NTR;
-        // fluxes and spectral radii of interior traces: as the inner kernel stored them
-        // (STORED, B.tfs), else recomputed here; the exterior state of a boundary face
-        // always here
-        const double *tfs = STORED ? B.tfs + (size_t)P.slot[i] * (M + 1) * P.ncell * NTR : nullptr;
-        double ui[FPT][M], ue[FPT][M], riI[FPT], riE[FPT];
-        int nbr[FPT];
+        const double *tr = B.tr + (size_t)P.slot[i] * M * cstr;
+        const double *sps = STORED ? B.tsp + (size_t)P.slot[i] * P.ncell * (2 * DIM) : nullptr;
+        const double bi = P.b[i];
 #pragma unroll
         for (int j = 0; j < FPT; ++j) {
-            int fp = node + j * NN;
-            nbr[j] = -1;
+            const int fp = node + j * NN;
+            const int face = fp / NF, pos = fp - face * NF, dir = face >> 1;
+            double ui[M], ue[M], alpha = 0.0;
             if (fp < NTR && active) {
-                int face = fp / NF, pos = fp - face * NF;
+                const int nb = nbr[j];
+                double f[M];
 #pragma unroll
-                for (int c = 0; c < M; ++c) ui[j][c] = tr[((size_t)c * P.ncell + cell) * NTR + fp];
-                int nb = neighbour_geo(P, cell, face);
-                nbr[j] = nb;
-                int ofp = (face ^ 1) * NF + pos;
+                for (int c = 0; c < M; ++c) ui[c] = tr[c * cstr + (size_t)cell * NTR + fp];
+                if constexpr (STORED) {
+                    alpha = sps[(size_t)cell * (2 * DIM) + face];
+                } else {
+                    alpha = fmax_nonneg(alpha, face_flux<PHYS, DIM>(P, ui, dir, true, f));
+#pragma unroll
+                    for (int c = 0; c < M; ++c) sI[fp][c] = fma(bi, f[c], sI[fp][c]);
+                }
                 if (nb >= 0) {
 #pragma unroll
-                    for (int c = 0; c < M; ++c) ue[j][c] = tr[((size_t)c * P.ncell + nb) * NTR + ofp];
+                    for (int c = 0; c < M; ++c) ue[c] = tr[c * cstr + noff[j]];
+                    if constexpr (STORED) alpha = fmax_nonneg(alpha, sps[(size_t)nb * (2 * DIM) + (face ^ 1)]);
                 } else {
                     double av[M];
 #pragma unroll
                     for (int c = 0; c < M; ++c) av[c] = B.tavg[((size_t)P.slot[i] * M + c) * P.ncell + cell];
                     if (P.geo != nullptr)
-                        geo_exterior<PHYS, DIM, N>(P, cell, face, pos, i, ui[j], av, ue[j]);
+                        geo_exterior<PHYS, DIM, N>(P, cell, face, pos, i, ui, av, ue);
                     else
-                        exterior_state<PHYS, DIM>(P, face, ui[j], av, ue[j]);
+                        exterior_state<PHYS, DIM>(P, face, ui, av, ue);
                 }
-                int dir = face >> 1;
-                double sI, sE;
-                if constexpr (STORED) {
-                    sI = tfs[((size_t)M * P.ncell + cell) * NTR + fp];
-                    if (nb >= 0) {
-                        sE = tfs[((size_t)M * P.ncell + nb) * NTR + ofp];
-                    } else {
-                        riE[j] = recip_rho<PHYS>(ue[j]);
-                        sE = speed_dir_ri<PHYS, DIM>(P, ue[j], dir, riE[j]);
-                    }
-                } else {
-                    riI[j] = recip_rho<PHYS>(ui[j]);
-                    riE[j] = recip_rho<PHYS>(ue[j]);
-                    sI = speed_dir_ri<PHYS, DIM>(P, ui[j], dir, riI[j]);
-                    sE = speed_dir_ri<PHYS, DIM>(P, ue[j], dir, riE[j]);
-                }
-                S.c[lc].al[fp] = fmax_nonneg(sI, sE);
-            } else if (fp < NTR) {
-                S.c[lc].al[fp] = 0.0;
-            }
-        }
-        cell_sync<C>();
+                if (!STORED || nb < 0) {
+                    alpha = fmax_nonneg(alpha, face_flux<PHYS, DIM>(P, ue, dir, true, f));
 #pragma unroll
-        for (int j = 0; j < FPT; ++j) {
-            int fp = node + j * NN;
+                    for (int c = 0; c < M; ++c) sE[fp][c] = fma(bi, f[c], sE[fp][c]);
+                }
+            }
+            __syncwarp();
+            alpha = face_max<C>(alpha, node);  // per-edge LF viscosity: max over the edge's points
             if (fp < NTR && active) {
-                int face = fp / NF, pos = fp - face * NF;
-                int dir = face >> 1;
-                double alpha = 0.0;  // per-edge LF viscosity: max over the edge's points
+                const double h = half_of(bi);
+                const double ba = ((face & 1) ? -h : h) * alpha;
 #pragma unroll
-                for (int q = 0; q < NF; ++q) alpha = fmax_nonneg(alpha, S.c[lc].al[face * NF + q]);
-                double fI[M], fE[M];
-                const int nb = nbr[j];
-                if constexpr (STORED) {
-#pragma unroll
-                    for (int c = 0; c < M; ++c) fI[c] = tfs[((size_t)c * P.ncell + cell) * NTR + fp];
-                    if (nb >= 0) {
-                        const int ofp = (face ^ 1) * NF + pos;
-#pragma unroll
-                        for (int c = 0; c < M; ++c) fE[c] = tfs[((size_t)c * P.ncell + nb) * NTR + ofp];
-                    } else {
-                        flux_dir_ri<PHYS, DIM>(P, ue[j], dir, riE[j], fE);
-                    }
-                } else {
-                    flux_dir_ri<PHYS, DIM>(P, ui[j], dir, riI[j], fI);
-                    flux_dir_ri<PHYS, DIM>(P, ue[j], dir, riE[j], fE);
-                }
-                // fhat - f_int = (f_ext - f_int) / 2 -+ alpha (u_ext - u_int) / 2, the sign of the
-                // side: both cells of a face form the same differences
-                const double ba = (face & 1) ? -0.5 * P.b[i] * alpha : 0.5 * P.b[i] * alpha;
-                const double bh = 0.5 * P.b[i];
-#pragma unroll
-                for (int c = 0; c < M; ++c) {
-                    dc[j][c] = fma(bh, fE[c] - fI[c], dc[j][c]);
-                    dc[j][c] = fma(ba, ue[j][c] - ui[j][c], dc[j][c]);
-                }
+                for (int c = 0; c < M; ++c) dc[j][c] = fma(ba, ue[c] - ui[c], dc[j][c]);
             }
         }
-        cell_sync<C>();
     }
+#pragma unroll
+    for (int j = 0; j < FPT; ++j) {
+        const int fp = node + j * NN;
+        if (fp < NTR && active)
+#pragma unroll
+            for (int c = 0; c < M; ++c) {
+                const double FI = STORED ? B.tsum[c * cstr + (size_t)cell * NTR + fp] : sI[fp][c];
+                const double FE = STORED && nbr[j] >= 0 ? B.tsum[c * cstr + noff[j]] : sE[fp][c];
+                dc[j][c] = fma(0.5, FE - FI, dc[j][c]);
+            }
+    }
+    cell_sync<C>();
     lift_faces<C>(P, S.c[lc], node, a, b, dc, u);
     if (P.pk) project_pk<C>(S, lc, node, u);
     if (P.mode == MODE_OP_F) {
@@ -2068,7 +2195,7 @@ cudaError_t launch_one(int kernel, cudaStream_t st, const Params &P, const Bufs 
     switch (kernel) {
     case K_INNER: k_inner<DIM, N, PHYS><<<nblocks, C::NT, 0, st>>>(P, B); break;
     case K_FINAL:
-        if (B.tfs)
+        if (B.tsum)
             k_final<DIM, N, PHYS, true><<<nblocks, C::NT, 0, st>>>(P, B);
         else
             k_final<DIM, N, PHYS, false><<<nblocks, C::NT, 0, st>>>(P, B);

@@ -23,7 +23,7 @@ __device__ __forceinline__ void ens_bufs(const EnsProblem &E, Bufs &B) {
     B.ustar = E.ustar;
     B.tr = E.tr;
     B.tavg = E.tavg;
-    B.tfs = nullptr;  // the final kernel recomputes the traces' fluxes
+    B.tsum = B.tsp = nullptr;  // the final kernel recomputes the traces' fluxes
     B.flag = &E.sc->flag;
     B.nlim = &E.sc->nlim;
     B.thmin = &E.sc->thmin;

@@ -96,6 +96,130 @@ CRKDG_HD double fx_double(long long x, int sh) {
 // the shift of a sum of values with exponent E and coefficients scaled by 2^k
 CRKDG_HD int fx_shift(int E, int k) { return E - 1025 - k; }
 
+// ----------------------------------------------------------------------- Euler fluxes
+//
+// The nonlinear part on the integer units: a value is m 2^(x - 61), m a signed 64-bit mantissa
+// (62 bits from an FP64 number), so a product is three IMAD.WIDE and a shift where FP64 takes
+// its pipe 76 cycles, and keeps about 60 bits.
+
+// 31-bit limbs of a mantissa |m| < 2^62
+struct Limb {
+    int h, l;
+};
+CRKDG_HD Limb fx_limb(long long m) { return Limb{(int)(m >> 31), (int)m & 0x7fffffff}; }
+// a b 2^-62 (value exponents: x_a + x_b + 1), within 2 units
+CRKDG_HD long long fx_mul(const Limb &a, const Limb &b) {
+    long long t = (long long)a.h * b.l;
+    t += (long long)a.l * b.h;
+    return (long long)a.h * b.h + (t >> 31);
+}
+// a b 2^-61 (value exponents: x_a + x_b), for |a b| < 2^124: up to 63 bits
+CRKDG_HD long long fx_mul_wide(const Limb &a, const Limb &b) {
+    long long t = (long long)a.h * b.l;
+    t += (long long)a.l * b.h;
+    return 2 * ((long long)a.h * b.h) + (t >> 30);
+}
+// m 2^-s, s >= 0 (rounded down)
+CRKDG_HD long long fx_shr(long long m, int s) { return m >> (s > 63 ? 63 : s); }
+
+// mantissa of x (exponent fx_exp(x) - 1023); zero and subnormal numbers give zero
+CRKDG_HD long long fx_mant(double x) {
+    const unsigned long long b = fx_bits(x);
+    long long m = (long long)(((b & 0xfffffffffffffull) | 0x10000000000000ull) << 9);
+    if ((long long)b < 0) m = -m;
+    if (((b >> 52) & 0x7ff) == 0) m = 0;
+    return m;
+}
+
+// 2^122 / M for M in [2^61, 2^62): the FP32 reciprocal of M's leading bits (2^-22), then
+// r (1 + e + e^2) with e = 1 - M r to 2^-60.
+CRKDG_HD long long fx_recip(long long M) {
+    const unsigned fb = 0x3f800000u | ((unsigned)(M >> 38) & 0x7fffffu);
+#ifdef __CUDA_ARCH__
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(__uint_as_float(fb)));
+    const int r0 = __float2int_rn(y * 1073741824.0f);
+#else
+    float f;
+    memcpy(&f, &fb, 4);
+    const int r0 = (int)lrintf((1.0f / f) * 1073741824.0f);
+#endif
+    const Limb m = fx_limb(M);
+    long long e = (1ll << 60) - (long long)m.h * r0;
+    e -= ((long long)m.l * r0) >> 31;
+    const int eh = (int)(e >> 8);  // |e| < 2^38
+    e += ((long long)eh * eh) >> 44;
+    const long long w = (long long)r0 * (int)(e >> 8) + (((long long)r0 * ((int)e & 255)) >> 8);
+    return ((long long)r0 << 31) + (w >> 21);
+}
+
+// gamma - 1 and gamma as mantissas: g1 2^-62 and g 2^(-61)
+struct FxGas {
+    Limb g1, g;
+};
+
+// Everything the fluxes of one state share.  Exponents are those of the values (m 2^(x - 61));
+// q[d] = m_d w_d, c = m_x w_y, p and H = E + p share the exponent X (H halved: X + 1).
+template <int DIM>
+struct FxPoint {
+    long long m[DIM], w[DIM], q[DIM], c, p, hh, r;
+    int xm[DIM], xw[DIM], xr, X;
+};
+constexpr int kFxNone = -4000;  // exponent of a zero
+
+// For rho > 0, E > 0, exponents within the fixed-point range and gamma < 2.
+template <int DIM>
+CRKDG_HD void fx_point(const double *u, const FxGas &gas, FxPoint<DIM> &o) {
+    o.xr = fx_exp(u[0]) - 1023;
+    o.r = fx_recip(fx_mant(u[0]));
+    const Limb R = fx_limb(o.r);
+    const int xe = fx_exp(u[DIM + 1]) - 1023;
+    o.X = xe;
+    Limb lm[DIM], lw[DIM];
+    int xq[DIM];
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) {
+        const int e = fx_exp(u[1 + d]);
+        o.xm[d] = e == 0 ? kFxNone : e - 1023;
+        o.m[d] = fx_mant(u[1 + d]);
+        lm[d] = fx_limb(o.m[d]);
+        o.w[d] = fx_mul_wide(lm[d], R);  // R <= 2^61: below 2^62
+        o.xw[d] = o.xm[d] - o.xr;
+        lw[d] = fx_limb(o.w[d]);
+        xq[d] = o.xm[d] + o.xw[d] + 1;
+        o.X = o.X > xq[d] ? o.X : xq[d];
+    }
+    long long k = 0;
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) {
+        o.q[d] = fx_shr(fx_mul(lm[d], lw[d]), o.X - xq[d]);
+        k += o.q[d];
+    }
+    o.c = 0;
+    if (DIM == 2) o.c = fx_shr(fx_mul(lm[0], lw[DIM - 1]), o.X - (o.xm[0] + o.xw[DIM - 1] + 1));
+    const long long E = fx_shr(fx_mant(u[DIM + 1]), o.X - xe);
+    o.p = fx_mul(fx_limb(E - (k >> 1)), gas.g1);
+    o.hh = (E + o.p) >> 1;
+}
+
+// (E + p) w_d, exponent X + xw[d] + 1, up to 63 bits
+template <int DIM>
+CRKDG_HD long long fx_energy_flux(const FxPoint<DIM> &o, int d) {
+    return fx_mul_wide(fx_limb(o.hh), fx_limb(DIM == 2 && d == 1 ? o.w[DIM - 1] : o.w[0]));
+}
+
+// limbs (dg_fixed's 59 bits) of m 2^(x - 61) in units of 2^(E - 1081), E - 1023 >= x (and one more
+// for |m| >= 2^62)
+CRKDG_HD Fx fx_limbs(long long m, int x, int E) {
+    const long long v = fx_shr(m, E - 1023 - x + 3);
+    Fx r;
+    r.h = (int)(v >> 28);
+    r.l = (int)v & 0xfffffff;
+    return r;
+}
+// m 2^(x - 61) as FP64
+CRKDG_HD double fx_value(long long m, int x) { return fx_double(m, x - 61); }
+
 // coefficient c scaled by 2^k, |c| 2^k < 2^58 (host)
 inline Fx fx_coef(double c, int k) {
     const long long C = llrint(ldexp(c, k));

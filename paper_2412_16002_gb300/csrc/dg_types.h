@@ -82,6 +82,7 @@ constexpr int kFxAvg = 57;    // the weights sum to 1
 struct FxOp {
     Fx cx[MAXN][MAXN], cy[MAXN][MAXN];
     Fx lx[MAXN][2], ly[MAXN][2];  // [0] the lower face, [1] the upper one
+    FxGas gas;                    // Euler, 1 < gamma < 2 (on = 0 otherwise)
     int k, on;
 };
 
@@ -176,7 +177,7 @@ inline void tvb_thresholds(Params &P) {
 }
 
 // The fixed-point coefficients of G from rhx, rhy and the tables of the degree (host side).
-inline void fx_operator(Params &P, const NodalTables &T, int dim, int n) {
+inline void fx_operator(Params &P, const NodalTables &T, int dim, int n, int phys) {
     FxOp &F = P.fx;
     memset(&F, 0, sizeof(F));
     double sx = 0.0, sy = 0.0;  // largest row sums
@@ -189,7 +190,12 @@ inline void fx_operator(Params &P, const NodalTables &T, int dim, int n) {
     auto moderate = [](double x) { return x == 0.0 || (fabs(x) > 0x1p-100 && fabs(x) < 0x1p100); };
     const double s = sx + sy;
     F.on = isfinite(s) && s > 0x1p-100 && s < 0x1p100 && moderate(P.gamma) && moderate(P.velx) && moderate(P.vely);
+    if (phys == PH_EULER) F.on = F.on && P.gamma > 1.0 && P.gamma < 2.0;
     if (!F.on) return;
+    if (phys == PH_EULER) {
+        F.gas.g1 = fx_limb(llrint(ldexp(P.gamma - 1.0, 62)));
+        F.gas.g = fx_limb(llrint(ldexp(P.gamma, 61)));
+    }
     int e;
     frexp(s, &e);  // s < 2^e
     F.k = 58 - e;
@@ -236,8 +242,10 @@ struct Bufs {
     double *unew;       // u^{n+1}
     double *tr;         // face traces of u~^(i): [slot][m][cell][face point]
     double *tavg;       // cell averages of the same u~^(i): [slot][m][cell] (outflow exterior state)
-    double *tfs = nullptr;  // optional: normal fluxes and spectral radii of the traces,
-                            // [slot][m + 1][cell][face point] (the final kernel recomputes them when null)
+    // optional (both or none; without them the final kernel recomputes): sum_i b_i f(u_int^(i)) . nu of
+    // the traces [m][cell][face point], and each traced stage's largest radius over a face's
+    // points [slot][cell][face]
+    double *tsum = nullptr, *tsp = nullptr;
     int *flag;          // set when a stage average leaves B
     unsigned long long *nlim;   // limited cells
     unsigned long long *thmin;  // bits of the smallest theta (non-negative double)
