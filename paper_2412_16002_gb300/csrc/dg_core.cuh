@@ -231,19 +231,16 @@ __device__ __forceinline__ double flux_speed_dir(const Params &P, const double *
     return speed_dir_ri<PHYS, DIM>(P, u, dir, ri);
 }
 
-// Exponents outside this range (a state's components; zero is fine) take the FP64 forms: products of
-// three such values and their differences stay far from overflow and underflow.
+// Largest exponent of a state's components (and smallest of the density) that the integer forms
+// take: products of three such values and their differences stay far from overflow.  Small
+// momenta and energies need no bound; results below 2^-1022 become zero.
 constexpr int kFxExpLo = 1023 - 150, kFxExpHi = 1023 + 150;
-__device__ __forceinline__ bool fx_range(double x) {
-    const int e = fx_exp(x);
-    return e == 0 ? !nonzero_bits(x) : (e >= kFxExpLo && e <= kFxExpHi);
-}
 // an Euler state that fx_point takes
 template <int DIM>
 __device__ __forceinline__ bool fx_state(const double *u) {
-    bool ok = positive_bits(u[0]) && positive_bits(u[DIM + 1]);
+    bool ok = positive_bits(u[0]) && positive_bits(u[DIM + 1]) && fx_exp(u[0]) >= kFxExpLo;
 #pragma unroll
-    for (int c = 0; c < DIM + 2; ++c) ok = ok && fx_range(u[c]);
+    for (int c = 0; c < DIM + 2; ++c) ok = ok && fx_exp(u[c]) <= kFxExpHi;
     return ok;
 }
 
@@ -1173,8 +1170,8 @@ __device__ __forceinline__ unsigned biased_exp(int x) { return (unsigned)max(x +
 //
 // Why: with FP64 maps and fluxes a warp issued about 145 FP64 instructions per Q^3 stage, 76 cycles
 // each; now about 40, with 2100 instructions on the other pipes beside them.  Set state, steps, get
-// state: 513^2 Q^3, 2 RK4 steps 15.9 -> 11.8 (maps) -> 5.8 ms (fluxes and the final stage); 1024^2
-// Q^2, 3 Heun steps 49.7 -> 40.0 -> 22.2 ms.
+// state: 513^2 Q^3, 2 RK4 steps 15.9 -> 11.8 (maps) -> 5.8 (fluxes and the final stage) -> 5.0 ms (no
+// fallback for small momenta); 1024^2 Q^2, 3 Heun steps 49.7 -> 40.0 -> 22.2 ms.
 template <class C, class Put, class Fn>
 __device__ __forceinline__ void eval_G_fx(const Params &P, Smem<C> &S, const BlockTab<C> &Tb, int lc, int node,
                                           const double *u, double *g, bool want_speed, bool want_avg, Put put,
@@ -1195,14 +1192,14 @@ __device__ __forceinline__ void eval_G_fx(const Params &P, Smem<C> &S, const Blo
     for (int k = 0; k < W; ++k) eu[k] = 0u;
 #pragma unroll
     for (int c = 0; c < M; ++c) {
-        if (!fx_range(u[c])) bad = true;
+        if (fx_exp(u[c]) > kFxExpHi) bad = true;
         eu[c >> 1] |= (unsigned)fx_exp(u[c]) << (16 * (c & 1));
     }
     const int e0 = eu[0] & 0xffffu;  // this node's density
 #pragma unroll
     for (int k = 0; k < W; ++k) eu[k] = cell_max_halves<C>(eu[k], node);
     if constexpr (PHYS == PH_EULER) {
-        if (!positive_bits(u[0]) || !positive_bits(u[M - 1]) || e0 < field(eu, 0) - 20) bad = true;
+        if (!fx_state<DIM>(u) || e0 < field(eu, 0) - 20) bad = true;
     }
     cell_sync<C>();  // earlier readers of the cell's arrays are done
 #pragma unroll
@@ -1621,7 +1618,7 @@ __device__ __forceinline__ void lift_faces(const Params &P, CellData<C> &D, int 
         for (int j = 0; j < FPT; ++j)
             if (node + j * NN < NTR) {
                 const int ej = fx_exp(dc[j][c]);
-                if (ej == 0 ? nonzero_bits(dc[j][c]) : (ej < 1023 - 600 || ej > 1023 + 600)) bad = true;
+                if (ej > 1023 + 800) bad = true;
                 e = max(e, ej);
             }
         ef[c >> 1] |= (unsigned)e << (16 * (c & 1));

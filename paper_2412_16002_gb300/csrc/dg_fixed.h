@@ -84,14 +84,18 @@ CRKDG_HD void fx_mac(FxSum &s, const Fx &v, const Fx &c) {
 // the sum in units of 2^56 2^(E - 1081) 2^-k
 CRKDG_HD long long fx_sum(const FxSum &s) { return s.hh + (s.mid >> 28); }
 
-// x 2^sh as FP64, rounded to nearest.  The result's exponent must be in the normal range.
+// x 2^sh as FP64, rounded to nearest (below 2^-1022 zero).  The result must not overflow.
 CRKDG_HD double fx_double(long long x, int sh) {
 #ifdef __CUDA_ARCH__
     const double r = __ll2double_rn(x);
+    const int hi = __double2hiint(r), e = (hi >> 20) & 0x7ff;
+    const bool z = e == 0 || e + sh <= 0;
+    return __hiloint2double(z ? 0 : hi + sh * 0x100000, z ? 0 : __double2loint(r));
 #else
     const double r = (double)x;
+    const int e = fx_exp(r);
+    return e == 0 || e + sh <= 0 ? 0.0 : fx_from_bits(fx_bits(r) + ((unsigned long long)(long long)sh << 52));
 #endif
-    return x == 0 ? 0.0 : fx_from_bits(fx_bits(r) + ((unsigned long long)(long long)sh << 52));
 }
 // the shift of a sum of values with exponent E and coefficients scaled by 2^k
 CRKDG_HD int fx_shift(int E, int k) { return E - 1025 - k; }
@@ -167,7 +171,7 @@ struct FxPoint {
 };
 constexpr int kFxNone = -4000;  // exponent of a zero
 
-// For rho > 0, E > 0, exponents within the fixed-point range and gamma < 2.
+// For rho > 0, E > 0, exponents below the overflow bounds (fx_state) and gamma < 2.
 template <int DIM>
 CRKDG_HD void fx_point(const double *u, const FxGas &gas, FxPoint<DIM> &o) {
     o.xr = fx_exp(u[0]) - 1023;
