@@ -273,7 +273,7 @@ struct crkdg_ctx {
     int own[4] = {0, 0, 0, 0};
     bool metric_on = false;       // cell sizes taken from the global mesh of a subdomain
     double rhx_g = 0.0, rhy_g = 0.0;
-    bool tc_on = true;            // split path: inner stages on the tensor cores where built
+    bool tc_on = false;           // split path: Q^3 inner stages on the tensor cores
     double *fst = nullptr;        // standard RKDG: F of each stage, then two stage buffers
     int fst_slots = 0;
     double *mass_part = nullptr;  // block sums of the component totals
@@ -422,10 +422,11 @@ void fill_f32(Params &P) {
     F.dt = (float)P.dt;
 }
 
-// The tensor-core inner stages serve 2D Euler Q^3 steps whose tableau has only a
-// sub-diagonal (every tableau of the paper); other cases run k_inner_x.
-bool use_tc(const crkdg_ctx *h, const Params &P) {
-    if (!h->tc_on || h->dim != 2 || h->phys != PH_EULER || h->n != 4 || P.mode != MODE_STEP) return false;
+// 2D Euler steps whose tableau has only a sub-diagonal (every tableau of the paper) run the inner
+// stages with one thread per cell, or for Q^3 on request on the tensor cores; other cases run
+// k_inner_x.
+bool sub_diagonal_euler(const crkdg_ctx *h, const Params &P) {
+    if (h->dim != 2 || h->phys != PH_EULER || P.mode != MODE_STEP) return false;
     for (int i = 0; i < P.s; ++i)
         for (int j = 0; j + 1 < i; ++j)
             if (P.A[i][j] != 0.0) return false;
@@ -436,7 +437,8 @@ cudaError_t launch_x(crkdg_ctx *h, int kernel, const Params &P0, const MixBufs &
     if ((kernel == KX_INNER || kernel == KX_FINAL) && !slots_ok(P0, X.tr, X.tavg)) return cudaErrorInvalidValue;
     Params P = P0;
     fill_f32(P);
-    if (kernel == KX_INNER && use_tc(h, P)) return crkdg_launch_inner_tc(h->st, P, X);
+    if (kernel == KX_INNER && sub_diagonal_euler(h, P))
+        return h->tc_on && h->n == 4 ? crkdg_launch_inner_tc(h->st, P, X) : crkdg_launch_inner_cell(h->n, h->st, P, X);
     int ncb = cells_per_block(h->dim, h->n);
     int nblocks = (h->ncell + ncb - 1) / ncb;
     if (h->dim == 1) return crkdg_launch_mx_1d(kernel, h->n, h->phys, nblocks, h->st, P, X);

@@ -1,6 +1,7 @@
 // dg_2d.cu -- 2D instantiations of the FP64 cRKDG kernels (see dg_core.cuh).
 #include "dg_core.cuh"
 #include "dg_mixed.cuh"
+#include "dg_cell.cuh"
 #include "dg_tc.cuh"
 
 using namespace crkdg;
@@ -21,4 +22,13 @@ cudaError_t crkdg_launch_mx_2d(int kernel, int n, int phys, int nblocks, cudaStr
 
 cudaError_t crkdg_launch_inner_tc(cudaStream_t st, const Params &P, const MixBufs &X) {
     return launch_inner_tc(st, P, X);
+}
+
+cudaError_t crkdg_launch_inner_cell(int n, cudaStream_t st, const Params &P, const MixBufs &X) {
+    switch (n) {
+    case 2: return launch_inner_c<2>(st, P, X);
+    case 3: return launch_inner_c<3>(st, P, X);
+    case 4: return launch_inner_c<4>(st, P, X);
+    default: return cudaErrorInvalidValue;
+    }
 }
