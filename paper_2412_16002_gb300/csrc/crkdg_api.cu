@@ -439,6 +439,8 @@ cudaError_t launch_x(crkdg_ctx *h, int kernel, const Params &P0, const MixBufs &
     fill_f32(P);
     if (kernel == KX_INNER && sub_diagonal_euler(h, P))
         return h->tc_on && h->n == 4 ? crkdg_launch_inner_tc(h->st, P, X) : crkdg_launch_inner_cell(h->n, h->st, P, X);
+    if (kernel == KX_FINAL && h->dim == 2 && h->phys == PH_EULER && P.mode == MODE_STEP && P.fx.kon)
+        return crkdg_launch_final_cell(h->n, h->st, P, X);
     int ncb = cells_per_block(h->dim, h->n);
     int nblocks = (h->ncell + ncb - 1) / ncb;
     if (h->dim == 1) return crkdg_launch_mx_1d(kernel, h->n, h->phys, nblocks, h->st, P, X);

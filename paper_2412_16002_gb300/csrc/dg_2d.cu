@@ -32,3 +32,12 @@ cudaError_t crkdg_launch_inner_cell(int n, cudaStream_t st, const Params &P, con
     default: return cudaErrorInvalidValue;
     }
 }
+
+cudaError_t crkdg_launch_final_cell(int n, cudaStream_t st, const Params &P, const MixBufs &X) {
+    switch (n) {
+    case 2: return launch_final_c<2>(st, P, X);
+    case 3: return launch_final_c<3>(st, P, X);
+    case 4: return launch_final_c<4>(st, P, X);
+    default: return cudaErrorInvalidValue;
+    }
+}

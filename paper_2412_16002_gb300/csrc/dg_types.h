@@ -84,6 +84,10 @@ struct FxOp {
     Fx lx[MAXN][2], ly[MAXN][2];  // [0] the lower face, [1] the upper one
     FxGas gas;                    // Euler, 1 < gamma < 2 (on = 0 otherwise)
     int k, on;
+    // face sums of the split path's averages: w1_pos / (2 h_x), w1_pos / (2 h_y) scaled by 2^kk (2D; kon:
+    // the scales are in range)
+    Fx kx[MAXN], ky[MAXN];
+    int kk, kon;
 };
 
 // FP32 copies of the parameters for the split-precision kernels, rounded once by
@@ -188,6 +192,19 @@ inline void fx_operator(Params &P, const NodalTables &T, int dim, int n, int phy
         if (dim == 2) sy = fmax(sy, fabs(P.rhy) * s);
     }
     auto moderate = [](double x) { return x == 0.0 || (fabs(x) > 0x1p-100 && fabs(x) < 0x1p100); };
+    if (dim == 2) {
+        const double r = fabs(P.rhx) + fabs(P.rhy);
+        F.kon = isfinite(r) && r > 0x1p-100 && r < 0x1p100;
+        if (F.kon) {
+            int e;
+            frexp(r, &e);  // the four faces' weights sum to r
+            F.kk = 58 - e;
+            for (int a = 0; a < n; ++a) {
+                F.kx[a] = fx_coef(0.5 * T.w1[a] * P.rhx, F.kk);
+                F.ky[a] = fx_coef(0.5 * T.w1[a] * P.rhy, F.kk);
+            }
+        }
+    }
     const double s = sx + sy;
     F.on = isfinite(s) && s > 0x1p-100 && s < 0x1p100 && moderate(P.gamma) && moderate(P.velx) && moderate(P.vely);
     if (phys == PH_EULER) F.on = F.on && P.gamma > 1.0 && P.gamma < 2.0;
@@ -390,6 +407,7 @@ cudaError_t crkdg_ens_control(int which, cudaStream_t st, crkdg::EnsProblem *E, 
 cudaError_t crkdg_launch_inner_tc(cudaStream_t st, const crkdg::Params &P, const crkdg::MixBufs &X);
 // The same stages on the CUDA cores, one thread per cell (2D Euler, n = 2, 3, 4, MODE_STEP, the same
 // tableaux; defined in dg_2d.cu).
+cudaError_t crkdg_launch_final_cell(int n, cudaStream_t st, const crkdg::Params &P, const crkdg::MixBufs &X);
 cudaError_t crkdg_launch_inner_cell(int n, cudaStream_t st, const crkdg::Params &P, const crkdg::MixBufs &X);
 // Closed-form nodal tables for n = 2, 3, 4 (defined in crkdg_api.cu).
 void crkdg_build_tables(crkdg::NodalTables *tab);
