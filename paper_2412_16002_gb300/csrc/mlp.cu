@@ -6,11 +6,10 @@
 // accuracy is kept by the three-product split (3xTF32): every operand x is
 // x_hi + x_lo with x_hi = tf32(x) and x_lo = tf32(x - x_hi), and the layer is
 // A_hi B_hi + A_hi B_lo + A_lo B_hi.  Bias, ReLU, the 64 -> 1 output layer and
-// the sigmoid run on the CUDA cores.  Training (k_mlp_grad): each block takes 64
-// samples, runs the forward and backward passes with the activations in shared
-// memory, and forms its part of the weight gradients as small contractions over
-// its samples before one atomic add per weight; k_mlp_adam applies the Adam
-// update.  The loss is the mean binary cross-entropy, written from the logits.
+// the sigmoid run on the CUDA cores.  Training (k_mlp_grad): each block walks tiles of
+// 64 samples, forward and backward, as register-tiled FP32 products with the activations
+// in shared memory, and adds its part of the weight gradients once at the end;
+// k_mlp_adam applies the Adam update.  The loss is the mean binary cross-entropy, written from the logits.
 //
 // Parameter vector (7105 floats): W1[64][44], b1[64], W2[64][64], b2[64],
 // w3[64], b3.
@@ -359,82 +358,225 @@ __global__ void __launch_bounds__(TM, 1) k_mlp_forward_tc(const float *__restric
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
 }
 
-constexpr int SB = 64;  // samples per block in the gradient kernel
+// ----------------------------------------------------------------------------- gradient
 
-__global__ void __launch_bounds__(SB) k_mlp_grad(const float *__restrict__ theta, const float *__restrict__ X,
-                                                 const float *__restrict__ y, int n, float inv_total,
-                                                 float *__restrict__ grad, float *__restrict__ loss) {
-    extern __shared__ float sm[];
-    float *w = sm;                  // NP
-    float *sx = w + NP;             // SB x NIN
-    float *sh1 = sx + SB * NIN;     // SB x NH  (h1)
-    float *sd1 = sh1 + SB * NH;     // SB x NH  (d a1)
-    float *sd2 = sd1 + SB * NH;     // SB x NH  (d a2)
-    float *sdz = sd2 + SB * NH;     // SB
-    float *sh2 = sdz + SB;          // SB x NH  (h2)
-    for (int i = threadIdx.x; i < NP; i += blockDim.x) w[i] = theta[i];
-    const int t = threadIdx.x;
-    const int r = blockIdx.x * SB + t;
-    const bool valid = r < n;
-    for (int k = 0; k < NIN; ++k) sx[t * NIN + k] = valid ? X[(size_t)r * NIN + k] : 0.0f;
-    __syncthreads();
-    // forward, one sample per thread
-    float a1[NH];
-    for (int j = 0; j < NH; ++j) {
-        float a = w[OB1 + j];
-        for (int k = 0; k < NIN; ++k) a = fmaf(w[OW1 + j * NIN + k], sx[t * NIN + k], a);
-        a1[j] = a;
-        sh1[t * NH + j] = fmaxf(a, 0.0f);
-    }
-    float z = w[OB3];
-    for (int j = 0; j < NH; ++j) {
-        float a = w[OB2 + j];
-        for (int i = 0; i < NH; ++i) a = fmaf(w[OW2 + j * NH + i], sh1[t * NH + i], a);
-        float h = fmaxf(a, 0.0f);
-        sh2[t * NH + j] = h;
-        sd2[t * NH + j] = a > 0.0f ? 1.0f : 0.0f;  // ReLU mask, scaled below
-        z = fmaf(w[OW3 + j], h, z);
-    }
-    float yy = valid ? y[r] : 0.0f;
-    float dz = valid ? (sigmoidf_(z) - yy) * inv_total : 0.0f;
-    if (valid) atomicAdd(loss, (softplus(z) - yy * z) * inv_total);
-    sdz[t] = dz;
-    // backward through the layers of this sample
-    for (int j = 0; j < NH; ++j) sd2[t * NH + j] *= dz * w[OW3 + j];
-    for (int i = 0; i < NH; ++i) {
-        float s = 0.0f;
-        for (int j = 0; j < NH; ++j) s = fmaf(sd2[t * NH + j], w[OW2 + j * NH + i], s);
-        sd1[t * NH + i] = a1[i] > 0.0f ? s : 0.0f;
-    }
-    __syncthreads();
-    // weight gradients: contractions over the block's samples, one atomic per weight
-    for (int e = t; e < NH * NIN; e += SB) {
-        int j = e / NIN, k = e - j * NIN;
-        float s = 0.0f;
-        for (int q = 0; q < SB; ++q) s = fmaf(sd1[q * NH + j], sx[q * NIN + k], s);
-        atomicAdd(&grad[OW1 + e], s);
-    }
-    for (int e = t; e < NH * NH; e += SB) {
-        int j = e / NH, i = e - j * NH;
-        float s = 0.0f;
-        for (int q = 0; q < SB; ++q) s = fmaf(sd2[q * NH + j], sh1[q * NH + i], s);
-        atomicAdd(&grad[OW2 + e], s);
-    }
-    if (t < NH) {
-        float s1 = 0.0f, s2 = 0.0f, s3 = 0.0f;
-        for (int q = 0; q < SB; ++q) {
-            s1 += sd1[q * NH + t];
-            s2 += sd2[q * NH + t];
-            s3 = fmaf(sdz[q], sh2[q * NH + t], s3);
+constexpr int SB = 64;    // samples per tile
+constexpr int GT = 256;   // threads: 16 x 16, each a 4 x 4 part of every 64 x 64 product
+constexpr int LH = NH + 4;  // row pitch of 64-wide arrays (eight rows on distinct banks in 16-byte reads)
+
+struct GradSmem {
+    float w1[NH][NIN], w2[NH][LH];                    // 44-float rows are conflict-free as they are
+    float x[SB][NIN], h1[SB][LH], d2[SB][LH], d1[SB][LH];
+    float b1[NH], b2[NH], w3[NH];
+    float part[GT / 32][3 * NH + 2];                  // warps' sums of gb1, gb2, gw3, gb3, loss
+};
+
+__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+// acc[m][n] += a_m . b_n for four components each
+__device__ __forceinline__ void dot4(float (&acc)[4][4], const float4 (&a)[4], const float4 (&b)[4]) {
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            acc[m][n] = fmaf(b[n].x, a[m].x, acc[m][n]);
+            acc[m][n] = fmaf(b[n].y, a[m].y, acc[m][n]);
+            acc[m][n] = fmaf(b[n].z, a[m].z, acc[m][n]);
+            acc[m][n] = fmaf(b[n].w, a[m].w, acc[m][n]);
         }
-        atomicAdd(&grad[OB1 + t], s1);
-        atomicAdd(&grad[OB2 + t], s2);
-        atomicAdd(&grad[OW3 + t], s3);
+}
+// acc += a b^T
+__device__ __forceinline__ void outer4(float (&acc)[4][4], const float4 &a, const float4 &b) {
+    const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+#pragma unroll
+        for (int n = 0; n < 4; ++n) acc[m][n] = fmaf(av[m], bv[n], acc[m][n]);
+}
+__device__ __forceinline__ void add4(float *dst, float a, float b, float c, float d) {
+    if (((uintptr_t)dst & 15u) == 0) {
+        atomicAdd(reinterpret_cast<float4 *>(dst), make_float4(a, b, c, d));
+    } else {
+        atomicAdd(dst, a);
+        atomicAdd(dst + 1, b);
+        atomicAdd(dst + 2, c);
+        atomicAdd(dst + 3, d);
     }
-    if (t == 0) {
+}
+
+// Loss and gradient: a block walks 64-sample tiles; every layer of a tile and both weight gradients
+// are 64-wide products with a 4 x 4 part per thread (16 fused multiply-adds per two 16-byte shared
+// reads), all arrays row-major: the forward products run along the rows of both factors, the
+// backward and weight-gradient ones over rows.  FP32 throughout; the sums over samples are formed per
+// tile, then over the block's tiles, then by one addition per block and weight, the loss likewise.
+// The sums over the inputs of a unit keep their order.  One thread per sample instead read its rows of
+// shared memory with 32-way bank conflicts and added every sample's loss to one address: loss, gradient
+// and update of 8192 samples took 155 us, now 67, most of it the launches of the pass.
+__global__ void __launch_bounds__(GT, 2) k_mlp_grad(const float *__restrict__ theta, const float *__restrict__ X,
+                                                    const float *__restrict__ y, int n, float inv_total,
+                                                    float *__restrict__ grad, float *__restrict__ loss) {
+    extern __shared__ __align__(16) unsigned char grad_sm[];
+    GradSmem &S = *reinterpret_cast<GradSmem *>(grad_sm);
+    const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
+    for (int i = t; i < NH * NIN; i += GT) (&S.w1[0][0])[i] = theta[OW1 + i];
+    for (int i = t; i < NH * NH; i += GT) S.w2[i / NH][i % NH] = theta[OW2 + i];
+    if (t < NH) {
+        S.b1[t] = theta[OB1 + t];
+        S.b2[t] = theta[OB2 + t];
+        S.w3[t] = theta[OW3 + t];
+    }
+    const float b3 = theta[OB3];
+    const int kj = t / 11 * 4, kk = t % 11 * 4;  // this thread's part of W1's gradient (t < 176)
+    float g2[4][4] = {}, g1[4][4] = {};          // W2: rows 4 ty.., columns 4 tx..; W1: rows kj.., columns kk..
+    float gb1[4] = {}, gb2[4] = {}, gw3[4] = {}, gb3 = 0.0f, ls = 0.0f;
+    const int ntiles = n / SB + (n % SB != 0);
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const int r0 = tile * SB, rows = n - r0 < SB ? n - r0 : SB;
+        __syncthreads();  // the weights are there; the last tile's arrays are free
+        for (int i = t; i < SB * NIN; i += GT) (&S.x[0][0])[i] = i < rows * NIN ? X[(size_t)r0 * NIN + i] : 0.0f;
+        float yy[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) yy[m] = ty + 16 * m < rows ? y[r0 + ty + 16 * m] : 0.0f;
+        __syncthreads();
+        // layer 1: samples ty + 16 m, units tx + 16 n
+        float acc[4][4];
+        float4 a[4], b[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[m][q] = S.b1[tx + 16 * q];
+#pragma unroll 1
+        for (int k = 0; k < NIN; k += 4) {
+#pragma unroll
+            for (int m = 0; m < 4; ++m) a[m] = ld4(&S.x[ty + 16 * m][k]), b[m] = ld4(&S.w1[tx + 16 * m][k]);
+            dot4(acc, a, b);
+        }
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) S.h1[ty + 16 * m][tx + 16 * q] = fmaxf(acc[m][q], 0.0f);
+        __syncthreads();
+        // layer 2, the output unit and its gradient
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[m][q] = S.b2[tx + 16 * q];
+#pragma unroll 1
+        for (int k = 0; k < NH; k += 4) {
+#pragma unroll
+            for (int m = 0; m < 4; ++m) a[m] = ld4(&S.h1[ty + 16 * m][k]), b[m] = ld4(&S.w2[tx + 16 * m][k]);
+            dot4(acc, a, b);
+        }
+        float w3[4], tb2[4] = {}, tw3[4] = {}, tb3 = 0.0f, tl = 0.0f;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) w3[q] = S.w3[tx + 16 * q];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            float z = 0.0f;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) z = fmaf(w3[q], fmaxf(acc[m][q], 0.0f), z);
+#pragma unroll
+            for (int o = 1; o < 16; o <<= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+            z += b3;
+            const bool valid = ty + 16 * m < rows;
+            const float dz = valid ? (sigmoidf_(z) - yy[m]) * inv_total : 0.0f;
+            if (valid && tx == 0) tl += (softplus(z) - yy[m] * z) * inv_total;
+            tb3 += dz;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float d = (acc[m][q] > 0.0f ? 1.0f : 0.0f) * (dz * w3[q]);
+                tb2[q] += d;
+                tw3[q] = fmaf(dz, fmaxf(acc[m][q], 0.0f), tw3[q]);
+                S.d2[ty + 16 * m][tx + 16 * q] = d;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) gb2[q] += tb2[q], gw3[q] += tw3[q];
+        gb3 += tb3, ls += tl;
+        __syncthreads();
+        // back to layer 1: samples ty + 16 m, units 4 tx + n
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[m][q] = 0.0f;
+#pragma unroll 1
+        for (int j = 0; j < NH; j += 4) {
+#pragma unroll
+            for (int m = 0; m < 4; ++m) a[m] = ld4(&S.d2[ty + 16 * m][j]), b[m] = ld4(&S.w2[j + m][4 * tx]);
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                const float av[4] = {a[m].x, a[m].y, a[m].z, a[m].w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    acc[m][0] = fmaf(av[k], b[k].x, acc[m][0]);
+                    acc[m][1] = fmaf(av[k], b[k].y, acc[m][1]);
+                    acc[m][2] = fmaf(av[k], b[k].z, acc[m][2]);
+                    acc[m][3] = fmaf(av[k], b[k].w, acc[m][3]);
+                }
+            }
+        }
+        float tb1[4] = {};
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            const float4 h = ld4(&S.h1[ty + 16 * m][4 * tx]);
+            const float4 d = make_float4(h.x > 0.0f ? acc[m][0] : 0.0f, h.y > 0.0f ? acc[m][1] : 0.0f,
+                                         h.z > 0.0f ? acc[m][2] : 0.0f, h.w > 0.0f ? acc[m][3] : 0.0f);
+            *reinterpret_cast<float4 *>(&S.d1[ty + 16 * m][4 * tx]) = d;
+            tb1[0] += d.x, tb1[1] += d.y, tb1[2] += d.z, tb1[3] += d.w;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) gb1[q] += tb1[q];
+        // weight gradients over the tile's samples
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[m][q] = 0.0f;
+#pragma unroll 4
+        for (int s = 0; s < SB; ++s) outer4(acc, ld4(&S.d2[s][4 * ty]), ld4(&S.h1[s][4 * tx]));
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) g2[m][q] += acc[m][q], acc[m][q] = 0.0f;
+        __syncthreads();
+        if (t < NH / 4 * (NIN / 4)) {
+#pragma unroll 4
+            for (int s = 0; s < SB; ++s) outer4(acc, ld4(&S.d1[s][kj]), ld4(&S.x[s][kk]));
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) g1[m][q] += acc[m][q];
+        }
+    }
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        add4(grad + OW2 + (4 * ty + m) * NH + 4 * tx, g2[m][0], g2[m][1], g2[m][2], g2[m][3]);
+        if (t < NH / 4 * (NIN / 4)) add4(grad + OW1 + (kj + m) * NIN + kk, g1[m][0], g1[m][1], g1[m][2], g1[m][3]);
+    }
+    // the sums held per sample group: the warp's two groups, then the warps
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        gb1[q] += __shfl_xor_sync(0xffffffffu, gb1[q], 16);
+        gb2[q] += __shfl_xor_sync(0xffffffffu, gb2[q], 16);
+        gw3[q] += __shfl_xor_sync(0xffffffffu, gw3[q], 16);
+    }
+    gb3 += __shfl_xor_sync(0xffffffffu, gb3, 16);
+    ls += __shfl_xor_sync(0xffffffffu, ls, 16);
+    float *part = S.part[t >> 5];
+    if ((t & 31) < 16) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            part[4 * tx + q] = gb1[q];
+            part[NH + tx + 16 * q] = gb2[q];
+            part[2 * NH + tx + 16 * q] = gw3[q];
+        }
+        if (tx == 0) part[3 * NH] = gb3, part[3 * NH + 1] = ls;
+    }
+    __syncthreads();
+    if (t < 3 * NH + 2) {
         float s = 0.0f;
-        for (int q = 0; q < SB; ++q) s += sdz[q];
-        atomicAdd(&grad[OB3], s);
+#pragma unroll
+        for (int w = 0; w < GT / 32; ++w) s += S.part[w][t];
+        atomicAdd(t < NH ? grad + OB1 + t : t < 2 * NH ? grad + OB2 + t - NH : t < 3 * NH ? grad + OW3 + t - 2 * NH
+                  : t == 3 * NH ? grad + OB3 : loss, s);
     }
 }
 
@@ -449,8 +591,6 @@ __global__ void k_mlp_adam(float *theta, float *m, float *v, const float *grad, 
     v[i] = vi;
     theta[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
 }
-
-size_t grad_smem() { return sizeof(float) * (NP + SB * NIN + 4 * SB * NH + SB); }
 
 }  // namespace
 
@@ -490,15 +630,21 @@ crkdg_status crkdg_mlp_fault(int *fault) {
 crkdg_status crkdg_mlp_grad(const float *params, const float *X, const float *y, int n, float *grad, float *loss,
                             void *stream) {
     if (!params || !X || !y || !grad || !loss || n <= 0) return CRKDG_E_ARG;
-    static bool configured = false;
-    if (!configured) {
-        if (cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)grad_smem()) !=
+    int dev = 0, nsm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return CRKDG_E_CUDA;
+    static int configured_dev = -1;  // the attribute is per device
+    if (configured_dev != dev) {
+        if (cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GradSmem)) !=
             cudaSuccess)
             return CRKDG_E_CUDA;
-        configured = true;
+        configured_dev = dev;
     }
-    k_mlp_grad<<<(n + SB - 1) / SB, SB, grad_smem(), (cudaStream_t)stream>>>(params, X, y, n, 1.0f / (float)n, grad,
-                                                                            loss);
+    // two blocks fit an SM; the same number of tiles for every block, so that few blocks add at the end
+    const int tiles = n / SB + (n % SB != 0), rounds = (tiles + 2 * nsm - 1) / (2 * nsm);
+    const int grid = (tiles + rounds - 1) / rounds;
+    k_mlp_grad<<<grid, GT, sizeof(GradSmem), (cudaStream_t)stream>>>(params, X, y, n, 1.0f / (float)n, grad, loss);
     return cudaGetLastError() == cudaSuccess ? CRKDG_OK : CRKDG_E_CUDA;
 }
 
