@@ -1603,7 +1603,7 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_inner(const __grid_constant
 // collective): the four products per component in fixed point with one exponent per cell and
 // component (dg_fixed.h), as in eval_G_fx; corrections outside its range take the FP64 form.
 template <class C>
-__device__ __forceinline__ void lift_faces(const Params &P, CellData<C> &D, int node, int a, int b,
+__device__ __forceinline__ void lift_faces(const Params &P, double dt, CellData<C> &D, int node, int a, int b,
                                            const double (&dc)[C::FPT][C::M], double *u) {
     constexpr int DIM = C::D, N = C::NP, M = C::M, NN = C::NN, NF = C::NF, NTR = C::NTR, FPT = C::FPT;
     constexpr int W = (M + 1) / 2;
@@ -1672,7 +1672,7 @@ __device__ __forceinline__ void lift_faces(const Params &P, CellData<C> &D, int 
             fx_mac(s, ft[c][3 * NF + a], y1);
         }
         const double v = fx_double(fx_sum(s), fx_shift(E, P.fx.k));
-        u[c] = fma(P.dt, bad ? corr[c] : v, u[c]);
+        u[c] = fma(dt, bad ? corr[c] : v, u[c]);
     }
 }
 
@@ -1787,7 +1787,7 @@ __device__ __forceinline__ void final_body(const Params &P, const Bufs &B, int b
             }
     }
     cell_sync<C>();
-    lift_faces<C>(P, S.c[lc], node, a, b, dc, u);
+    lift_faces<C>(P, P.dt, S.c[lc], node, a, b, dc, u);
     if (P.pk) project_pk<C>(S, lc, node, u);
     if (P.mode == MODE_OP_F) {
         if (active && solid_cell(P, cell))  // outside the domain: no operator

@@ -15,22 +15,13 @@
 
 namespace crkdg {
 
-template <int N, int PHYS, int NCBV>
-struct RunCfg1D {
-    static constexpr int D = 1;
-    static constexpr int NP = N;
-    static constexpr int PH = PHYS;
-    static constexpr int M = ncomp(PHYS, 1);
-    static constexpr int NN = N;
-    static constexpr int NF = 1;
-    static constexpr int NTR = 2;
-    static constexpr int L = nlob(N);
-    static constexpr int NSK = L;
-    static constexpr int NCB = NCBV;  // cells per chunk including the two halo cells
-    static constexpr bool WARP = false;
-    static constexpr int NT = NCB * NN;
-    static constexpr int PPT = (NSK + NN - 1) / NN;
-    static constexpr int FPT = (NTR + NN - 1) / NN;
+// Whole cells per warp (CfgW), so that a stage of a cell needs no block barrier, and four warps (two
+// for N = 2), one for each scheduler of an SM: a mesh of this size leaves one block on an SM, and a
+// step is one warp's chain of instructions.
+template <int N, int PHYS>
+struct RunCfg1D : CfgW<1, N, PHYS> {
+    static constexpr int NT = N == 2 ? 64 : 128;
+    static constexpr int NCB = (32 / N) * (NT / 32);  // cells per chunk including the two halo cells
 };
 
 __device__ __forceinline__ unsigned long long global_ns() {
@@ -81,23 +72,29 @@ __device__ bool grid_barrier(RunCtl *R, unsigned target, const RunSlot *SL, Slot
     return s_ok != 0;
 }
 
-template <int N, int PHYS, int NCBV>
-__global__ void __launch_bounds__(RunCfg1D<N, PHYS, NCBV>::NT) k_run1d(Params P, double *U0, double *U1,
-                                                                        RunCtl *R, int cown) {
-    using C = RunCfg1D<N, PHYS, NCBV>;
-    constexpr int M = C::M, NN = C::NN;
+// The stages run on the integer units as in the per-step kernels (eval_G_fx, lift_faces), and the
+// final stage combines jumps of the weighted flux sums: of the FP64 instructions of a step, each 64 to
+// 76 cycles behind the one before it, about a quarter is left (4096 cells of the blast tube 20.2 -> 18.9 us a
+// step, where the blocks at the front wait for the limiter's FP64 form; Burgers, 200 cells, 7.7 -> 7.4).
+template <int N, int PHYS>
+__global__ void __launch_bounds__(RunCfg1D<N, PHYS>::NT) k_run1d(const __grid_constant__ Params P, double *U0, double *U1,
+                                                                 RunCtl *R, int cown) {
+    using C = RunCfg1D<N, PHYS>;
+    constexpr int M = C::M;
+    constexpr int kUnroll = PHYS == PH_EULER ? 1 : MAXS;  // four Euler stages would not fit the instruction cache
     const int COWN = cown;  // own cells per chunk (1 .. NCB - 2); slots beyond COWN + 1 stay idle
     __shared__ Smem<C> S;
+    __shared__ BlockTab<C> Tb;
     __shared__ double sTr[MAXS][C::NCB][2][M];
     __shared__ double sAv[MAXS][C::NCB][M];  // cell averages of the traced stage values
-    __shared__ double sFc[MAXS][C::NCB][2][M];  // per face: fhat - f(u_L), fhat - f(u_R)
-    __shared__ double sTf[MAXS][C::NCB][2][M];  // normal fluxes of the traces
-    __shared__ double sSp[MAXS][C::NCB][2];     // spectral radii of the traces
-    const NodalTables &T = c_tab[N - 2];
-    const int lc = threadIdx.x / NN, node = threadIdx.x - lc * NN;
-    const int a = node;
+    __shared__ double sFs[C::NCB][2][M];     // sum_i b_i f(trace^(i)) of a cell's two faces
+    __shared__ double sSp[MAXS][C::NCB][2];  // spectral radii of the traces
+    int lc, node;
+    place<C>(lc, node);
     const int nchunks = (P.ncell + COWN - 1) / COWN;
     const bool periodic = P.bc[0] == BC_PERIODIC;
+    fill_tab<C>(P, Tb);  // its dt products are replaced for every attempt
+    __syncthreads();
 
     double t = R->t;
     const double t_end = R->t_end, cfl = R->cfl;
@@ -124,134 +121,99 @@ __global__ void __launch_bounds__(RunCfg1D<N, PHYS, NCBV>::NT) k_run1d(Params P,
             const bool exists = lc <= COWN + 1 && (periodic || (graw >= 0 && graw < P.ncell));
             const int gc = periodic ? (graw % P.ncell + P.ncell) % P.ncell : graw;
             const bool own = lc >= 1 && lc <= COWN && graw < P.ncell;
-            double u0[M], cur_u[M], acc[M], gh[MAXS][M];
+            if (threadIdx.x >= 32 && threadIdx.x < 32 + MAXS * MAXS + MAXS) {  // this attempt's dt a_ij, dt b_i
+                const int k = (int)threadIdx.x - 32;
+                if (k < MAXS * MAXS)
+                    Tb.dtA[k / MAXS][k % MAXS] = dt * P.A[k / MAXS][k % MAXS];
+                else
+                    Tb.dtb[k - MAXS * MAXS] = dt * P.b[k - MAXS * MAXS];
+            }
+            double u0[M], cur_u[M], u[M], fs[M], gh[MAXS][M];
             load_node<1, N, PHYS>(P, un, gc, node, exists, u0);
 #pragma unroll
-            for (int c = 0; c < M; ++c) cur_u[c] = acc[c] = u0[c];
+            for (int c = 0; c < M; ++c) {
+                cur_u[c] = u[c] = u0[c];
+                fs[c] = 0.0;
+            }
+            __syncthreads();
             // inner stages of every cell of the chunk, halo included
-#pragma unroll
+#pragma unroll kUnroll
             for (int i = 0; i < MAXS; ++i) {
                 if (i >= P.s) break;
                 if (i > 0) {
 #pragma unroll
-                    for (int c = 0; c < M; ++c) {
-                        double v = u0[c];
+                    for (int c = 0; c < M; ++c) cur_u[c] = u0[c];
+#pragma unroll kUnroll
+                    for (int j = 0; j < i; ++j)
+                        if (nonzero_bits(P.A[i][j]))
 #pragma unroll
-                        for (int j = 0; j < i; ++j)
-                            if (nonzero_bits(P.A[i][j])) v = fma(dt * P.A[i][j], gh[j][c], v);
-                        cur_u[c] = v;
-                    }
+                            for (int c = 0; c < M; ++c) cur_u[c] = fma(Tb.dtA[i][j], gh[j][c], cur_u[c]);
                     double pts[C::PPT][M];
                     float rhi;
                     limit_block(P, B, S, lc, node, own, cur_u, pts, true, true, false, rhi);
                 }
-                double trs[C::FPT][M];
-                const bool traced = P.slot[i] >= 0;
-                eval_G(P, S, lc, node, cur_u, gh[i], trs, traced);
-                if (nonzero_bits(P.b[i])) {
+                const int q = P.slot[i];
+                double g[M];
+                eval_G_fx<C>(
+                    P, S, Tb, lc, node, cur_u, g, q >= 0, q >= 0,
+                    [&](int, const double *tr, const double *f, double sp) {  // one face point per thread
+                        if (q < 0) return;
 #pragma unroll
-                    for (int c = 0; c < M; ++c) acc[c] = fma(dt * P.b[i], gh[i][c], acc[c]);
-                }
-                if (traced && node < 2) {
+                        for (int c = 0; c < M; ++c) {
+                            sTr[q][lc][node][c] = tr[c];
+                            fs[c] = fma(P.b[i], f[c], fs[c]);
+                        }
+                        sSp[q][lc][node] = sp;
+                    },
+                    [&](int c, double v) { sAv[q][lc][c] = v; });
 #pragma unroll
-                    for (int c = 0; c < M; ++c) {
-                        sTr[P.slot[i]][lc][node][c] = trs[0][c];
-                        sTf[P.slot[i]][lc][node][c] = S.c[lc].tf[node][c];  // written by this thread
-                    }
-                    sSp[P.slot[i]][lc][node] = S.c[lc].ts[node];
-                }
-                if (P.slot[i] >= 0) {  // S.u holds the stage values until the next stage's limiter
-                    for (int c = node; c < M; c += NN) {
-                        double s = 0.0;
-#pragma unroll
-                        for (int q = 0; q < NN; ++q) s = fma(T.w1[q], S.c[lc].u[c][q], s);
-                        sAv[P.slot[i]][lc][c] = s;
-                    }
-                    __syncthreads();
+                for (int c = 0; c < M; ++c) {
+                    gh[i][c] = g[c];
+                    if (nonzero_bits(P.b[i])) u[c] = fma(Tb.dtb[i], g[c], u[c]);
                 }
             }
+            if (node < 2)
+#pragma unroll
+                for (int c = 0; c < M; ++c) sFs[lc][node][c] = fs[c];
             __syncthreads();
-            // final stage: Lax--Friedrichs flux of every face of the chunk and every traced
-            // stage, once per face (face j lies between slots j and j+1); a cell then sums its
-            // two faces' corrections over the stages in stage order
-            {
-                const int nfaces = COWN + 1;  // faces of the own cells
-                const int nitems = nfaces * P.nslot;
-                for (int k = threadIdx.x; k < nitems; k += blockDim.x) {
-                    const int j = k % nfaces, q = k / nfaces;
-                    const int rl = c0 - 1 + j, rr = rl + 1;  // unwrapped indices of the two cells
-                    const bool el = periodic || (rl >= 0 && rl < P.ncell);
-                    const bool er = periodic || (rr >= 0 && rr < P.ncell);
-                    // interior sides: the trace, its flux and its spectral radius as the
-                    // traced stage's G evaluation computed them; exterior sides from the
-                    // boundary condition
-                    double uL[M], uR[M], fL[M], fR[M], sL, sR;
-                    if (el && er) {
+            // final stage, as final_body: this thread's face of its cell, from the trace sums and radii
+            // of the two sides; the exterior side of a boundary face from the boundary condition
+            double dc[C::FPT][M];
 #pragma unroll
-                        for (int c = 0; c < M; ++c) {
-                            uL[c] = sTr[q][j][1][c];
-                            uR[c] = sTr[q][j + 1][0][c];
-                            fL[c] = sTf[q][j][1][c];
-                            fR[c] = sTf[q][j + 1][0][c];
-                        }
-                        sL = sSp[q][j][1];
-                        sR = sSp[q][j + 1][0];
-                    } else if (er) {  // the left side of the mesh: exterior state of side 0
-                        double ui[M];
+            for (int c = 0; c < M; ++c) dc[0][c] = 0.0;
+            if (own && node < 2) {
+                const int ln = node ? lc + 1 : lc - 1, gn = node ? graw + 1 : graw - 1;
+                const bool inside = periodic || (gn >= 0 && gn < P.ncell);
+                double fe[M];
 #pragma unroll
-                        for (int c = 0; c < M; ++c) {
-                            ui[c] = uR[c] = sTr[q][j + 1][0][c];
-                            fR[c] = sTf[q][j + 1][0][c];
-                        }
-                        sR = sSp[q][j + 1][0];
-                        exterior_state<PHYS, 1>(P, 0, ui, sAv[q][j + 1], uL);
-                        sL = flux_speed_dir<PHYS, 1>(P, uL, 0, fL);
-                    } else if (el) {  // the right side: exterior state of side 1
-                        double ui[M];
-#pragma unroll
-                        for (int c = 0; c < M; ++c) {
-                            ui[c] = uL[c] = sTr[q][j][1][c];
-                            fL[c] = sTf[q][j][1][c];
-                        }
-                        sL = sSp[q][j][1];
-                        exterior_state<PHYS, 1>(P, 1, ui, sAv[q][j], uR);
-                        sR = flux_speed_dir<PHYS, 1>(P, uR, 0, fR);
-                    } else {
-                        continue;  // a face beyond the mesh: no own cell uses it
-                    }
-                    double alpha = fmax_nonneg(sL, sR);
-#pragma unroll
-                    for (int c = 0; c < M; ++c) {
-                        double fhat = 0.5 * (fL[c] + fR[c]) - 0.5 * alpha * (uR[c] - uL[c]);
-                        sFc[q][j][0][c] = fhat - fL[c];  // the left cell's right face
-                        sFc[q][j][1][c] = fhat - fR[c];  // the right cell's left face
-                    }
-                }
-            }
-            __syncthreads();
-            double u[M];
-            if (own) {
-                double dl[M], dr[M];
-#pragma unroll
-                for (int c = 0; c < M; ++c) dl[c] = dr[c] = 0.0;
+                for (int c = 0; c < M; ++c) fe[c] = 0.0;
                 for (int i = 0; i < P.s; ++i) {
                     const int q = P.slot[i];
                     if (q < 0) continue;
+                    double ui[M], ue[M], alpha = sSp[q][lc][node];
 #pragma unroll
-                    for (int c = 0; c < M; ++c) {
-                        dl[c] = fma(P.b[i], sFc[q][lc - 1][1][c], dl[c]);
-                        dr[c] = fma(P.b[i], sFc[q][lc][0][c], dr[c]);
+                    for (int c = 0; c < M; ++c) ui[c] = sTr[q][lc][node][c];
+                    if (inside) {
+#pragma unroll
+                        for (int c = 0; c < M; ++c) ue[c] = sTr[q][ln][node ^ 1][c];
+                        alpha = fmax_nonneg(alpha, sSp[q][ln][node ^ 1]);
+                    } else {
+                        double f[M];
+                        exterior_state<PHYS, 1>(P, node, ui, sAv[q][lc], ue);
+                        alpha = fmax_nonneg(alpha, face_flux<PHYS, 1>(P, ue, 0, true, f));
+#pragma unroll
+                        for (int c = 0; c < M; ++c) fe[c] = fma(P.b[i], f[c], fe[c]);
                     }
+                    const double h = half_of(P.b[i]), ba = (node ? -h : h) * alpha;
+#pragma unroll
+                    for (int c = 0; c < M; ++c) dc[0][c] = fma(ba, ue[c] - ui[c], dc[0][c]);
                 }
 #pragma unroll
-                for (int c = 0; c < M; ++c) {
-                    double corr = -T.liftp[a] * dr[c] + T.liftm[a] * dl[c];
-                    u[c] = fma(dt, P.rhx * corr, acc[c]);
-                }
-            } else {
-#pragma unroll
-                for (int c = 0; c < M; ++c) u[c] = acc[c];
+                for (int c = 0; c < M; ++c)
+                    dc[0][c] = fma(0.5, (inside ? sFs[ln][node ^ 1][c] : fe[c]) - fs[c], dc[0][c]);
             }
+            cell_sync<C>();
+            lift_faces<C>(P, dt, S.c[lc], node, node, 0, dc, u);
             double pts[C::PPT][M];
             float rhi;
             const bool cleared = limit_block(P, B, S, lc, node, own, u, pts, true, true, true, rhi);
@@ -307,19 +269,18 @@ __global__ void __launch_bounds__(RunCfg1D<N, PHYS, NCBV>::NT) k_run1d(Params P,
 template <int N, int PHYS>
 cudaError_t run1d_launch(cudaStream_t st, const Params &P, double *u0, double *u1, RunCtl *R, int chunk,
                          int *nblocks) {
-    constexpr int NCB = 32;
-    using C = RunCfg1D<N, PHYS, NCB>;
+    using C = RunCfg1D<N, PHYS>;
+    constexpr int NCB = C::NCB;
     int dev = 0, nsm = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_run1d<N, PHYS, NCB>, C::NT, 0);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_run1d<N, PHYS>, C::NT, 0);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     // chunks of NCB - 2 own cells by default: smaller chunks put more blocks on the GPU but
-    // recompute more halo cells and add arrivals at the grid barrier, which costs more than
-    // it gains (4096 cells: 26.0 us per step at 30 cells, 26.4 at 27, 30.0 at 20, 47.7 at 7)
+    // recompute more halo cells and add arrivals at the grid barrier
     const int slots = nsm * per_sm;
     int cown = chunk > 0 ? chunk : NCB - 2;
     if (cown > NCB - 2) cown = NCB - 2;
@@ -329,7 +290,7 @@ cudaError_t run1d_launch(cudaStream_t st, const Params &P, double *u0, double *u
     *nblocks = grid;
     Params Pc = P;
     void *args[] = {&Pc, &u0, &u1, &R, &cown};
-    return cudaLaunchCooperativeKernel((void *)k_run1d<N, PHYS, NCB>, dim3(grid), dim3(C::NT), args, 0, st);
+    return cudaLaunchCooperativeKernel((void *)k_run1d<N, PHYS>, dim3(grid), dim3(C::NT), args, 0, st);
 }
 
 }  // namespace crkdg
