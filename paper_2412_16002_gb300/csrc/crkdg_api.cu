@@ -1142,7 +1142,7 @@ crkdg_status attempt_once(crkdg_t h, Params &P, double dt, bool want_mass) {
 }
 
 // Accept the attempt in h->hs: the new state becomes u^n.
-void accept_attempt(crkdg_t h, double dt, int restarts, crkdg_step_info *info) {
+void accept_attempt(crkdg_t h, double dt, int restarts, crkdg_step_info *info, bool mass) {
     h->t += dt;
     if (h->mixed) {
         h->xcur = 1 - h->xcur;
@@ -1159,6 +1159,8 @@ void accept_attempt(crkdg_t h, double dt, int restarts, crkdg_step_info *info) {
         info->cells_limited = (long long)h->hs->nlim;
         info->theta_min = from_bits(h->hs->thmin);
         info->troubled = (long long)h->hs->ntrb;
+    }
+    if (info && mass) {
         // relative change of the first component's total over the step
         const double m0 = h->mass_n[0], m1 = h->hs->mass[0];
         info->mass_drift = (m1 - m0) / (m0 != 0.0 ? fabs(m0) : 1.0);
@@ -1172,18 +1174,20 @@ void accept_attempt(crkdg_t h, double dt, int restarts, crkdg_step_info *info) {
 
 extern "C" {
 
-crkdg_status crkdg_step(crkdg_t h, double dt, const crkdg_tableau *tab, crkdg_step_info *info) {
-    if (!h) return CRKDG_E_ARG;
+// One step with its restarts; mass: also the component totals behind info->mass_drift (a pass over the
+// new state, which the step loops of crkdg_advance and crkdg_advance_fixed do not report: a step without
+// it takes 97 us instead of 112 at 64^2 Q^2 and 100 instead of 121 at 131^2 Q^3 in split precision).
+static crkdg_status step_once(crkdg_t h, double dt, const crkdg_tableau *tab, crkdg_step_info *info, bool mass) {
     try {
         Params P;
-        crkdg_status s = prepare_step(h, dt, tab, info != nullptr, P);
+        crkdg_status s = prepare_step(h, dt, tab, mass, P);
         if (s) return s;
         h->pending = false;
         for (int r = 0; r <= h->opt.max_halvings; ++r) {
-            s = attempt_once(h, P, dt, info != nullptr);
+            s = attempt_once(h, P, dt, mass);
             if (s) return s;
             if (h->hs->flag == 0) {
-                accept_attempt(h, dt, r, info);
+                accept_attempt(h, dt, r, info, mass);
                 return CRKDG_OK;
             }
             dt *= 0.5;
@@ -1192,6 +1196,11 @@ crkdg_status crkdg_step(crkdg_t h, double dt, const crkdg_tableau *tab, crkdg_st
     } catch (...) {
         return CRKDG_E_OOM;
     }
+}
+
+crkdg_status crkdg_step(crkdg_t h, double dt, const crkdg_tableau *tab, crkdg_step_info *info) {
+    if (!h) return CRKDG_E_ARG;
+    return step_once(h, dt, tab, info, info != nullptr);
 }
 
 crkdg_status crkdg_step_attempt(crkdg_t h, double dt, const crkdg_tableau *tab, int *violated) {
@@ -1218,7 +1227,7 @@ crkdg_status crkdg_step_accept(crkdg_t h, crkdg_step_info *info) {
     if (h->hs->flag != 0) return fail(h, CRKDG_E_ARG, "step_accept: the attempt left the admissible set");
     h->pending = false;
     crkdg_step_info tmp;
-    accept_attempt(h, h->pending_dt, 0, info ? info : &tmp);
+    accept_attempt(h, h->pending_dt, 0, info ? info : &tmp, true);
     return CRKDG_OK;
 }
 
@@ -1308,7 +1317,7 @@ crkdg_status crkdg_advance(crkdg_t h, int nsteps, double cfl, double t_end, cons
         if (s) break;
         if (dt > t_end - *t) dt = t_end - *t;
         crkdg_step_info info;
-        s = crkdg_step(h, dt, tab, &info);
+        s = step_once(h, dt, tab, &info, false);
         if (s) break;
         *t += info.dt_taken;
         ++done;
@@ -1338,7 +1347,7 @@ crkdg_status crkdg_advance_fixed(crkdg_t h, int nsteps, double dt, double t_end,
         if (!(*t < t_end)) break;
         double d = dt < t_end - *t ? dt : t_end - *t;
         crkdg_step_info info;
-        s = crkdg_step(h, d, tab, &info);
+        s = step_once(h, d, tab, &info, false);
         if (s) break;
         *t += info.dt_taken;
         if (t_end - *t <= 1e-14 * fabs(t_end)) *t = t_end;
