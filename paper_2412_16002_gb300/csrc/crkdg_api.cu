@@ -212,7 +212,14 @@ void build_tables(NodalTables *tab) {
             T.tlx[1][a] = fx_coef(T.lp[a], kFxTrace);
             T.w1x[a] = fx_coef(T.w1[a], kFxAvg);
         }
-        for (int q = 0; q < n * n; ++q) T.w2x[q] = fx_coef(T.w2[q], kFxAvg);
+        for (int q = 0; q < n * n; ++q) {
+            T.w2x[q] = fx_coef(T.w2[q], kFxAvg);
+            for (int d = 0; d < 2; ++d) T.pm2x[d][q] = fx_coef(T.pm2[d][q], kFxAvg);
+        }
+        for (int a = 0; a < n; ++a) {
+            T.xgf[0][a] = (float)T.xg[a];
+            T.xgf[1][a] = (float)(T.xg[a] - (double)T.xgf[0][a]);
+        }
     }
 }
 
@@ -422,11 +429,13 @@ void fill_f32(Params &P) {
     F.dt = (float)P.dt;
 }
 
+bool euler_2d(const crkdg_ctx *h) { return h->dim == 2 && h->phys == PH_EULER; }
+
 // 2D Euler steps whose tableau has only a sub-diagonal (every tableau of the paper) run the inner
 // stages with one thread per cell, or for Q^3 on request on the tensor cores; other cases run
 // k_inner_x.
 bool sub_diagonal_euler(const crkdg_ctx *h, const Params &P) {
-    if (h->dim != 2 || h->phys != PH_EULER || P.mode != MODE_STEP) return false;
+    if (!euler_2d(h) || P.mode != MODE_STEP) return false;
     for (int i = 0; i < P.s; ++i)
         for (int j = 0; j + 1 < i; ++j)
             if (P.A[i][j] != 0.0) return false;
@@ -438,9 +447,10 @@ cudaError_t launch_x(crkdg_ctx *h, int kernel, const Params &P0, const MixBufs &
     Params P = P0;
     fill_f32(P);
     if (kernel == KX_INNER && sub_diagonal_euler(h, P))
-        return h->tc_on && h->n == 4 ? crkdg_launch_inner_tc(h->st, P, X) : crkdg_launch_inner_cell(h->n, h->st, P, X);
-    if (kernel == KX_FINAL && h->dim == 2 && h->phys == PH_EULER && P.mode == MODE_STEP && P.fx.kon)
-        return crkdg_launch_final_cell(h->n, h->st, P, X);
+        return h->tc_on && h->n == 4 ? crkdg_launch_inner_tc(h->st, P, X) : crkdg_launch_cell(kernel, h->n, h->st, P, X);
+    if (euler_2d(h) && ((kernel == KX_FINAL && P.mode == MODE_STEP && P.fx.kon) || kernel == KX_TROUBLE ||
+                        kernel == KX_SPLIT || kernel == KX_MERGE))
+        return crkdg_launch_cell(kernel, h->n, h->st, P, X);
     int ncb = cells_per_block(h->dim, h->n);
     int nblocks = (h->ncell + ncb - 1) / ncb;
     if (h->dim == 1) return crkdg_launch_mx_1d(kernel, h->n, h->phys, nblocks, h->st, P, X);
@@ -836,11 +846,13 @@ crkdg_status crkdg_set_state(crkdg_t h, const double *nodal, size_t count, int o
             X.nod_in = src;
             X.ub_n = h->xub[h->xcur];
             X.dv_n = h->xdv[h->xcur];
-            CK(h, launch_x(h, KX_SPLIT, P, X));
-            X = base_xbufs(h);
-            X.dv_n = h->xdv[h->xcur];
             P.mode = MODE_RATE;  // the limiter also posts the trial-step rate of the limited state
-            CK(h, launch_x(h, KX_LIMIT, P, X));
+            CK(h, launch_x(h, KX_SPLIT, P, X));
+            if (!euler_2d(h)) {  // 2D Euler: in the same pass
+                X = base_xbufs(h);
+                X.dv_n = h->xdv[h->xcur];
+                CK(h, launch_x(h, KX_LIMIT, P, X));
+            }
             crkdg_status s = queue_mass(h, nullptr, h->xub[h->xcur]);
             if (s == CRKDG_OK) s = read_scalars(h);
             if (s) return s;

@@ -24,20 +24,11 @@ cudaError_t crkdg_launch_inner_tc(cudaStream_t st, const Params &P, const MixBuf
     return launch_inner_tc(st, P, X);
 }
 
-cudaError_t crkdg_launch_inner_cell(int n, cudaStream_t st, const Params &P, const MixBufs &X) {
+cudaError_t crkdg_launch_cell(int kernel, int n, cudaStream_t st, const Params &P, const MixBufs &X) {
     switch (n) {
-    case 2: return launch_inner_c<2>(st, P, X);
-    case 3: return launch_inner_c<3>(st, P, X);
-    case 4: return launch_inner_c<4>(st, P, X);
-    default: return cudaErrorInvalidValue;
-    }
-}
-
-cudaError_t crkdg_launch_final_cell(int n, cudaStream_t st, const Params &P, const MixBufs &X) {
-    switch (n) {
-    case 2: return launch_final_c<2>(st, P, X);
-    case 3: return launch_final_c<3>(st, P, X);
-    case 4: return launch_final_c<4>(st, P, X);
+    case 2: return launch_cell<2>(kernel, st, P, X);
+    case 3: return launch_cell<3>(kernel, st, P, X);
+    case 4: return launch_cell<4>(kernel, st, P, X);
     default: return cudaErrorInvalidValue;
     }
 }

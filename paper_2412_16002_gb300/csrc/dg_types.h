@@ -71,6 +71,8 @@ struct NodalTables {
     // fixed-point copies (dg_fixed.h): l_a(-1), l_a(+1) scaled by 2^kFxTrace, the average weights
     // by 2^kFxAvg
     Fx tlx[2][MAXN], w1x[MAXN], w2x[MAXN * MAXN];
+    Fx pm2x[2][MAXN * MAXN];  // pm2 scaled by 2^kFxAvg (its magnitudes sum to less than 2)
+    float xgf[2][MAXN];       // xg as a sum of two floats
 };
 constexpr int kFxTrace = 56;  // sum_a |l_a(+-1)| < 4
 constexpr int kFxAvg = 57;    // the weights sum to 1
@@ -407,8 +409,8 @@ cudaError_t crkdg_ens_control(int which, cudaStream_t st, crkdg::EnsProblem *E, 
 cudaError_t crkdg_launch_inner_tc(cudaStream_t st, const crkdg::Params &P, const crkdg::MixBufs &X);
 // The same stages on the CUDA cores, one thread per cell (2D Euler, n = 2, 3, 4, MODE_STEP, the same
 // tableaux; defined in dg_2d.cu).
-cudaError_t crkdg_launch_final_cell(int n, cudaStream_t st, const crkdg::Params &P, const crkdg::MixBufs &X);
-cudaError_t crkdg_launch_inner_cell(int n, cudaStream_t st, const crkdg::Params &P, const crkdg::MixBufs &X);
+// (kernel KX_INNER, KX_FINAL, KX_TROUBLE, KX_SPLIT with MODE_RATE also as KX_LIMIT, KX_MERGE)
+cudaError_t crkdg_launch_cell(int kernel, int n, cudaStream_t st, const crkdg::Params &P, const crkdg::MixBufs &X);
 // Closed-form nodal tables for n = 2, 3, 4 (defined in crkdg_api.cu).
 void crkdg_build_tables(crkdg::NodalTables *tab);
 // The same tables, built once per process (host memory).
