@@ -2,6 +2,7 @@
 #include "dg_core.cuh"
 #include "dg_mixed.cuh"
 #include "dg_cell.cuh"
+#include "dg_line.cuh"
 #include "dg_tc.cuh"
 
 using namespace crkdg;
@@ -26,9 +27,9 @@ cudaError_t crkdg_launch_inner_tc(cudaStream_t st, const Params &P, const MixBuf
 
 cudaError_t crkdg_launch_cell(int kernel, int n, cudaStream_t st, const Params &P, const MixBufs &X) {
     switch (n) {
-    case 2: return launch_cell<2>(kernel, st, P, X);
-    case 3: return launch_cell<3>(kernel, st, P, X);
-    case 4: return launch_cell<4>(kernel, st, P, X);
+    case 2: return launch_line<2>(kernel, st, P, X);
+    case 3: return launch_line<3>(kernel, st, P, X);
+    case 4: return launch_line<4>(kernel, st, P, X);
     default: return cudaErrorInvalidValue;
     }
 }
