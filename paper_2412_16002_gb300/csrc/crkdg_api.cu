@@ -214,9 +214,13 @@ void build_tables(NodalTables *tab) {
         }
         for (int q = 0; q < n * n; ++q) {
             T.w2x[q] = fx_coef(T.w2[q], kFxAvg);
-            for (int d = 0; d < 2; ++d) T.pm2x[d][q] = fx_coef(T.pm2[d][q], kFxAvg);
+            for (int d = 0; d < 2; ++d) {
+                T.pm2x[d][q] = fx_coef(T.pm2[d][q], kFxAvg);
+                for (int e = 0; e < 2; ++e) T.trw2x[d][e][q] = fx_coef(T.trw2[d][e][q], kFxTrace);
+            }
         }
         for (int a = 0; a < n; ++a) {
+            T.pm1x[a] = fx_coef(T.pm1[a], kFxAvg);
             T.xgf[0][a] = (float)T.xg[a];
             T.xgf[1][a] = (float)(T.xg[a] - (double)T.xgf[0][a]);
         }

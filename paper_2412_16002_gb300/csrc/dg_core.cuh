@@ -1957,6 +1957,55 @@ __device__ __forceinline__ bool tvb_changes(double t, double dp, double dm, doub
     return m != tb && ((m | tb) << 1) != 0ull;  // +0 and -0 compare equal
 }
 
+// The same decision in fixed point, all in one unit: t the deviation of the face average, dp and dm the
+// neighbour differences, thr the threshold (below zero: none).
+__device__ __forceinline__ bool tvb_changes_fx(long long t, long long dp, long long dm, long long thr) {
+    if (thr >= 0 && (t < 0 ? -t : t) <= thr) return false;
+    return t > 0 ? dp < t || dm < t : t < 0 && (dp > t || dm > t);
+}
+// x in units of 2^(E - 1081), E >= fx_exp(x), as one number
+__device__ __forceinline__ long long fx_whole(double x, int E) {
+    const Fx f = fx_of(x, E);
+    return ((long long)f.h << 28) + f.l;
+}
+// The plain indicator's decision of one direction and component: sR, sL the face averages in units of
+// 2^(En - 1081) (sums of node values with the weights scaled by 2^kFxTrace), own, lo, hi the averages of the
+// cell and its neighbours.  FP64 sums of the node values took 18 fused multiply-adds (76 cycles each) in Q^2:
+// 501 x 397 Q^2, troubled-cell pass 186 -> 110 us, features 247 -> 164 us.
+__device__ __forceinline__ bool tvb_pair(long long sR, long long sL, int En, double own, double lo, double hi,
+                                         double thr) {
+    const int E = max(max(En, fx_exp(own)), max(fx_exp(lo), fx_exp(hi)));
+    if (E == 0x7ff) return true;  // infinities and NaN
+    const int sh = min(E - En, 63);
+    const long long o = fx_whole(own, E), l = fx_whole(lo, E), h = fx_whole(hi, E);
+    const int et = fx_exp(thr);
+    long long th = 1ll << 62;  // larger than every deviation
+    if (!(thr >= 0.0)) th = -1;
+    else if (et <= E) th = fx_whole(thr, E);
+    else if (et <= E + 3) th = fx_whole(thr, et) << (et - E);
+    return tvb_changes_fx((sR >> sh) - o, h - o, o - l, th) || tvb_changes_fx(o - (sL >> sh), h - o, o - l, th);
+}
+
+// 2^k, k in [-126, 127]
+__device__ __forceinline__ float pow2f(int k) { return __int_as_float((k + 127) << 23); }
+
+// u as a sum of two floats: its leading 24 bits and the rest, on the integer units
+__device__ __forceinline__ void two_floats(double u, float &h, float &l) {
+    h = trunc_f(u);
+    const int e = (int)((dbits(u) >> 52) & 0x7ffu) - 1023;
+    const float r = (float)(int)(dbits(u) & 0x1fffffffull) * 1.862645149230957e-09f;  // 2^-29
+    l = e - 23 >= -126 && e < 128 ? copysignf(r * pow2f(e - 23), h) : 0.0f;
+}
+// d 2^-60 likewise
+__device__ __forceinline__ void two_floats_fx(long long d, float &h, float &l) {
+    const unsigned long long m = d < 0 ? 0ull - (unsigned long long)d : (unsigned long long)d;
+    const int z = min(__clzll((long long)m), 63);
+    const unsigned long long a = m << z;
+    h = (float)(int)(a >> 40) * pow2f(-20 - z);
+    l = (float)((int)(a >> 16) & 0xffffff) * pow2f(-44 - z);
+    if (d < 0) h = -h, l = -l;
+}
+
 // Average of component c of the neighbour of `cell` across `side` (the averages are in
 // aux, [cell][m]); across a domain boundary, the boundary condition applied to the
 // cell's own average.
@@ -1996,49 +2045,65 @@ __device__ __forceinline__ void trouble_body(const Params &P, const Bufs &B, int
     const int a = node % N, b = DIM == 2 ? node / N : 0;
     double u[M];
     load_node<DIM, N, PHYS>(P, B.unew, cell, node, active, u);
+    // node values in fixed point with one exponent per cell and component
+    Fx(&fu)[M][NN] = reinterpret_cast<Fx(&)[M][NN]>(S.c[lc].u);
+    constexpr int W = (M + 1) / 2;
+    unsigned eu[W];
 #pragma unroll
-    for (int c = 0; c < M; ++c) S.c[lc].u[c][node] = u[c];
+    for (int k = 0; k < W; ++k) eu[k] = 0u;
+#pragma unroll
+    for (int c = 0; c < M; ++c) eu[c >> 1] |= (unsigned)fx_exp(u[c]) << (16 * (c & 1));
+#pragma unroll
+    for (int k = 0; k < W; ++k) eu[k] = cell_max_halves<C>(eu[k], node);
+    auto field = [&](int c) { return (int)((eu[W > 1 ? c >> 1 : 0] >> (16 * (c & 1))) & 0xffffu); };
+#pragma unroll
+    for (int c = 0; c < M; ++c) fu[c][node] = fx_of(u[c], field(c));
     if (node == 0) sTr[lc] = 0;
     cell_sync<C>();
-    // the (direction, component) pairs are spread over the cell's threads: each takes the
-    // decision and the limited first moment of its pairs
-    for (int j = node; j < DIM * M && active; j += NN) {
-        const int d = j / M, c = j - d * M;
-        const double thr = P.thr[d];
-        const double own = B.aux[(size_t)cell * M + c];
-        const double lo = nb_average<PHYS, DIM>(P, B.aux, cell, 2 * d, c);
-        const double hi = nb_average<PHYS, DIM>(P, B.aux, cell, 2 * d + 1, c);
-        double fr = 0.0, fl = 0.0, p1 = 0.0;
-        for (int q = 0; q < NN; ++q) {
-            double v = S.c[lc].u[c][q];
-            if constexpr (DIM == 2) {
-                fr = fma(T.trw2[d][0][q], v, fr);
-                fl = fma(T.trw2[d][1][q], v, fl);
-                p1 = fma(T.pm2[d][q], v, p1);
-            } else {
-                fr = fma(T.lp[q], v, fr);
-                fl = fma(T.lm[q], v, fl);
-                p1 = fma(T.pm1[q], v, p1);
+    // the decision, its (direction, component) pairs spread over the cell's threads
+    if (P.ind_stage < 2) {
+        for (int j = node; j < DIM * M && active; j += NN) {
+            const int d = j / M, c = j - d * M;
+            const Fx *wr = DIM == 2 ? T.trw2x[d][0] : T.tlx[1], *wl = DIM == 2 ? T.trw2x[d][1] : T.tlx[0];
+            FxSum sr{0, 0}, sl{0, 0};
+#pragma unroll
+            for (int q = 0; q < NN; ++q) {
+                const Fx v = fu[c][q];
+                fx_mac(sr, v, wr[q]);
+                fx_mac(sl, v, wl[q]);
             }
+            if (tvb_pair(fx_sum(sr), fx_sum(sl), field(c), B.aux[(size_t)cell * M + c],
+                         nb_average<PHYS, DIM>(P, B.aux, cell, 2 * d, c),
+                         nb_average<PHYS, DIM>(P, B.aux, cell, 2 * d + 1, c), P.thr[d]))
+                atomicOr(&sTr[lc], 1);
         }
-        double utR = fr - own, utL = own - fl;
-        double dp = hi - own, dm = own - lo;
-        const bool thr_ok = thr >= 0.0;
-        if (tvb_changes(utR, dp, dm, thr, thr_ok) || tvb_changes(utL, dp, dm, thr, thr_ok)) atomicOr(&sTr[lc], 1);
-        sP1[lc][d][c] = minmod3_bits(p1, dp, dm);
+        cell_sync<C>();
     }
-    cell_sync<C>();
     bool troubled = active && (P.ind_stage >= 2 ? B.tflags[cell] != 0 : sTr[lc] != 0);
     if (P.ind_stage == 3 && active) {  // learned flags: p > 0.6 troubled, p < 0.4 smooth, else the plain flag
         const float pr = B.prob[cell];
         troubled = pr > 0.6f ? true : (pr < 0.4f ? false : troubled);
     }
-    if (troubled) {
+    if (__any_sync(0xffffffffu, troubled)) {  // the limited first moments, spread likewise
+        for (int j = node; j < DIM * M && troubled; j += NN) {
+            const int d = j / M, c = j - d * M;
+            const Fx *w = DIM == 2 ? T.pm2x[d] : T.pm1x;
+            FxSum s{0, 0};
 #pragma unroll
-        for (int c = 0; c < M; ++c) {
-            double v = fma(sP1[lc][0][c], T.xg[a], B.aux[(size_t)cell * M + c]);
-            if constexpr (DIM == 2) v = fma(sP1[lc][1][c], T.xg[b], v);
-            u[c] = v;
+            for (int q = 0; q < NN; ++q) fx_mac(s, fu[c][q], w[q]);
+            const double own = B.aux[(size_t)cell * M + c];
+            sP1[lc][d][c] = minmod3_bits(fx_double(fx_sum(s), fx_shift(field(c), kFxAvg)),
+                                         nb_average<PHYS, DIM>(P, B.aux, cell, 2 * d + 1, c) - own,
+                                         own - nb_average<PHYS, DIM>(P, B.aux, cell, 2 * d, c));
+        }
+        cell_sync<C>();
+        if (troubled) {
+#pragma unroll
+            for (int c = 0; c < M; ++c) {
+                double v = fma(sP1[lc][0][c], T.xg[a], B.aux[(size_t)cell * M + c]);
+                if constexpr (DIM == 2) v = fma(sP1[lc][1][c], T.xg[b], v);
+                u[c] = v;
+            }
         }
     }
     if (node == 0 && active) {
@@ -2107,11 +2172,11 @@ __device__ __forceinline__ void stencil_features(const Params &P, const double *
     const double thr = P.thr_feat;
 #pragma unroll
     for (int c = 0; c < M; ++c) {
-        double mean = 0.0;
         unsigned long long kmx = kKeyNegInf, kmn = kKeyPosInf, kab = 0ull;
+        int E = 0;
 #pragma unroll
         for (int q = 0; q < 9; ++q) {
-            mean += v[q][c];
+            E = max(E, fx_exp(v[q][c]));
             if (!isnan_bits(v[q][c])) {  // fmax / fmin ignore NaN
                 const unsigned long long k = ordbits(v[q][c]);
                 kmx = umax64(kmx, k);
@@ -2120,8 +2185,32 @@ __device__ __forceinline__ void stencil_features(const Params &P, const double *
             }
         }
         const double mx = ordbits_inv(kmx), mn = ordbits_inv(kmn), amax = bitsd(kab);
+        const double den = fmax(mx - mn, thr) + (1e-6 * amax + 1e-30);
+        scale[c] = recip_nr(den);
+        if (E < 1900) {
+            // 9 (v - mean) exactly in fixed point, times scale / 9 as a product of sums of two floats, rounded
+            // once: the FP64 sums, division, products and conversions took 38 FP64 instructions a component
+            long long m[9], sum = 0;
+#pragma unroll
+            for (int q = 0; q < 9; ++q) {
+                m[q] = fx_whole(v[q][c], E) >> 2;
+                sum += m[q];
+            }
+            float sh, sl;  // 2^(E - 1079) scale / 9 for mantissas in units of 2^-60
+            two_floats(scale[c] * (1.0 / 9.0) * bitsd((unsigned long long)(E + 4) << 52), sh, sl);
+#pragma unroll
+            for (int q = 0; q < 9; ++q) {
+                float dh, dl;
+                two_floats_fx(9 * m[q] - sum, dh, dl);
+                const float p = __fmul_rn(dh, sh);
+                f[c * 9 + q] = p + (fmaf(dh, sh, -p) + fmaf(dh, sl, dl * sh));
+            }
+            continue;
+        }
+        double mean = 0.0;
+#pragma unroll
+        for (int q = 0; q < 9; ++q) mean += v[q][c];
         mean /= 9.0;
-        scale[c] = recip_nr(fmax(mx - mn, thr) + (1e-6 * amax + 1e-30));
 #pragma unroll
         for (int q = 0; q < 9; ++q) f[c * 9 + q] = (float)((v[q][c] - mean) * scale[c]);
     }
@@ -2140,40 +2229,36 @@ __device__ __forceinline__ void features_body(const Params &P, const Bufs &B, in
         double v[9][M], scale[M];
         stencil_features<PHYS>(P, B.aux, cell, B.feat + (size_t)cell * 44, v, scale);
         float *f = B.feat + (size_t)cell * 44;
+        // the first moments, and the plain indicator's decision for this cell (the troubled-cell kernel's
+        // arithmetic): the label of harvested features and the fallback of the learned flags
+        int trouble = 0;
 #pragma unroll
         for (int c = 0; c < M; ++c) {
             const double *u = B.unew + ((size_t)c * P.ncell + cell) * NN;
-            double cx = 0.0, cy = 0.0;
+            double w[NN];
+            int En = 0;
 #pragma unroll
             for (int q = 0; q < NN; ++q) {
-                int qa = q % N, qb = q / N;
-                double w = T.mom2[q] * u[q];
-                cx = fma(w, T.xg[qa], cx);
-                cy = fma(w, T.xg[qb], cy);
+                w[q] = u[q];
+                En = max(En, fx_exp(w[q]));
             }
-            f[36 + 2 * c] = (float)(cx * scale[c]);
-            f[37 + 2 * c] = (float)(cy * scale[c]);
-        }
-        // the plain indicator's decision for this cell, with the troubled-cell kernel's
-        // arithmetic: the label of harvested features and the fallback of the learned flags
-        int trouble = 0;
+            FxSum s[2] = {{0, 0}, {0, 0}}, r[2] = {{0, 0}, {0, 0}}, l[2] = {{0, 0}, {0, 0}};
 #pragma unroll
-        for (int d = 0; d < 2; ++d) {
-            const double thr = P.thr[d];
-            const double *lo = v[d == 0 ? 3 : 1], *hi = v[d == 0 ? 5 : 7], *own = v[4];
-            const bool thr_ok = thr >= 0.0;
+            for (int q = 0; q < NN; ++q) {
+                const Fx x = fx_of(w[q], En);
 #pragma unroll
-            for (int c = 0; c < M; ++c) {
-                const double *uc = B.unew + ((size_t)c * P.ncell + cell) * NN;
-                double fr = 0.0, fl = 0.0;
-                for (int q = 0; q < NN; ++q) {
-                    double val = uc[q];
-                    fr = fma(T.trw2[d][0][q], val, fr);
-                    fl = fma(T.trw2[d][1][q], val, fl);
+                for (int d = 0; d < 2; ++d) {
+                    fx_mac(s[d], x, T.pm2x[d][q]);
+                    fx_mac(r[d], x, T.trw2x[d][0][q]);
+                    fx_mac(l[d], x, T.trw2x[d][1][q]);
                 }
-                double utR = fr - own[c], utL = own[c] - fl;
-                double dp = hi[c] - own[c], dm = own[c] - lo[c];
-                if (tvb_changes(utR, dp, dm, thr, thr_ok) || tvb_changes(utL, dp, dm, thr, thr_ok)) trouble = 1;
+            }
+#pragma unroll
+            for (int d = 0; d < 2; ++d) {
+                const double m = En == 0x7ff ? NAN : fx_double(fx_sum(s[d]), fx_shift(En, kFxAvg));
+                f[36 + 2 * c + d] = (float)(m * scale[c]);
+                if (tvb_pair(fx_sum(r[d]), fx_sum(l[d]), En, v[4][c], v[d == 0 ? 3 : 1][c], v[d == 0 ? 5 : 7][c], P.thr[d]))
+                    trouble = 1;
             }
         }
         if (B.tflags) B.tflags[cell] = trouble;

@@ -63,14 +63,6 @@ __device__ __forceinline__ float cell_max(float x, int base) {
                  __shfl_sync(0xffffffffu, x, base + 2));
 }
 
-// u as a sum of two floats: its leading 24 bits and the rest, on the integer units
-__device__ __forceinline__ void two_floats(double u, float &h, float &l) {
-    h = trunc_f(u);
-    const int e = (int)((dbits(u) >> 52) & 0x7ffu) - 1023;
-    const float r = (float)(int)(dbits(u) & 0x1fffffffull) * 1.862645149230957e-09f;  // 2^-29
-    l = e - 23 >= -126 && e < 128 ? copysignf(r * pow2f(e - 23), h) : 0.0f;
-}
-
 // One line of a cell (direction DIR): u the deviations at its nodes, dens the density rule; g the line's
 // part of G (volume term and lifts), tr its end traces, gsum the face sums with weight wk.
 template <int N, int DIR, class Density>
