@@ -360,6 +360,7 @@ Bufs base_bufs(const crkdg_ctx *h) {
     B.tavg = h->tr ? h->tr + (size_t)h->tr_slots * h->m * h->ncell * h->ntr : nullptr;
     B.tsum = h->tr ? h->tr + (size_t)h->tr_slots * h->m * h->ncell * (h->ntr + 1) : nullptr;
     B.tsp = h->tr ? B.tsum + (size_t)h->m * h->ncell * h->ntr : nullptr;
+    B.fc = h->tr && h->dim == 2 ? B.tsp + (size_t)h->tr_slots * h->ncell * 4 : nullptr;
     B.flag = &h->scal->flag;
     B.nlim = &h->scal->nlim;
     B.thmin = &h->scal->thmin;
@@ -542,10 +543,10 @@ crkdg_status ensure_traces(crkdg_ctx *h, int slots) {
     h->tr = nullptr;
     h->tr_slots = 0;
     // traces [slot][m][cell][face point], the traced stages' cell averages [slot][m][cell], then
-    // the weighted sum of the traces' normal fluxes [m][cell][face point] and each stage's
-    // largest radius per face [slot][cell][face]
+    // the weighted sum of the traces' normal fluxes [m][cell][face point], each stage's
+    // largest radius per face [slot][cell][face], and in 2D the faces' corrections (Bufs::fc)
     size_t bytes = ((size_t)slots * h->m * h->ncell * (h->ntr + 1) + (size_t)h->m * h->ncell * h->ntr +
-                    (size_t)slots * h->ncell * 2 * h->dim) *
+                    (size_t)slots * h->ncell * 2 * h->dim + (h->dim == 2 ? (size_t)h->m * h->ncell * h->ntr : 0)) *
                    sizeof(double);
     CK(h, cudaMalloc(&h->tr, bytes));
     h->tr_slots = slots;

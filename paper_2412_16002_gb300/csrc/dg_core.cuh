@@ -1676,14 +1676,53 @@ __device__ __forceinline__ void lift_faces(const Params &P, double dt, CellData<
     }
 }
 
+// Corrections of the interior faces of a 2D mesh, one thread per face point (a cell's lower faces): for the
+// cells on both sides dc = sum_i b_i (fhat^(i) - f_int^(i)) = (F_ext - F_int) / 2 - sum_i b_i alpha^(i) (u_R^(i) -
+// u_L^(i)) / 2, F the weighted flux sums, from what the inner kernel stored.  In the final kernel every face
+// was evaluated by both of its cells, in Q^2 by two rounds of nine threads for twelve points, all on the
+// FP64 pipe (84% busy).
+template <int N, int PHYS>
+__global__ void __launch_bounds__(128) k_faces(const __grid_constant__ Params P, const __grid_constant__ Bufs B) {
+    constexpr int M = ncomp(PHYS, 2), NTR = 4 * N;
+    const size_t per = (size_t)P.ncell * N, e = (size_t)blockIdx.x * 128 + threadIdx.x;  // points of a direction
+    if (e >= 2 * per) return;
+    const int dir = e >= per, face = 2 * dir;
+    const size_t at = dir ? e - per : e;  // cell * N + pos
+    const int cell = (int)(at / N), pos = (int)(at - (size_t)cell * N);
+    // the cell below, whatever condition either side of the face has: the final kernel decides side by side
+    const int cy = cell / P.nx, cx = cell - cy * P.nx;
+    const bool wrap = P.bc[face] == BC_PERIODIC || P.bc[face + 1] == BC_PERIODIC;
+    if ((dir ? cy : cx) == 0 && !wrap) return;
+    const int nb = dir ? (cy > 0 ? cell - P.nx : cell + (P.ny - 1) * P.nx) : (cx > 0 ? cell - 1 : cell + P.nx - 1);
+    const size_t cstr = (size_t)P.ncell * NTR, ro = (size_t)cell * NTR + face * N + pos, lo = (size_t)nb * NTR + (face + 1) * N + pos;
+    double dc[M];
+#pragma unroll
+    for (int c = 0; c < M; ++c) dc[c] = 0.0;
+    for (int i = 0; i < P.s; ++i) {
+        const int q = P.slot[i];
+        if (q < 0) continue;
+        const double *tr = B.tr + (size_t)q * M * cstr, *sp = B.tsp + (size_t)q * P.ncell * 4;
+        const double ba = half_of(P.b[i]) * fmax_nonneg(sp[(size_t)cell * 4 + face], sp[(size_t)nb * 4 + face + 1]);
+#pragma unroll
+        for (int c = 0; c < M; ++c) dc[c] = fma(ba, tr[c * cstr + lo] - tr[c * cstr + ro], dc[c]);
+    }
+#pragma unroll
+    for (int c = 0; c < M; ++c) {
+        const double d = B.tsum[c * cstr + lo] - B.tsum[c * cstr + ro];
+        B.fc[(size_t)(2 * dir * M + c) * per + at] = fma(0.5, d, dc[c]);         // the cell above the face
+        B.fc[(size_t)((2 * dir + 1) * M + c) * per + at] = fma(-0.5, d, dc[c]);  // and below
+    }
+}
+
 // Final stage: u^{n+1} = u* + dt lift( sum_i b_i (fhat^(i) - f(u_int^(i))) ), then the
 // limiter, the admissibility test and a0 of the new state.  Each face flux is
 // evaluated from the same differences by both cells sharing the face, so the update is
-// conservative to round-off.  Bound by the FP64 pipe: 9 FP64 instructions per face point and
-// traced stage are left of 28 (the inner kernel leaves the weighted flux sums, one set for all
-// stages, and the faces' radii), the lift runs in fixed point, and the rate is taken only by
-// warps that can raise it (513^2 Q^3: 1.15 ms a launch with the fluxes of every stage read back).
-template <int DIM, int N, int PHYS, bool STORED = false>
+// conservative to round-off.  The face corrections come from k_faces (FACES: 2D steps), boundary faces
+// excepted; or from the flux sums and radii that the inner kernel stored (STORED: ensembles, 1D); or
+// all of it is evaluated here (RECOMPUTED: the operators without a handle).  The lift runs in fixed
+// point, and the rate is taken only by warps that can raise it.
+enum FaceSource { RECOMPUTED = 0, STORED = 1, FACES = 2 };
+template <int DIM, int N, int PHYS, int FROM = RECOMPUTED>
 __device__ __forceinline__ void final_body(const Params &P, const Bufs &B, int blk) {
     using C = CfgW<DIM, N, PHYS>;
     constexpr int M = C::M, NN = C::NN, NF = C::NF, NTR = C::NTR, FPT = C::FPT;
@@ -1699,8 +1738,7 @@ __device__ __forceinline__ void final_body(const Params &P, const Bufs &B, int b
 
     // dc = sum_i b_i (fhat^(i) - f_int^(i)) = (F_ext - F_int) / 2 -+ sum_i b_i alpha^(i) (u_ext^(i) - u_int^(i)) / 2
     // with F = sum_i b_i f^(i), the sign of the side: both cells of a face form the same
-    // differences.  F and the faces' radii as the inner kernel stored them (STORED), else
-    // recomputed here; the exterior state of a boundary face always here.
+    // differences.  The exterior state of a boundary face is always evaluated here.
     CellData<C> &D = S.c[lc];
     double(&sI)[NTR][M] = D.tf;  // this thread's running sums F (own face points only)
     double(&sE)[NTR][M] = reinterpret_cast<double(&)[NTR][M]>(D.f);
@@ -1708,83 +1746,95 @@ __device__ __forceinline__ void final_body(const Params &P, const Bufs &B, int b
     double dc[FPT][M];
     size_t noff[FPT];  // the partner point's offset within a component's block
     int nbr[FPT];
+    bool here = FROM != FACES;  // a face point of this thread is evaluated here
 #pragma unroll
     for (int j = 0; j < FPT; ++j) {
-        const int fp = node + j * NN;
+        const int fp = node + j * NN, face = fp / NF, pos = fp - face * NF;
         nbr[j] = -1;
         noff[j] = 0;
         if (fp < NTR && active) {
-            const int face = fp / NF, pos = fp - face * NF;
             nbr[j] = neighbour_geo(P, cell, face);
             if (nbr[j] >= 0) noff[j] = (size_t)nbr[j] * NTR + (face ^ 1) * NF + pos;
+            here = here || nbr[j] < 0;
         }
 #pragma unroll
-        for (int c = 0; c < M; ++c) {
-            dc[j][c] = 0.0;
-            if (fp < NTR) sE[fp][c] = sI[fp][c] = 0.0;
+        for (int c = 0; c < M; ++c) dc[j][c] = 0.0;
+        if (FROM == FACES && nbr[j] >= 0) {
+            const double *fc = B.fc + (size_t)face * M * P.ncell * NF + (size_t)((face & 1) ? nbr[j] : cell) * NF + pos;
+#pragma unroll
+            for (int c = 0; c < M; ++c) dc[j][c] = fc[(size_t)c * P.ncell * NF];
         }
     }
-    for (int i = 0; i < P.s; ++i) {
-        if (P.slot[i] < 0) continue;
-        const double *tr = B.tr + (size_t)P.slot[i] * M * cstr;
-        const double *sps = STORED ? B.tsp + (size_t)P.slot[i] * P.ncell * (2 * DIM) : nullptr;
-        const double bi = P.b[i];
+    if (__any_sync(0xffffffffu, here)) {
+#pragma unroll
+        for (int j = 0; j < FPT; ++j)
+            if (node + j * NN < NTR)
+#pragma unroll
+                for (int c = 0; c < M; ++c) sE[node + j * NN][c] = sI[node + j * NN][c] = 0.0;
+        for (int i = 0; i < P.s; ++i) {
+            if (P.slot[i] < 0) continue;
+            const double *tr = B.tr + (size_t)P.slot[i] * M * cstr;
+            const double *sps = FROM != RECOMPUTED ? B.tsp + (size_t)P.slot[i] * P.ncell * (2 * DIM) : nullptr;
+            const double bi = P.b[i];
+#pragma unroll
+            for (int j = 0; j < FPT; ++j) {
+                const int fp = node + j * NN;
+                const int face = fp / NF, pos = fp - face * NF, dir = face >> 1;
+                const bool mine = fp < NTR && active && (FROM != FACES || nbr[j] < 0);
+                double ui[M], ue[M], alpha = 0.0;
+                if (mine) {
+                    const int nb = nbr[j];
+                    double f[M];
+#pragma unroll
+                    for (int c = 0; c < M; ++c) ui[c] = tr[c * cstr + (size_t)cell * NTR + fp];
+                    if constexpr (FROM != RECOMPUTED) {
+                        alpha = sps[(size_t)cell * (2 * DIM) + face];
+                    } else {
+                        alpha = fmax_nonneg(alpha, face_flux<PHYS, DIM>(P, ui, dir, true, f));
+#pragma unroll
+                        for (int c = 0; c < M; ++c) sI[fp][c] = fma(bi, f[c], sI[fp][c]);
+                    }
+                    if (nb >= 0) {
+#pragma unroll
+                        for (int c = 0; c < M; ++c) ue[c] = tr[c * cstr + noff[j]];
+                        if constexpr (FROM != RECOMPUTED)
+                            alpha = fmax_nonneg(alpha, sps[(size_t)nb * (2 * DIM) + (face ^ 1)]);
+                    } else {
+                        double av[M];
+#pragma unroll
+                        for (int c = 0; c < M; ++c) av[c] = B.tavg[((size_t)P.slot[i] * M + c) * P.ncell + cell];
+                        if (P.geo != nullptr)
+                            geo_exterior<PHYS, DIM, N>(P, cell, face, pos, i, ui, av, ue);
+                        else
+                            exterior_state<PHYS, DIM>(P, face, ui, av, ue);
+                    }
+                    if (FROM == RECOMPUTED || nb < 0) {
+                        alpha = fmax_nonneg(alpha, face_flux<PHYS, DIM>(P, ue, dir, true, f));
+#pragma unroll
+                        for (int c = 0; c < M; ++c) sE[fp][c] = fma(bi, f[c], sE[fp][c]);
+                    }
+                }
+                __syncwarp();
+                alpha = face_max<C>(alpha, node);  // per-edge LF viscosity: max over the edge's points
+                if (mine) {
+                    const double h = half_of(bi);
+                    const double ba = ((face & 1) ? -h : h) * alpha;
+#pragma unroll
+                    for (int c = 0; c < M; ++c) dc[j][c] = fma(ba, ue[c] - ui[c], dc[j][c]);
+                }
+            }
+        }
 #pragma unroll
         for (int j = 0; j < FPT; ++j) {
             const int fp = node + j * NN;
-            const int face = fp / NF, pos = fp - face * NF, dir = face >> 1;
-            double ui[M], ue[M], alpha = 0.0;
-            if (fp < NTR && active) {
-                const int nb = nbr[j];
-                double f[M];
+            if (fp < NTR && active && (FROM != FACES || nbr[j] < 0))
 #pragma unroll
-                for (int c = 0; c < M; ++c) ui[c] = tr[c * cstr + (size_t)cell * NTR + fp];
-                if constexpr (STORED) {
-                    alpha = sps[(size_t)cell * (2 * DIM) + face];
-                } else {
-                    alpha = fmax_nonneg(alpha, face_flux<PHYS, DIM>(P, ui, dir, true, f));
-#pragma unroll
-                    for (int c = 0; c < M; ++c) sI[fp][c] = fma(bi, f[c], sI[fp][c]);
+                for (int c = 0; c < M; ++c) {
+                    const double FI = FROM != RECOMPUTED ? B.tsum[c * cstr + (size_t)cell * NTR + fp] : sI[fp][c];
+                    const double FE = FROM != RECOMPUTED && nbr[j] >= 0 ? B.tsum[c * cstr + noff[j]] : sE[fp][c];
+                    dc[j][c] = fma(0.5, FE - FI, dc[j][c]);
                 }
-                if (nb >= 0) {
-#pragma unroll
-                    for (int c = 0; c < M; ++c) ue[c] = tr[c * cstr + noff[j]];
-                    if constexpr (STORED) alpha = fmax_nonneg(alpha, sps[(size_t)nb * (2 * DIM) + (face ^ 1)]);
-                } else {
-                    double av[M];
-#pragma unroll
-                    for (int c = 0; c < M; ++c) av[c] = B.tavg[((size_t)P.slot[i] * M + c) * P.ncell + cell];
-                    if (P.geo != nullptr)
-                        geo_exterior<PHYS, DIM, N>(P, cell, face, pos, i, ui, av, ue);
-                    else
-                        exterior_state<PHYS, DIM>(P, face, ui, av, ue);
-                }
-                if (!STORED || nb < 0) {
-                    alpha = fmax_nonneg(alpha, face_flux<PHYS, DIM>(P, ue, dir, true, f));
-#pragma unroll
-                    for (int c = 0; c < M; ++c) sE[fp][c] = fma(bi, f[c], sE[fp][c]);
-                }
-            }
-            __syncwarp();
-            alpha = face_max<C>(alpha, node);  // per-edge LF viscosity: max over the edge's points
-            if (fp < NTR && active) {
-                const double h = half_of(bi);
-                const double ba = ((face & 1) ? -h : h) * alpha;
-#pragma unroll
-                for (int c = 0; c < M; ++c) dc[j][c] = fma(ba, ue[c] - ui[c], dc[j][c]);
-            }
         }
-    }
-#pragma unroll
-    for (int j = 0; j < FPT; ++j) {
-        const int fp = node + j * NN;
-        if (fp < NTR && active)
-#pragma unroll
-            for (int c = 0; c < M; ++c) {
-                const double FI = STORED ? B.tsum[c * cstr + (size_t)cell * NTR + fp] : sI[fp][c];
-                const double FE = STORED && nbr[j] >= 0 ? B.tsum[c * cstr + noff[j]] : sE[fp][c];
-                dc[j][c] = fma(0.5, FE - FI, dc[j][c]);
-            }
     }
     cell_sync<C>();
     lift_faces<C>(P, P.dt, S.c[lc], node, a, b, dc, u);
@@ -1831,10 +1881,10 @@ __device__ __forceinline__ void final_body(const Params &P, const Bufs &B, int b
 // Resident blocks per SM the FP64 final kernel's register budget is sized for (96 registers).
 constexpr int fp64_final_min_blocks() { return 5; }
 
-template <int DIM, int N, int PHYS, bool STORED>
+template <int DIM, int N, int PHYS, int FROM>
 __global__ void __launch_bounds__(kWarpThreads, fp64_final_min_blocks())
     k_final(Params P, Bufs B) {
-    final_body<DIM, N, PHYS, STORED>(P, B, blockIdx.x);
+    final_body<DIM, N, PHYS, FROM>(P, B, blockIdx.x);
 }
 
 // Limiter applied to a state (set-up projection, operator checks): un -> unew.  In
@@ -2270,6 +2320,11 @@ __global__ void k_features(Params P, Bufs B) {
     features_body<DIM, N, PHYS>(P, B, blockIdx.x);
 }
 
+// Meshes from this size on take the faces' corrections in a pass of their own (k_faces): below it a step is
+// bound by latency, and the pass is one more launch (64^2 Q^2 9 + 18 us against 20 for the final kernel alone;
+// 1024^2 Q^2 0.43 + 0.56 ms against 1.86, 513^2 Q^3 0.24 + 0.21 against 0.67).  The bits are the same.
+constexpr int kFacesCells = 16384;
+
 template <int DIM, int N, int PHYS>
 cudaError_t launch_one(int kernel, cudaStream_t st, const Params &P, const Bufs &B) {
     using C = CfgW<DIM, N, PHYS>;
@@ -2277,10 +2332,15 @@ cudaError_t launch_one(int kernel, cudaStream_t st, const Params &P, const Bufs 
     switch (kernel) {
     case K_INNER: k_inner<DIM, N, PHYS><<<nblocks, C::NT, 0, st>>>(P, B); break;
     case K_FINAL:
-        if (B.tsum)
-            k_final<DIM, N, PHYS, true><<<nblocks, C::NT, 0, st>>>(P, B);
-        else
-            k_final<DIM, N, PHYS, false><<<nblocks, C::NT, 0, st>>>(P, B);
+        if (!B.tsum) {
+            k_final<DIM, N, PHYS, RECOMPUTED><<<nblocks, C::NT, 0, st>>>(P, B);
+        } else if (DIM == 2 && P.ncell >= kFacesCells) {
+            const size_t points = 2 * (size_t)P.ncell * N;
+            k_faces<N, PHYS><<<(unsigned)((points + 127) / 128), 128, 0, st>>>(P, B);
+            k_final<DIM, N, PHYS, FACES><<<nblocks, C::NT, 0, st>>>(P, B);
+        } else {
+            k_final<DIM, N, PHYS, STORED><<<nblocks, C::NT, 0, st>>>(P, B);
+        }
         break;
     case K_LIMIT: k_limit<DIM, N, PHYS><<<nblocks, C::NT, 0, st>>>(P, B); break;
     case K_TROUBLE: k_trouble<DIM, N, PHYS><<<nblocks, C::NT, 0, st>>>(P, B); break;

@@ -23,7 +23,11 @@ __device__ __forceinline__ void ens_bufs(const EnsProblem &E, Bufs &B) {
     B.ustar = E.ustar;
     B.tr = E.tr;
     B.tavg = E.tavg;
-    B.tsum = B.tsp = nullptr;  // the final kernel recomputes the traces' fluxes
+    // behind the traces: the weighted flux sums and the faces' radii (the host's sizes)
+    const size_t face_values = (size_t)4 * E.P.ncell * (4 * N);
+    B.tsum = E.tr + (size_t)max(E.P.nslot, 1) * face_values;
+    B.tsp = B.tsum + face_values;
+    B.fc = nullptr;
     B.flag = &E.sc->flag;
     B.nlim = &E.sc->nlim;
     B.thmin = &E.sc->thmin;
@@ -41,7 +45,7 @@ __device__ __forceinline__ void ens_body(const Params &P, const Bufs &B, int blk
     if constexpr (KIND == ENS_INNER) {
         inner_body<2, N, PH_EULER>(P, B, blk);
     } else if constexpr (KIND == ENS_FINAL) {
-        final_body<2, N, PH_EULER>(P, B, blk);
+        final_body<2, N, PH_EULER, STORED>(P, B, blk);
     } else if constexpr (KIND == ENS_TROUBLE) {
         trouble_body<2, N, PH_EULER>(P, B, blk);
     } else {

@@ -266,6 +266,9 @@ struct Bufs {
     // the traces [m][cell][face point], and each traced stage's largest radius over a face's
     // points [slot][cell][face]
     double *tsum = nullptr, *tsp = nullptr;
+    // 2D, with tsum: the faces' corrections for the cells above and below them
+    // [direction][above, below][m][cell of the lower face][face point]
+    double *fc = nullptr;
     int *flag;          // set when a stage average leaves B
     unsigned long long *nlim;   // limited cells
     unsigned long long *thmin;  // bits of the smallest theta (non-negative double)
