@@ -8,8 +8,8 @@ dt control).  One bench step = one cRKDG time step of the workload.
 Default workload (N=1): the largest single-GPU configuration, the 2D Euler
 (gamma 1.4) Sedov-type blast on [0,1.1]^2, 2048 x 2048 cells, Q^3, four-stage
 fourth-order cRKDG (CFL 0.103), split precision: FP64 cell averages, limiter
-decisions, conservation sums and time step; FP32-level operators, the inner stages'
-maps as three-product TF32 tensor-core GEMMs.  Other configurations: --workload
+decisions, conservation sums and time step; FP32-level operators, line by line
+(the inner stages on request as three-product TF32 tensor-core GEMMs).  Other configurations: --workload
 (e.g. sedov_shell_2048_q3_mixed times the same configuration on a developed blast).
 
 Arms:
@@ -74,13 +74,14 @@ DEFAULT_STEPS = {"euler1d": 2000, "burgers": 2000, "sedov": 50, "sedov_shell": 5
                  "double_mach": 50, "shock_diffraction": 50}
 
 
-def launches_per_attempt(precision, indicator):
-    """Kernels one step attempt launches: the inner and final stages; the indicator: the
+def launches_per_attempt(precision, indicator, cells=0):
+    """Kernels one step attempt launches: the inner and final stages; in FP64 on a 2D mesh of 16384
+    cells and more the face pass; the indicator: the
     troubled-cell pass, after (learned) the feature kernel and the network's forward pass, on
     the split path also the merge to FP64 nodal values the feature kernel reads; then the
     component totals of the new state for the step's conservation drift (two reduction
     kernels, after the FP64 path's cell-average kernel)."""
-    n = 2 + (2 if precision == "mixed" else 3)
+    n = 2 + (2 if precision == "mixed" else 3) + (precision != "mixed" and cells >= 16384)
     if indicator == "tvb":
         n += 1
     elif indicator == "mlp":
@@ -503,8 +504,9 @@ def run_decomposed(args, wl, name):
         avg_inner = kt["inner"] / max(kn["inner"], 1)
         avg_final = kt["final"] / max(kn["final"], 1)
         sfx = "_x" if precision == "mixed" else ""
-        isfx = "_tc" if (precision == "mixed" and wl.dim == 2 and wl.k == 3 and wl.flux == "euler") else sfx
-        dom_k, avg_ms, fl = ("k_inner" + isfx, avg_inner, inner_f) if avg_inner >= avg_final else \
+        if precision == "mixed" and wl.dim == 2 and wl.flux == "euler":
+            sfx = "_l"
+        dom_k, avg_ms, fl = ("k_inner" + sfx, avg_inner, inner_f) if avg_inner >= avg_final else \
             ("k_final" + sfx, avg_final, final_f)
         achieved = fl * lay.nxl * lay.nyl / (avg_ms / 1e3) / 1e12
         peak = FP32_PEAK_TFLOPS if precision == "mixed" else FP64_PEAK_TFLOPS
@@ -522,7 +524,7 @@ def run_decomposed(args, wl, name):
                          "note": "rank 0's dominant kernel over its local cells (owned block and halo ring)"},
             "e2e": {"value": e2e_value, "unit": "cell-DOF-stage/s", "h2d_bytes_per_step": nbytes,
                     "d2h_bytes_per_step": nbytes},
-            "gpu_launches": int(kn["inner"]) * launches_per_attempt(precision, "off") * world,
+            "gpu_launches": int(kn["inner"]) * launches_per_attempt(precision, "off", lay.nxl * lay.nyl) * world,
             "clocks": clocks,
         }
         print(json.dumps(line))
@@ -636,15 +638,16 @@ def run_gb300(args, wl, name):
         avg_inner = kt["inner"] / max(kn["inner"], 1)
         avg_final = kt["final"] / max(kn["final"], 1)
         sfx = "_x" if precision == "mixed" else ""
-        # the split path's 2D Euler Q^3 inner stages run on the tensor cores (k_inner_tc)
-        isfx = "_tc" if (precision == "mixed" and wl.dim == 2 and wl.k == 3 and wl.flux == "euler") else sfx
+        # the split path's 2D Euler stages run line by line (k_inner_l, k_final_l)
+        if precision == "mixed" and wl.dim == 2 and wl.flux == "euler":
+            sfx = "_l"
         if kn["run"] > 0:
             avg_run = kt["run"] / kn["run"]
             dom, avg_ms, fl = "k_run1d", avg_run, (inner_f + final_f) * args.steps
         elif avg_inner >= avg_final or indicator != "off":
             # with an indicator the final window also holds the indicator's kernels; the
             # inner window is one kernel
-            dom, avg_ms, fl = "k_inner" + isfx, avg_inner, inner_f
+            dom, avg_ms, fl = "k_inner" + sfx, avg_inner, inner_f
         else:
             dom, avg_ms, fl = "k_final" + sfx, avg_final, final_f
         achieved = fl * active_cells(wl) / (avg_ms / 1e3) / 1e12
@@ -676,7 +679,7 @@ def run_gb300(args, wl, name):
                          "flops_per_cell": {"k_inner": inner_f, "k_final": final_f}},
             "e2e": {"value": e2e_value, "unit": "cell-DOF-stage/s", "h2d_bytes_per_step": nbytes,
                     "d2h_bytes_per_step": nbytes},
-            "gpu_launches": int(kn["run"]) if kn["run"] else int(kn["inner"]) * launches_per_attempt(precision, indicator),
+            "gpu_launches": int(kn["run"]) if kn["run"] else int(kn["inner"]) * launches_per_attempt(precision, indicator, wl.nx * wl.ny if wl.dim == 2 else 0),
             "clocks": clocks,
         }
         if world == 1 and not args.no_cpu_baseline:

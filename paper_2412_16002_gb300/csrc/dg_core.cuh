@@ -263,9 +263,13 @@ __device__ __forceinline__ double fx_face_speed(const FxGas &gas, const FxPoint<
     const int d = DIM == 2 ? dir : 0;
     const long long w = DIM == 2 && d ? o.w[DIM - 1] : o.w[0];
     const int xw = DIM == 2 && d ? o.xw[DIM - 1] : o.xw[0];
-    double c = 0.0;  // sound speed: c^2 = gamma p / rho
-    if (o.p > 0) c = sqrt(fx_value(fx_mul(fx_limb(fx_mul(fx_limb(o.p), fx_limb(o.r))), gas.g), o.X - o.xr + 2));
-    return __dadd_rn(fx_value(w < 0 ? -w : w, xw), c);
+    const long long a = w < 0 ? -w : w;
+    if (o.p <= 0) return fx_value(a, xw);
+    // sound speed: c^2 = gamma p / rho
+    int xc;
+    const long long c = fx_root(fx_mul(fx_limb(fx_mul(fx_limb(o.p), fx_limb(o.r))), gas.g), o.X - o.xr + 2, xc);
+    const int x = xw > xc ? xw : xc;
+    return fx_value(fx_shr(a, x - xw) + fx_shr(c, x - xc), x);
 }
 
 // Normal flux f and spectral radius (returned) of one state at a face point: on the integer
@@ -1169,9 +1173,11 @@ __device__ __forceinline__ unsigned biased_exp(int x) { return (unsigned)max(x +
 // shares a warp with.
 //
 // Why: with FP64 maps and fluxes a warp issued about 145 FP64 instructions per Q^3 stage, 76 cycles
-// each; now about 40, with 2100 instructions on the other pipes beside them.  Set state, steps, get
+// each; now about 30, with 2000 instructions on the other pipes beside them.  Set state, steps, get
 // state: 513^2 Q^3, 2 RK4 steps 15.9 -> 11.8 (maps) -> 5.8 (fluxes and the final stage) -> 5.0 ms (no
-// fallback for small momenta); 1024^2 Q^2, 3 Heun steps 49.7 -> 40.0 -> 22.2 ms.
+// fallback for small momenta); 1024^2 Q^2, 3 Heun steps 49.7 -> 40.0 -> 22.2 ms.  The integer root of the
+// sound speed, a sub-diagonal tableau's G in registers and face rounds without a branch: a launch 1.56 ->
+// 1.43 ms and 4.92 -> 4.50 ms.
 template <class C, class Put, class Fn>
 __device__ __forceinline__ void eval_G_fx(const Params &P, Smem<C> &S, const BlockTab<C> &Tb, int lc, int node,
                                           const double *u, double *g, bool want_speed, bool want_avg, Put put,
@@ -1185,6 +1191,8 @@ __device__ __forceinline__ void eval_G_fx(const Params &P, Smem<C> &S, const Blo
     Fx(&ff)[C::D][M][NN] = reinterpret_cast<Fx(&)[C::D][M][NN]>(D.f);
     Fx(&ft)[M][NTR] = reinterpret_cast<Fx(&)[M][NTR]>(D.tf);
     auto field = [](const unsigned (&w)[W], int c) { return (int)((w[c >> 1] >> (16 * (c & 1))) & 0xffffu); };
+    // whether round j gives this thread a face point: known at compile time but for a ragged last round
+    auto is_point = [&](int j) { return (j + 1) * NN <= NTR || node + j * NN < NTR; };
     bool bad = P.fx.on == 0;
     // 1. node values in fixed point
     unsigned eu[W];
@@ -1214,7 +1222,7 @@ __device__ __forceinline__ void eval_G_fx(const Params &P, Smem<C> &S, const Blo
 #pragma unroll
     for (int j = 0; j < FPT; ++j) {
         const int fp = node + j * NN;
-        if (fp < NTR) {
+        if (is_point(j)) {
             const int face = fp / NF, pos = fp - face * NF;
             const int at = DIM == 1 || face < 2 ? pos * N : pos, step = DIM == 1 || face < 2 ? 1 : N;
             Fx l[N];
@@ -1237,7 +1245,7 @@ __device__ __forceinline__ void eval_G_fx(const Params &P, Smem<C> &S, const Blo
     for (int j = 0; j < FPT; ++j) {
         const int fp = node + j * NN;
         double f[M], sp = 0.0;
-        if (fp < NTR) {
+        if (is_point(j)) {
             const int dir = fp / NF >> 1;
             if constexpr (PHYS == PH_EULER) {
                 FxPoint<DIM> o;
@@ -1264,7 +1272,7 @@ __device__ __forceinline__ void eval_G_fx(const Params &P, Smem<C> &S, const Blo
             }
         }
         if (want_speed) sp = face_max<C>(sp, node);
-        if (fp < NTR && !mine) put(j, t[j], f, sp);
+        if (is_point(j) && !mine) put(j, t[j], f, sp);
     }
     if (want_avg) {
         if constexpr (DIM == 2 && NN == 16 && M == 4) {  // four lanes of four nodes per component
@@ -1317,7 +1325,7 @@ __device__ __forceinline__ void eval_G_fx(const Params &P, Smem<C> &S, const Blo
 #pragma unroll
         for (int j = 0; j < FPT; ++j) {
             const int fp = node + j * NN;
-            if (fp < NTR) {
+            if (is_point(j)) {
                 ft[0][fp] = fx_limbs(tm[j][0], tx[j][0], E0);
                 ft[1][fp] = fx_limbs(tm[j][1], tx[j][1], E1);
                 if constexpr (DIM == 2) ft[2][fp] = fx_limbs(tm[j][2], tx[j][1], E1);
@@ -1337,7 +1345,7 @@ __device__ __forceinline__ void eval_G_fx(const Params &P, Smem<C> &S, const Blo
         if constexpr (DIM == 2) ff[1][0][node] = fx_of(fy[0], (int)e.w0);
 #pragma unroll
         for (int j = 0; j < FPT; ++j)
-            if (node + j * NN < NTR) ft[0][node + j * NN] = fx_of(tf0[j], (int)e.w0);
+            if (is_point(j)) ft[0][node + j * NN] = fx_of(tf0[j], (int)e.w0);
     }
     cell_sync<C>();
     // 4. G: the row, the column and the four lifted face fluxes
@@ -1380,7 +1388,7 @@ __device__ __forceinline__ void eval_G_fx(const Params &P, Smem<C> &S, const Blo
 #pragma unroll
             for (int j = 0; j < FPT; ++j) {
                 const int fp = node + j * NN;
-                if (fp < NTR) {
+                if (is_point(j)) {
                     double sp = 0.0;
                     if (want_speed)
                         for (int q = 0; q < NF; ++q) sp = fmax_nonneg(sp, D.ts[fp / NF * NF + q]);
@@ -1521,7 +1529,12 @@ __device__ __forceinline__ void inner_body(const Params &P, const Bufs &B, int b
     const bool active = cell < P.ncell;
     const bool own = active && owned(P, cell) && !solid_cell(P, cell);  // counts in the flag and statistics
     fill_tab<C>(P, Tb);
-    double un[M], cur[M], acc[M], gh[MAXS][M];  // gh is indexed by the stage loop: local memory, in L1
+    double un[M], cur[M], acc[M], g[M];
+    // only a tableau with entries below its sub-diagonal needs the earlier stages' G: local memory
+    bool sub = true;
+    for (int i = 2; i < P.s; ++i)
+        for (int j = 0; j + 1 < i; ++j) sub = sub && !nonzero_bits(P.A[i][j]);
+    double gh[MAXS][M];
     load_node<DIM, N, PHYS>(P, B.un, cell, node, active, un);
 #pragma unroll
     for (int c = 0; c < M; ++c) cur[c] = acc[c] = un[c];
@@ -1538,17 +1551,21 @@ __device__ __forceinline__ void inner_body(const Params &P, const Bufs &B, int b
         if (i > 0) {
 #pragma unroll
             for (int c = 0; c < M; ++c) cur[c] = un[c];
-#pragma unroll 1
-            for (int j = 0; j < i; ++j)
-                if (nonzero_bits(P.A[i][j]))
+            if (sub) {
 #pragma unroll
-                    for (int c = 0; c < M; ++c) cur[c] = fma(Tb.dtA[i][j], gh[j][c], cur[c]);
+                for (int c = 0; c < M; ++c) cur[c] = fma(Tb.dtA[i][i - 1], g[c], cur[c]);
+            } else {
+#pragma unroll 1
+                for (int j = 0; j < i; ++j)
+                    if (nonzero_bits(P.A[i][j]))
+#pragma unroll
+                        for (int c = 0; c < M; ++c) cur[c] = fma(Tb.dtA[i][j], gh[j][c], cur[c]);
+            }
             if (P.pk) project_pk<C>(S, lc, node, cur);
             double pts[C::PPT][M];
             float rhi;
             limit_block(P, B, S, lc, node, own, cur, pts, true, true, false, rhi);
         }
-        double g[M];
         const int slot = P.slot[i];
         const bool traced = slot >= 0 && active;
         const bool keep_faces = slot >= 0 && B.tsum != nullptr;
@@ -1571,8 +1588,9 @@ __device__ __forceinline__ void inner_body(const Params &P, const Bufs &B, int b
                 if (active) B.tavg[((size_t)slot * M + c) * P.ncell + cell] = v;  // outflow exterior state
             });
         if (P.source && active) add_source<DIM, N, PHYS>(P, cell, node, i, g);
+        if (!sub)
 #pragma unroll
-        for (int c = 0; c < M; ++c) gh[i][c] = g[c];
+            for (int c = 0; c < M; ++c) gh[i][c] = g[c];
         if (P.mode == MODE_OP_G) {
 #pragma unroll
             for (int c = 0; c < M; ++c) acc[c] = g[c];

@@ -157,6 +157,45 @@ CRKDG_HD long long fx_recip(long long M) {
     return ((long long)r0 << 31) + (w >> 21);
 }
 
+// Mantissa and exponent (m 2^(xr - 61), 2^60 <= m <= 2^61) of the root of v 2^(x - 61), v >= 0: with f the
+// value over an even power of two in [1, 4), y the FP32 reciprocal root of its leading bits (e = 1 - f y^2
+// below 2^-21) and t = f y, t (1 + e/2 + 3 e^2 / 8), within about 2^-57.  Eight IMAD.WIDE, where FP64's root
+// holds its pipe for about 690 cycles.
+CRKDG_HD long long fx_root(long long v, int x, int &xr) {
+    if (v <= 0) {
+        xr = -4000;
+        return 0;
+    }
+#ifdef __CUDA_ARCH__
+    const int z = __clzll(v);
+#else
+    const int z = __builtin_clzll((unsigned long long)v);
+#endif
+    const long long M = v << (z - 1);    // [2^62, 2^63)
+    const int e2 = x - 61 - z + 1 + 62;  // the value is (M 2^-62) 2^e2
+    const int odd = e2 & 1, h = (e2 - odd) >> 1;
+    const unsigned fb = (0x3f800000u + ((unsigned)odd << 23)) | ((unsigned)(M >> 39) & 0x7fffffu);
+#ifdef __CUDA_ARCH__
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(__uint_as_float(fb)));
+    const int y0 = __float2int_rn(y * 1073741824.0f);
+#else
+    float f;
+    memcpy(&f, &fb, 4);
+    const int y0 = (int)lrintf((1.0f / sqrtf(f)) * 1073741824.0f);
+#endif
+    const long long a = M >> (2 - odd);  // f 2^60
+    const int ah = (int)(a >> 31), al = (int)a & 0x7fffffff;
+    const long long t = (((long long)ah * y0) << 1) + (((long long)al * y0) >> 30);
+    const int th = (int)(t >> 31), tl = (int)t & 0x7fffffff;
+    const long long e = (1ll << 60) - ((((long long)th * y0) << 1) + (((long long)tl * y0) >> 30));
+    const int eh = (int)(e >> 8);
+    const long long c = (e >> 1) + ((3 * (((long long)eh * eh) >> 44)) >> 3);
+    const int ch = (int)(c >> 8), cl = (int)c & 255;
+    xr = h + 1;
+    return t + (((long long)th * ch) >> 21) + (((long long)th * cl) >> 29) + (((long long)tl * ch) >> 52);
+}
+
 // gamma - 1 and gamma as mantissas: g1 2^-62 and g 2^(-61)
 struct FxGas {
     Limb g1, g;
