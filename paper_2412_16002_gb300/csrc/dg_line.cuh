@@ -468,66 +468,80 @@ __device__ __forceinline__ bool line_rate(const Params &P, float eps, const floa
     return ok;
 }
 
-// One face of a cell (this thread's R points of it): the sum over the traced stages of b_i (fhat - f_int) (dc)
-// and of b_i fhat (fh).
-template <int N, int FACE>
+// The two faces of a cell across direction DIR (this thread's R points of each): the sums over the traced stages
+// of b_i (fhat - f_int) (dc) and of b_i fhat (fh).  A stage's loads for both faces are issued together:
+// the kernel waits on them with three to five warps a scheduler (face by face 3.14 ms, 26 and 370 us).
+template <int N, int DIR>
 __device__ __forceinline__ void face_sums(const Params &P, const MixBufs &X, int cell, bool active, int h, int base,
-                                          float (&dc)[M][Line<N>::R], float (&fh)[M][Line<N>::R]) {
-    constexpr int R = Line<N>::R, DIR = FACE >> 1, NTR = 4 * N;
+                                          float (&dc)[2][M][Line<N>::R], float (&fh)[2][M][Line<N>::R]) {
+    constexpr int R = Line<N>::R, NTR = 4 * N;
     const size_t cs = (size_t)P.ncell, tcs = cs * NTR;
-    const int nb = active ? neighbour(P, cell, FACE) : -1;
-    const size_t io = (size_t)(active ? cell : 0) * NTR + FACE * N + R * h, eo = (size_t)max(nb, 0) * NTR + (FACE ^ 1) * N + R * h;
+    int nb[2];
+    size_t io[2], eo[2];
 #pragma unroll
-    for (int c = 0; c < M; ++c)
+    for (int f = 0; f < 2; ++f) {
+        const int face = 2 * DIR + f;
+        nb[f] = active ? neighbour(P, cell, face) : -1;
+        io[f] = (size_t)(active ? cell : 0) * NTR + face * N + R * h;
+        eo[f] = (size_t)max(nb[f], 0) * NTR + (face ^ 1) * N + R * h;
 #pragma unroll
-        for (int r = 0; r < R; ++r) dc[c][r] = fh[c][r] = 0.0f;
+        for (int c = 0; c < M; ++c)
+#pragma unroll
+            for (int r = 0; r < R; ++r) dc[f][c][r] = fh[f][c][r] = 0.0f;
+    }
 #pragma unroll 1
     for (int i = 0; i < P.s; ++i) {
         const int slot = P.slot[i];
         if (slot < 0) continue;
         const float *tr = X.tr + (size_t)slot * M * tcs;
-        float ui[M][R], ue[M][R];
+        float ui[2][M][R], ue[2][M][R];
 #pragma unroll
-        for (int c = 0; c < M; ++c) {
+        for (int f = 0; f < 2; ++f)
 #pragma unroll
-            for (int r = 0; r < R; ++r) ui[c][r] = ue[c][r] = c == 0 || c == M - 1 ? 1.0f : 0.0f;
-            if (active) load_run<R>(tr + c * tcs + io, ui[c]);
-            if (nb >= 0) load_run<R>(tr + c * tcs + eo, ue[c]);
-        }
-        if (active && nb < 0) {
-            float av[M];
+            for (int c = 0; c < M; ++c) {
 #pragma unroll
-            for (int c = 0; c < M; ++c) av[c] = X.tavg[((size_t)slot * M + c) * cs + cell];
+                for (int r = 0; r < R; ++r) ui[f][c][r] = ue[f][c][r] = c == 0 || c == M - 1 ? 1.0f : 0.0f;
+                if (active) load_run<R>(tr + c * tcs + io[f], ui[f][c]);
+                if (nb[f] >= 0) load_run<R>(tr + c * tcs + eo[f], ue[f][c]);
+            }
+        const float bi = P.f.b[i];
+#pragma unroll
+        for (int f = 0; f < 2; ++f) {
+            if (active && nb[f] < 0) {
+                float av[M];
+#pragma unroll
+                for (int c = 0; c < M; ++c) av[c] = X.tavg[((size_t)slot * M + c) * cs + cell];
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    float a[M], b[M];
+#pragma unroll
+                    for (int c = 0; c < M; ++c) a[c] = ui[f][c][r];
+                    exterior_state_f<PH_EULER, 2>(P, 2 * DIR + f, a, av, b);
+#pragma unroll
+                    for (int c = 0; c < M; ++c) ue[f][c][r] = b[c];
+                }
+            }
+            float fi[R][M], fe[R][M], alpha = 0.0f;
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 float a[M], b[M];
 #pragma unroll
-                for (int c = 0; c < M; ++c) a[c] = ui[c][r];
-                exterior_state_f<PH_EULER, 2>(P, FACE, a, av, b);
-#pragma unroll
-                for (int c = 0; c < M; ++c) ue[c][r] = b[c];
+                for (int c = 0; c < M; ++c) a[c] = ui[f][c][r], b[c] = ue[f][c][r];
+                alpha = fmaxf(alpha, face_flux_f<DIR>(P, a, fi[r]));
+                alpha = fmaxf(alpha, face_flux_f<DIR>(P, b, fe[r]));
             }
+            alpha = cell_max<N>(alpha, base);
+            const float ha = -0.5f * alpha;
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int c = 0; c < M; ++c) {
+                    const float du = f ? __fsub_rn(ue[f][c][r], ui[f][c][r]) : __fsub_rn(ui[f][c][r], ue[f][c][r]);
+                    const float fhat = fmaf(ha, du, __fmul_rn(0.5f, __fadd_rn(fi[r][c], fe[r][c])));
+                    dc[f][c][r] = fmaf(bi, __fsub_rn(fhat, fi[r][c]), dc[f][c][r]);
+                    fh[f][c][r] = fmaf(bi, fhat, fh[f][c][r]);
+                }
         }
-        float fi[R][M], fe[R][M], alpha = 0.0f;
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            float a[M], b[M];
-#pragma unroll
-            for (int c = 0; c < M; ++c) a[c] = ui[c][r], b[c] = ue[c][r];
-            alpha = fmaxf(alpha, face_flux_f<DIR>(P, a, fi[r]));
-            alpha = fmaxf(alpha, face_flux_f<DIR>(P, b, fe[r]));
-        }
-        alpha = cell_max<N>(alpha, base);
-        const float bi = P.f.b[i], ha = -0.5f * alpha;
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-#pragma unroll
-            for (int c = 0; c < M; ++c) {
-                const float du = (FACE & 1) ? __fsub_rn(ue[c][r], ui[c][r]) : __fsub_rn(ui[c][r], ue[c][r]);
-                const float fhat = fmaf(ha, du, __fmul_rn(0.5f, __fadd_rn(fi[r][c], fe[r][c])));
-                dc[c][r] = fmaf(bi, __fsub_rn(fhat, fi[r][c]), dc[c][r]);
-                fh[c][r] = fmaf(bi, fhat, fh[c][r]);
-            }
     }
 }
 
@@ -551,7 +565,7 @@ __device__ __forceinline__ RunSum cell_run(const RunSum &p, int base) {
 // four faces, their lifts along its rows and columns, and their fixed-point sums into the averages; then
 // the limiter, or with the indicator the averages and the unlimited deviations for the troubled-cell
 // pass.  The FP64 part of the averages is spread over the cell's threads.  Against one thread per cell:
-// 2048^2 Q^3 3.53 -> 3.14 ms a launch, 131^2 Q^3 47 -> 26 us, 1024^2 Q^2 376 -> 370 us.
+// 2048^2 Q^3 3.53 -> 3.11 ms a launch, 131^2 Q^3 47 -> 23 us, 1024^2 Q^2 376 -> 347 us.
 template <int N>
 __global__ void __launch_bounds__(pc::LT, pc::Line<N>::BLOCKS) k_final_l(const __grid_constant__ Params P, const __grid_constant__ MixBufs X) {
     using namespace pc;
@@ -573,15 +587,16 @@ __global__ void __launch_bounds__(pc::LT, pc::Line<N>::BLOCKS) k_final_l(const _
 #pragma unroll
     for (int c = 0; c < M; ++c) sum[c] = RunSum{0, 0};
     {
-        float da[M][R], db[M][R], fh[M][R];
-        auto add = [&](const Fx *k, bool minus) {
+        float dc[2][M][R], fh[2][M][R];
+        auto add = [&](const Fx *k) {
 #pragma unroll
-            for (int c = 0; c < M; ++c) run_add<R>(sum[c], fh[c], k + R * h, minus);
+            for (int c = 0; c < M; ++c) {
+                run_add<R>(sum[c], fh[0][c], k + R * h, false);
+                run_add<R>(sum[c], fh[1][c], k + R * h, true);
+            }
         };
-        face_sums<N, 2>(P, X, cell, active, h, base, da, fh);
-        add(P.fx.ky, false);
-        face_sums<N, 3>(P, X, cell, active, h, base, db, fh);
-        add(P.fx.ky, true);
+        face_sums<N, 1>(P, X, cell, active, h, base, dc, fh);
+        add(P.fx.ky);
 #pragma unroll
         for (int c = 0; c < M; ++c)
 #pragma unroll
@@ -589,19 +604,17 @@ __global__ void __launch_bounds__(pc::LT, pc::Line<N>::BLOCKS) k_final_l(const _
 #pragma unroll
                 for (int b = 0; b < N; ++b)
                     s_buf[c][cl][N * b + R * h + j] =
-                        fmaf(-T.liftpf[b], P.f.rhy * db[c][j], T.liftmf[b] * (P.f.rhy * da[c][j]));
+                        fmaf(-T.liftpf[b], P.f.rhy * dc[1][c][j], T.liftmf[b] * (P.f.rhy * dc[0][c][j]));
         __syncwarp();
-        face_sums<N, 0>(P, X, cell, active, h, base, da, fh);
-        add(P.fx.kx, false);
-        face_sums<N, 1>(P, X, cell, active, h, base, db, fh);
-        add(P.fx.kx, true);
+        face_sums<N, 0>(P, X, cell, active, h, base, dc, fh);
+        add(P.fx.kx);
 #pragma unroll
         for (int c = 0; c < M; ++c)
 #pragma unroll
             for (int r = 0; r < R; ++r)
 #pragma unroll
                 for (int a = 0; a < N; ++a)
-                    dv[c][r][a] = fmaf(-T.liftpf[a], P.f.rhx * db[c][r], T.liftmf[a] * (P.f.rhx * da[c][r]));
+                    dv[c][r][a] = fmaf(-T.liftpf[a], P.f.rhx * dc[1][c][r], T.liftmf[a] * (P.f.rhx * dc[0][c][r]));
         add_rows<N>(s_buf, cl, h, dv);
         __syncwarp();
     }
