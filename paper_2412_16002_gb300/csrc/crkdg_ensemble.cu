@@ -54,11 +54,12 @@ struct crkdg_ensemble_ctx {
     long long total_cells = 0;
     bool harvest = false;
     // work items: [group n=3,4][0 cell blocks, 1 feature blocks]
+    int final_kind = ENS_FINAL;  // or ENS_FINAL_BARE
     EnsItem *ditems[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
     int nitems[2][2] = {{0, 0}, {0, 0}};
     int cap_items[2][2] = {{0, 0}, {0, 0}};
     int tile[NCLASS] = {4, 4, 4, 4, 4, 4};
-    int occ[2][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}};  // resident blocks per SM, [group][kind]
+    int occ[2][5] = {};  // resident blocks per SM, [group][kind]
     cudaGraphExec_t g_step = nullptr, g_attempt = nullptr;
     bool graphs_valid = false;
     bool prof = false;
@@ -143,7 +144,7 @@ crkdg_status enqueue_attempt(crkdg_ens_t e) {
         return cudaSuccess;
     };
     ECK(e, run(ENS_INNER, 0));
-    ECK(e, run(ENS_FINAL, 0));
+    ECK(e, run(e->final_kind, 0));
     const int ind = e->opt.indicator;
     if (ind != CRKDG_IND_OFF) {
         const bool learned = ind == CRKDG_IND_MLP;
@@ -355,7 +356,7 @@ crkdg_status crkdg_ensemble_create(int count, const crkdg_ens_problem *problems,
         return bail(CRKDG_E_CUDA);
     if (cudaStreamCreateWithFlags(&e->st, cudaStreamNonBlocking) != cudaSuccess) return bail(CRKDG_E_CUDA);
     for (int g = 0; g < 2; ++g)
-        for (int kind = 0; kind < 4; ++kind) e->occ[g][kind] = crkdg_ens_occupancy(kind, g + 3);
+        for (int kind = 0; kind < 5; ++kind) e->occ[g][kind] = crkdg_ens_occupancy(kind, g + 3);
     NodalTables tab[3];
     crkdg_build_tables(tab);
     if (crkdg_upload_tables_2d(tab) != cudaSuccess || crkdg_upload_tables_ens(tab) != cudaSuccess)
@@ -363,9 +364,9 @@ crkdg_status crkdg_ensemble_create(int count, const crkdg_ens_problem *problems,
 
     // sizes and arena offsets (slices aligned to 32 doubles)
     const bool ind = e->opt.indicator != CRKDG_IND_OFF;
-    std::vector<size_t> off_u(count), off_tr(count), off_tavg(count), off_aux(count);
+    std::vector<size_t> off_u(count), off_tr(count), off_bare(count), off_tavg(count), off_aux(count);
     std::vector<long long> off_cell(count);
-    size_t tot_u = 0, tot_tr = 0, tot_tavg = 0, tot_aux = 0;
+    size_t tot_u = 0, tot_tr = 0, tot_bare = 0, tot_tavg = 0, tot_aux = 0;
     long long tot_cells = 0;
     for (int i = 0; i < count; ++i) {
         const int n = problems[i].k + 1;
@@ -377,6 +378,8 @@ crkdg_status crkdg_ensemble_create(int count, const crkdg_ens_problem *problems,
         off_tr[i] = tot_tr;
         // the traces of each stage, their weighted flux sums, and the faces' radii of each stage
         tot_tr += align_up((size_t)(std::max(ns, 1) + 1) * 4 * nc * 4 * n + (size_t)std::max(ns, 1) * nc * 4, 32);
+        off_bare[i] = tot_bare;  // the traces alone
+        tot_bare += align_up((size_t)std::max(ns, 1) * 4 * nc * 4 * n, 32);
         off_tavg[i] = tot_tavg;
         tot_tavg += align_up((size_t)std::max(ns, 1) * 4 * nc, 32);
         off_aux[i] = tot_aux;
@@ -387,8 +390,7 @@ crkdg_status crkdg_ensemble_create(int count, const crkdg_ens_problem *problems,
     e->total_cells = tot_cells;
     auto alloc = [&](void **p, size_t bytes) { return cudaMalloc(p, std::max<size_t>(bytes, 256)) == cudaSuccess; };
     bool ok = alloc((void **)&e->arena_u[0], tot_u * 8) && alloc((void **)&e->arena_u[1], tot_u * 8) &&
-              alloc((void **)&e->arena_ustar, tot_u * 8) && alloc((void **)&e->arena_tr, tot_tr * 8) &&
-              alloc((void **)&e->arena_tavg, tot_tavg * 8) &&
+              alloc((void **)&e->arena_ustar, tot_u * 8) && alloc((void **)&e->arena_tavg, tot_tavg * 8) &&
               alloc((void **)&e->arena_aux, tot_aux * 8) && alloc((void **)&e->dsc, sizeof(EnsScal) * count) &&
               alloc((void **)&e->dctl, sizeof(EnsCtl)) && alloc((void **)&e->dprob, sizeof(EnsProblem) * count);
     if (ok && ind) ok = alloc((void **)&e->arena_flags, sizeof(int) * (size_t)tot_cells);
@@ -396,6 +398,14 @@ crkdg_status crkdg_ensemble_create(int count, const crkdg_ens_problem *problems,
         ok = alloc((void **)&e->arena_feat, sizeof(float) * CRKDG_MLP_NIN * (size_t)tot_cells) &&
              alloc((void **)&e->arena_prob, sizeof(float) * (size_t)tot_cells) &&
              alloc((void **)&e->mlp, sizeof(float) * CRKDG_MLP_NPARAM);
+    }
+    // last: where the flux sums and radii do not fit beside the traces, the final kernel recomputes them
+    bool stored = true;
+    if (ok && !alloc((void **)&e->arena_tr, tot_tr * 8)) {
+        cudaGetLastError();
+        stored = false;
+        e->final_kind = ENS_FINAL_BARE;
+        ok = alloc((void **)&e->arena_tr, tot_bare * 8);
     }
     if (!ok) return bail(CRKDG_E_OOM);
     if (cudaMallocHost(&e->hpend, sizeof(int)) != cudaSuccess) return bail(CRKDG_E_OOM);
@@ -448,7 +458,8 @@ crkdg_status crkdg_ensemble_create(int count, const crkdg_ens_problem *problems,
         p.u[0] = e->arena_u[0] + off_u[i];
         p.u[1] = e->arena_u[1] + off_u[i];
         p.ustar = e->arena_ustar + off_u[i];
-        p.tr = e->arena_tr + off_tr[i];
+        p.tr = e->arena_tr + (stored ? off_tr[i] : off_bare[i]);
+        p.stored = stored ? 1 : 0;
         p.tavg = e->arena_tavg + off_tavg[i];
         p.aux = e->arena_aux + off_aux[i];
         p.tflags = ind ? e->arena_flags + off_cell[i] : nullptr;
@@ -661,7 +672,7 @@ crkdg_status crkdg_ensemble_autotune(crkdg_ens_t e, int reps, int chosen[6]) {
                     err = crkdg_ens_launch(ENS_INNER, g + 3, grid_of(e, ENS_INNER, g + 3, cnt), e->st, e->dprob,
                                            e->ditems[g][0], cnt, e->dctl, 0, 0);
                 if (err == cudaSuccess)
-                    err = crkdg_ens_launch(ENS_FINAL, g + 3, grid_of(e, ENS_FINAL, g + 3, cnt), e->st, e->dprob,
+                    err = crkdg_ens_launch(e->final_kind, g + 3, grid_of(e, e->final_kind, g + 3, cnt), e->st, e->dprob,
                                            e->ditems[g][0], cnt, e->dctl, 1, 0);
                 if (err == cudaSuccess) err = cudaEventRecord(ev1, e->st);
                 if (err == cudaSuccess) err = cudaEventSynchronize(ev1);

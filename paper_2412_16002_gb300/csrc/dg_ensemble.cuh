@@ -23,10 +23,10 @@ __device__ __forceinline__ void ens_bufs(const EnsProblem &E, Bufs &B) {
     B.ustar = E.ustar;
     B.tr = E.tr;
     B.tavg = E.tavg;
-    // behind the traces: the weighted flux sums and the faces' radii (the host's sizes)
+    // behind the traces: the weighted flux sums and the faces' radii (the host's sizes), where they fit
     const size_t face_values = (size_t)4 * E.P.ncell * (4 * N);
-    B.tsum = E.tr + (size_t)max(E.P.nslot, 1) * face_values;
-    B.tsp = B.tsum + face_values;
+    B.tsum = E.stored ? E.tr + (size_t)max(E.P.nslot, 1) * face_values : nullptr;
+    B.tsp = E.stored ? B.tsum + face_values : nullptr;
     B.fc = nullptr;
     B.flag = &E.sc->flag;
     B.nlim = &E.sc->nlim;
@@ -46,6 +46,8 @@ __device__ __forceinline__ void ens_body(const Params &P, const Bufs &B, int blk
         inner_body<2, N, PH_EULER>(P, B, blk);
     } else if constexpr (KIND == ENS_FINAL) {
         final_body<2, N, PH_EULER, STORED>(P, B, blk);
+    } else if constexpr (KIND == ENS_FINAL_BARE) {
+        final_body<2, N, PH_EULER, RECOMPUTED>(P, B, blk);
     } else if constexpr (KIND == ENS_TROUBLE) {
         trouble_body<2, N, PH_EULER>(P, B, blk);
     } else {
@@ -61,7 +63,7 @@ constexpr int ens_threads() {
 // Persistent launch over the work items of one degree.  stage: the troubled-cell
 // kernel's ind_stage (ENS_TROUBLE only).
 template <int N, int KIND>
-__global__ void __launch_bounds__(ens_threads<N, KIND>(), KIND == ENS_FEATURES ? 1 : KIND == ENS_FINAL ? 5 : 4) k_ens(EnsProblem *E, const EnsItem *items, int nitems,
+__global__ void __launch_bounds__(ens_threads<N, KIND>(), KIND == ENS_FEATURES ? 1 : KIND == ENS_FINAL || KIND == ENS_FINAL_BARE ? 5 : 4) k_ens(EnsProblem *E, const EnsItem *items, int nitems,
                                                                 EnsCtl *ctl, int counter, int stage) {
     __shared__ Params sP;
     __shared__ Bufs sB;

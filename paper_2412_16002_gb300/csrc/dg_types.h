@@ -337,7 +337,7 @@ struct EnsProblem {
     int status;              // 0, or CRKDG_E_BOUNDS after max_halvings
     int restarts;            // halvings of the current step
     int klass;               // (n - 3) * 3 + size class, for tuning
-    int pad;
+    int stored;              // tr also holds the flux sums and the faces' radii
     double t, t_end, cfl, a0;
     long long steps, restarts_total;
     // the last accepted step
@@ -352,7 +352,8 @@ struct EnsItem {
 };
 
 enum { ENS_COUNTERS = 16 };
-enum EnsKernelKind { ENS_INNER = 0, ENS_FINAL = 1, ENS_TROUBLE = 2, ENS_FEATURES = 3 };
+// ENS_FINAL_BARE: the final stage of ensembles whose flux sums and radii do not fit (EnsProblem::stored)
+enum EnsKernelKind { ENS_INNER = 0, ENS_FINAL = 1, ENS_TROUBLE = 2, ENS_FEATURES = 3, ENS_FINAL_BARE = 4 };
 struct EnsCtl {
     unsigned int counter[ENS_COUNTERS];  // one work counter per persistent launch of an attempt
     int any_pending;
