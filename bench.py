@@ -654,7 +654,8 @@ def run_gb300(args, wl, name):
         # the split path runs its operators in FP32: its roofline is the FP32 peak
         peak = FP32_PEAK_TFLOPS if precision == "mixed" else FP64_PEAK_TFLOPS
         peak_src = ("FP32 derived from unit count and clock (152 SMs x 128 lanes x 2 x 2070 MHz)" if precision == "mixed"
-                    else "FP64 derived from unit count and clock (152 SMs x 4 flop/clk x 2070 MHz)")
+                    else "FP64 derived from unit count and clock (152 SMs x 4 flop/clk x 2070 MHz); Euler sums, fluxes "
+                         "and roots run on the integer units, so the fraction can exceed 1")
         line = {
             "metric": "cell-DOF updates/s per RK stage",
             "value": value,
