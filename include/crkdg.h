@@ -332,8 +332,8 @@ crkdg_status crkdg_set_run1d_chunk(crkdg_t h, int cells);
 /* Split precision (CRKDG_PREC_MIXED), 2D Euler, k = 3, tableaux whose A has only a
  * sub-diagonal (eq. cRKDG2-4): on = 1 runs the inner stages on the tensor cores
  * (tcgen05.mma kind::tf32 with the three-product split, FP32-level accuracy), on = 0
- * (the default, the faster form at every measured size) on the CUDA cores with one
- * thread per cell.  Both keep FP64 where the split path does; they differ by FP32
+ * (the default, the faster form at every measured size) on the CUDA cores with two
+ * threads per cell.  Both keep FP64 where the split path does; they differ by FP32
  * rounding.  Other cases always use the CUDA cores.  A wait for the tensor cores that
  * runs out (1 s) makes crkdg_step return CRKDG_E_TIMEOUT with the state at u^n. */
 crkdg_status crkdg_set_tensor_cores(crkdg_t h, int on);

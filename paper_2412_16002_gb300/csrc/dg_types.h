@@ -412,9 +412,9 @@ cudaError_t crkdg_ens_control(int which, cudaStream_t st, crkdg::EnsProblem *E, 
 // Inner stages of the split-precision path on the tensor cores (2D Euler, n = 4, MODE_STEP,
 // tableaux whose A has only a sub-diagonal; defined in dg_2d.cu).
 cudaError_t crkdg_launch_inner_tc(cudaStream_t st, const crkdg::Params &P, const crkdg::MixBufs &X);
-// The same stages on the CUDA cores, one thread per cell (2D Euler, n = 2, 3, 4, MODE_STEP, the same
-// tableaux; defined in dg_2d.cu).
-// (kernel KX_INNER, KX_FINAL, KX_TROUBLE, KX_SPLIT with MODE_RATE also as KX_LIMIT, KX_MERGE)
+// The split path's passes of 2D Euler, n = 2, 3, 4: the stages by lines (KX_INNER for the same tableaux,
+// KX_FINAL, MODE_STEP), the others with one thread per cell (KX_TROUBLE, KX_MERGE, KX_SPLIT, with
+// MODE_RATE also as KX_LIMIT); defined in dg_2d.cu.
 cudaError_t crkdg_launch_cell(int kernel, int n, cudaStream_t st, const crkdg::Params &P, const crkdg::MixBufs &X);
 // Closed-form nodal tables for n = 2, 3, 4 (defined in crkdg_api.cu).
 void crkdg_build_tables(crkdg::NodalTables *tab);
