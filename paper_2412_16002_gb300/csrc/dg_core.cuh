@@ -498,6 +498,13 @@ __device__ __forceinline__ void place(int &lc, int &node) {
     }
 }
 
+// whether this lane shadows a cell's last node: what a thread reads and rewrites in shared memory is for
+// the node's own lane alone, a shadow's turn would count it again
+template <class C>
+__device__ __forceinline__ bool shadow_lane() {
+    return C::WARP && (int)(threadIdx.x & 31) >= (32 / C::NN) * C::NN;
+}
+
 // barrier (with a vote) over the threads that share a cell's data
 template <class C>
 __device__ __forceinline__ void cell_sync() {
@@ -1758,7 +1765,10 @@ __device__ __forceinline__ void final_body(const Params &P, const Bufs &B, int b
     // with F = sum_i b_i f^(i), the sign of the side: both cells of a face form the same
     // differences.  The exterior state of a boundary face is always evaluated here.
     CellData<C> &D = S.c[lc];
-    double(&sI)[NTR][M] = D.tf;  // this thread's running sums F (own face points only)
+    // running sums F of this thread's face points: the point's own lane forms them, and the lanes that shadow it
+    // read them behind the warp barrier (six Q^2 lanes hold the same point)
+    const bool first = !shadow_lane<C>();
+    double(&sI)[NTR][M] = D.tf;
     double(&sE)[NTR][M] = reinterpret_cast<double(&)[NTR][M]>(D.f);
     const size_t cstr = (size_t)P.ncell * NTR;
     double dc[FPT][M];
@@ -1786,7 +1796,7 @@ __device__ __forceinline__ void final_body(const Params &P, const Bufs &B, int b
     if (__any_sync(0xffffffffu, here)) {
 #pragma unroll
         for (int j = 0; j < FPT; ++j)
-            if (node + j * NN < NTR)
+            if (node + j * NN < NTR && first)
 #pragma unroll
                 for (int c = 0; c < M; ++c) sE[node + j * NN][c] = sI[node + j * NN][c] = 0.0;
         for (int i = 0; i < P.s; ++i) {
@@ -1809,8 +1819,9 @@ __device__ __forceinline__ void final_body(const Params &P, const Bufs &B, int b
                         alpha = sps[(size_t)cell * (2 * DIM) + face];
                     } else {
                         alpha = fmax_nonneg(alpha, face_flux<PHYS, DIM>(P, ui, dir, true, f));
+                        if (first)
 #pragma unroll
-                        for (int c = 0; c < M; ++c) sI[fp][c] = fma(bi, f[c], sI[fp][c]);
+                            for (int c = 0; c < M; ++c) sI[fp][c] = fma(bi, f[c], sI[fp][c]);
                     }
                     if (nb >= 0) {
 #pragma unroll
@@ -1828,8 +1839,9 @@ __device__ __forceinline__ void final_body(const Params &P, const Bufs &B, int b
                     }
                     if (FROM == RECOMPUTED || nb < 0) {
                         alpha = fmax_nonneg(alpha, face_flux<PHYS, DIM>(P, ue, dir, true, f));
+                        if (first)
 #pragma unroll
-                        for (int c = 0; c < M; ++c) sE[fp][c] = fma(bi, f[c], sE[fp][c]);
+                            for (int c = 0; c < M; ++c) sE[fp][c] = fma(bi, f[c], sE[fp][c]);
                     }
                 }
                 __syncwarp();
@@ -1842,6 +1854,7 @@ __device__ __forceinline__ void final_body(const Params &P, const Bufs &B, int b
                 }
             }
         }
+        __syncwarp();  // the sums are complete
 #pragma unroll
         for (int j = 0; j < FPT; ++j) {
             const int fp = node + j * NN;
