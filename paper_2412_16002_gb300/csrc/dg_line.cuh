@@ -370,10 +370,13 @@ __global__ void __launch_bounds__(pc::LT, pc::Line<N>::BLOCKS) k_inner_l(const _
             float u[M][N], gl[M][N], tr[2][M];
             get_column<N>(S.buf, cl, R * h + j, u);
             line_G<N, 1>(rhy, gm1, ubf, u, density, 0.5f * wr[j], gl, tr, gsum);
+            // a column is read by its own thread and, in Q^2, by the two lanes that shadow the last one: they have
+            // read it before any of them writes
+            if constexpr (K::CPW * K::TPC < 32) __syncwarp();
 #pragma unroll
             for (int c = 0; c < M; ++c) {
 #pragma unroll
-                for (int b = 0; b < N; ++b) S.buf[c][cl][N * b + R * h + j] = gl[c][b];  // nobody else reads this column
+                for (int b = 0; b < N; ++b) S.buf[c][cl][N * b + R * h + j] = gl[c][b];
                 S.tr[c][cl][2 * N + R * h + j] = tr[0][c];
                 S.tr[c][cl][3 * N + R * h + j] = tr[1][c];
             }

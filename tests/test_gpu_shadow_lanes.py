@@ -56,3 +56,22 @@ def test_face_sums_on_every_lane(nx, ny, k):
                                    C.c_void_p(out.data_ptr()), C.c_void_p(torch.cuda.current_stream().cuda_stream))
     assert rc == L.OK
     assert torch.isfinite(out).all() and torch.equal(out, ref)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("k", [1, 2, 3])
+@pytest.mark.parametrize("thin", [False, True])
+def test_equal_cells_stay_equal(precision, k, thin):
+    """A periodic mesh of equal cells: after a step all cells have the same bits."""
+    from paper_2412_16002_gb300.solver import Solver
+
+    nx, ny = 29, 11
+    one = inputs.random_euler(2, 1, 1, k, seed=k, osc=0.2)
+    if thin:
+        one[0, 0, 0, 0, 0] *= 2.0 ** -24
+    U = np.ascontiguousarray(np.broadcast_to(one, (4, ny, nx, k + 1, k + 1)))
+    g = Solver(2, nx, ny, k, (0.0, 1.0, 0.0, 1.0 * ny / nx), "euler", precision=precision)
+    g.set_state(torch.from_numpy(U).cuda())
+    g.step(g.max_dt(0.05), "rk4")
+    V = g.get_state().reshape(4, ny * nx, -1)
+    assert np.isfinite(V).all() and np.array_equal(V, np.broadcast_to(V[:, :1], V.shape))
