@@ -411,29 +411,6 @@ MixBufs base_xbufs(const crkdg_ctx *h) {
     return X;
 }
 
-void fill_f32(Params &P) {
-    ParamsF &F = P.f;
-    F.rhx = (float)P.rhx;
-    F.rhy = (float)P.rhy;
-    F.gamma = (float)P.gamma;
-    F.gm1 = (float)(P.gamma - 1.0);
-    F.velx = (float)P.velx;
-    F.vely = (float)P.vely;
-    F.lo = (float)P.lo;
-    F.hi = (float)P.hi;
-    F.eps = (float)P.eps;
-    F.thr[0] = (float)P.thr[0];
-    F.thr[1] = (float)P.thr[1];
-    for (int s = 0; s < 4; ++s)
-        for (int c = 0; c < MAXM; ++c) F.bcs[s][c] = (float)P.bcs[s][c];
-    for (int i = 0; i < MAXS; ++i) {
-        for (int j = 0; j < MAXS; ++j) F.dtA[i][j] = (float)(P.dt * P.A[i][j]);
-        F.dtb[i] = (float)(P.dt * P.b[i]);
-        F.b[i] = (float)P.b[i];
-    }
-    F.dt = (float)P.dt;
-}
-
 bool euler_2d(const crkdg_ctx *h) { return h->dim == 2 && h->phys == PH_EULER; }
 
 // 2D Euler steps whose tableau has only a sub-diagonal (every tableau of the paper) run the inner

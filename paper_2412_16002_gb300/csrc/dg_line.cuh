@@ -72,7 +72,7 @@ __device__ __forceinline__ void line_G(float rh, float gm1, const float *ubf, co
     float f[M][N];
 #pragma unroll
     for (int a = 0; a < N; ++a) {
-        const float r = dens(u[0][a]), mx = ubf[1] + u[1][a], my = ubf[2] + u[2][a], E = ubf[3] + u[3][a];
+        const float r = dens(u[0][a], false), mx = ubf[1] + u[1][a], my = ubf[2] + u[2][a], E = ubf[3] + u[3][a];
         const float ri = recip_f(r), wx = mx * ri, wy = my * ri;
         const float p = gm1 * (E - 0.5f * (mx * wx + my * wy)), s = rh * (DIR ? wy : wx);
         f[0][a] = rh * (DIR ? my : mx);
@@ -100,7 +100,7 @@ __device__ __forceinline__ void line_G(float rh, float gm1, const float *ubf, co
             for (int a = 0; a < N; ++a) s = fmaf(l[a], u[c][a], s);
             d[c] = s;
         }
-        const float r = dens(d[0]), mx = ubf[1] + d[1], my = ubf[2] + d[2], E = ubf[3] + d[3];
+        const float r = dens(d[0], true), mx = ubf[1] + d[1], my = ubf[2] + d[2], E = ubf[3] + d[3];
         tr[e][0] = r, tr[e][1] = mx, tr[e][2] = my, tr[e][3] = E;
         const float ri = recip_f(r), wx = mx * ri, wy = my * ri;
         const float p = gm1 * (E - 0.5f * (mx * wx + my * wy)), s = rh * (DIR ? wy : wx);
@@ -335,12 +335,14 @@ __global__ void __launch_bounds__(pc::LT, pc::Line<N>::BLOCKS) k_inner_l(const _
         dmn = -cell_max<N>(-dmn, base);
         const float spread = 3.0f * (dmx - dmn);
         const bool thin = __any_sync(0xffffffffu, !(ubf[0] - spread > 9.5367431640625e-07f * (ubf[0] + spread)));
-        auto density = [&](float d) {
+        // at a trace, an S_K point, at least eps (a cell that the limiter left as it was has been tested with its
+        // mean taken off, which these values keep)
+        auto density = [&](float d, bool trace) {
             float r = ubf[0] + d;
             if (thin && rho_ill(r, ubf[0], d)) {
-                double ub[M];
-                average(ub);
-                r = (float)(ub[0] + (double)d);
+                const double u = active ? X.ub[cell] : 1.0;
+                r = (float)((i > 0 ? u + (double)(a_prev * gb[0]) : u) + (double)d);
+                if (trace) r = fmaxf(r, P.scr_eps);
             }
             return r;
         };
