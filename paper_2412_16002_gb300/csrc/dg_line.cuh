@@ -63,21 +63,25 @@ __device__ __forceinline__ float cell_max(float x, int base) {
                  __shfl_sync(0xffffffffu, x, base + 2));
 }
 
-// One line of a cell (direction DIR): u the deviations at its nodes, dens the density rule; g the line's
-// part of G (volume term and lifts), tr its end traces, gsum the face sums with weight wk.
+// One line of a cell (direction DIR): u the deviations at its nodes, thin whether a density of the warp may be
+// ill-conditioned, dens the density rule of a trace; g the line's part of G (volume term and lifts), tr
+// its end traces, gsum the face sums with weight wk.  A node with an ill-conditioned density takes
+// no part here (add_ill_nodes).
 template <int N, int DIR, class Density>
-__device__ __forceinline__ void line_G(float rh, float gm1, const float *ubf, const float (&u)[M][N], Density dens,
+__device__ __forceinline__ void line_G(float rh, float gm1, const float *ubf, const float (&u)[M][N], bool thin, Density dens,
                                        float wk, float (&g)[M][N], float (&tr)[2][M], float (&gsum)[M]) {
     const NodalTables &T = c_tab[N - 2];
     float f[M][N];
 #pragma unroll
     for (int a = 0; a < N; ++a) {
-        const float r = dens(u[0][a], false), mx = ubf[1] + u[1][a], my = ubf[2] + u[2][a], E = ubf[3] + u[3][a];
+        const float mx = ubf[1] + u[1][a], my = ubf[2] + u[2][a], E = ubf[3] + u[3][a];
+        float r = ubf[0] + u[0][a], k = rh;
+        if (thin && rho_ill(r, ubf[0], u[0][a])) r = 1.0f, k = 0.0f;
         const float ri = recip_f(r), wx = mx * ri, wy = my * ri;
-        const float p = gm1 * (E - 0.5f * (mx * wx + my * wy)), s = rh * (DIR ? wy : wx);
-        f[0][a] = rh * (DIR ? my : mx);
-        f[1][a] = DIR ? mx * s : fmaf(mx, s, rh * p);
-        f[2][a] = DIR ? fmaf(my, s, rh * p) : my * s;
+        const float p = gm1 * (E - 0.5f * (mx * wx + my * wy)), s = k * (DIR ? wy : wx);
+        f[0][a] = k * (DIR ? my : mx);
+        f[1][a] = DIR ? mx * s : fmaf(mx, s, k * p);
+        f[2][a] = DIR ? fmaf(my, s, k * p) : my * s;
         f[3][a] = (E + p) * s;
     }
 #pragma unroll
@@ -100,7 +104,7 @@ __device__ __forceinline__ void line_G(float rh, float gm1, const float *ubf, co
             for (int a = 0; a < N; ++a) s = fmaf(l[a], u[c][a], s);
             d[c] = s;
         }
-        const float r = dens(d[0], true), mx = ubf[1] + d[1], my = ubf[2] + d[2], E = ubf[3] + d[3];
+        const float r = dens(d[0]), mx = ubf[1] + d[1], my = ubf[2] + d[2], E = ubf[3] + d[3];
         tr[e][0] = r, tr[e][1] = mx, tr[e][2] = my, tr[e][3] = E;
         const float ri = recip_f(r), wx = mx * ri, wy = my * ri;
         const float p = gm1 * (E - 0.5f * (mx * wx + my * wy)), s = rh * (DIR ? wy : wx);
@@ -180,6 +184,36 @@ __device__ __forceinline__ void add_rows(const float (*buf)[Line<N>::CPB][Line<N
                 for (int a = 0; a < N; ++a) g[c][r][a] += p[a];
             }
         }
+}
+// The volume terms of this thread's nodes d with an ill-conditioned density (rho_ill), which line_G left out: the
+// flux in FP64 from ub + (double)d, rounded once, added to the node's row and column in the cell's part
+// of the buffer.  The cell's threads take turns (their columns cross); out of line: near vacuum only.
+template <int N>
+__device__ __noinline__ void add_ill_nodes(const Params &P, const double *ub, const float *ubf, const float (*d)[Line<N>::NV],
+                                           float (*buf)[Line<N>::CPB][Line<N>::LD], int cl, int h, bool first) {
+    using K = Line<N>;
+    const NodalTables &T = c_tab[N - 2];
+#pragma unroll 1
+    for (int k = 0; k < K::TPC; ++k) {
+        if (k == h && first) {
+#pragma unroll 1
+            for (int q = 0; q < K::NV; ++q) {
+                if (!rho_ill(ubf[0] + d[0][q], ubf[0], d[0][q])) continue;
+                float x[M], fx[M], fy[M];
+                for (int c = 0; c < M; ++c) x[c] = d[c][q];
+                flux_xy_fallback<2>(P, ub, x, fx, fy);
+                const int b = K::R * h + q / N, a = q % N;
+                for (int c = 0; c < M; ++c) {
+                    float *g = buf[c][cl];
+                    for (int j = 0; j < N; ++j) {
+                        g[N * b + j] = fmaf(T.Dhatf[j][a], P.f.rhx * fx[c], g[N * b + j]);
+                        g[N * j + a] = fmaf(T.Dhatf[j][b], P.f.rhy * fy[c], g[N * j + a]);
+                    }
+                }
+            }
+        }
+        __syncwarp();
+    }
 }
 // Consecutive values in global memory (16-byte accesses where rows are whole vectors).
 template <int K>
@@ -322,8 +356,8 @@ __global__ void __launch_bounds__(pc::LT, pc::Line<N>::BLOCKS) k_inner_l(const _
                 __syncwarp();
             }
         }
-        // near vacuum (rho_ill) a density is the rounded FP64 value; a uniform branch asks first
-        // whether any density of the warp's cells is that small: sum_a |l_a(+-1)| < 3, so a trace
+        // near vacuum (rho_ill) a trace's density is the rounded FP64 value and a node's flux is formed in
+        // FP64; a uniform branch asks first whether any density of the warp's cells is that small: sum_a |l_a(+-1)| < 3, so a trace
         // deviation is above 3 min - 3 max of the nodes'
         float dmx = 0.0f, dmn = 0.0f;
 #pragma unroll
@@ -335,14 +369,13 @@ __global__ void __launch_bounds__(pc::LT, pc::Line<N>::BLOCKS) k_inner_l(const _
         dmn = -cell_max<N>(-dmn, base);
         const float spread = 3.0f * (dmx - dmn);
         const bool thin = __any_sync(0xffffffffu, !(ubf[0] - spread > 9.5367431640625e-07f * (ubf[0] + spread)));
-        // at a trace, an S_K point, at least eps (a cell that the limiter left as it was has been tested with its
-        // mean taken off, which these values keep)
-        auto density = [&](float d, bool trace) {
+        // a trace's; an S_K point, so at least eps (a cell that the limiter left as it was has been tested
+        // with its mean taken off, which these values keep)
+        auto density = [&](float d) {
             float r = ubf[0] + d;
             if (thin && rho_ill(r, ubf[0], d)) {
                 const double u = active ? X.ub[cell] : 1.0;
-                r = (float)((i > 0 ? u + (double)(a_prev * gb[0]) : u) + (double)d);
-                if (trace) r = fmaxf(r, P.scr_eps);
+                r = fmaxf((float)((i > 0 ? u + (double)(a_prev * gb[0]) : u) + (double)d), P.scr_eps);
             }
             return r;
         };
@@ -358,7 +391,7 @@ __global__ void __launch_bounds__(pc::LT, pc::Line<N>::BLOCKS) k_inner_l(const _
             for (int c = 0; c < M; ++c)
 #pragma unroll
                 for (int a = 0; a < N; ++a) u[c][a] = dv[c][r][a];
-            line_G<N, 0>(rhx, gm1, ubf, u, density, 0.5f * wr[r], gl, tr, gsum);
+            line_G<N, 0>(rhx, gm1, ubf, u, thin, density, 0.5f * wr[r], gl, tr, gsum);
 #pragma unroll
             for (int c = 0; c < M; ++c) {
 #pragma unroll
@@ -371,7 +404,7 @@ __global__ void __launch_bounds__(pc::LT, pc::Line<N>::BLOCKS) k_inner_l(const _
         for (int j = 0; j < R; ++j) {
             float u[M][N], gl[M][N], tr[2][M];
             get_column<N>(S.buf, cl, R * h + j, u);
-            line_G<N, 1>(rhy, gm1, ubf, u, density, 0.5f * wr[j], gl, tr, gsum);
+            line_G<N, 1>(rhy, gm1, ubf, u, thin, density, 0.5f * wr[j], gl, tr, gsum);
             // a column is read by its own thread and, in Q^2, by the two lanes that shadow the last one: they have
             // read it before any of them writes
             if constexpr (K::CPW * K::TPC < 32) __syncwarp();
@@ -384,6 +417,24 @@ __global__ void __launch_bounds__(pc::LT, pc::Line<N>::BLOCKS) k_inner_l(const _
             }
         }
         __syncwarp();
+        if (thin) {
+            bool ill = false;
+#pragma unroll
+            for (int q = 0; q < NV; ++q)
+                ill = ill || rho_ill(ubf[0] + dv[0][q / N][q % N], ubf[0], dv[0][q / N][q % N]);
+            if (__any_sync(0xffffffffu, ill)) {
+                double ub[M];
+                float d[M][NV], uf[M];
+                average(ub);
+#pragma unroll
+                for (int c = 0; c < M; ++c) {
+                    uf[c] = ubf[c];
+#pragma unroll
+                    for (int q = 0; q < NV; ++q) d[c][q] = dv[c][q / N][q % N];
+                }
+                add_ill_nodes<N>(P, ub, uf, d, S.buf, cl, h, (t & 31) < K::CPW * K::TPC);
+            }
+        }
         add_rows<N>(S.buf, cl, h, g);
         if (slot >= 0) {
 #pragma unroll

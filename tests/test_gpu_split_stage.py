@@ -123,3 +123,51 @@ def test_limited_traces_are_in_bounds(stages, k, nx, ny):
     assert flag == 0 and limited > 0.9 * nx * ny and np.isfinite(tr).all()
     assert rho.min() >= np.float32(eps)
     assert not ((rho > 0) & (rho < 1.01 * eps)).any()
+
+
+def _line(n):
+    """Dhat, the end values of the basis and the Gauss weights on [-1, 1]."""
+    x, w = np.polynomial.legendre.leggauss(n)
+    inv = np.linalg.inv(np.polynomial.legendre.legvander(x, n - 1))
+    at = lambda y: np.polynomial.legendre.legvander(np.array([y]), n - 1)[0] @ inv  # noqa: E731
+    der = np.stack([np.polynomial.legendre.legval(x, np.polynomial.legendre.legder(np.eye(n)[j])) for j in range(n)], 1) @ inv
+    return der.T * w[None, :] / w[:, None], at(-1.0), at(1.0), w
+
+
+def _flux(u, d):
+    w = u[1 + d] / u[0]
+    p = 0.4 * (u[3] - 0.5 * (u[1] ** 2 + u[2] ** 2) / u[0])
+    return np.stack([u[1 + d], u[1] * w + (p if d == 0 else 0), u[2] * w + (p if d == 1 else 0), (u[3] + p) * w])
+
+
+@pytest.mark.parametrize("k,node", [(2, 4), (3, 5), (3, 10)])
+def test_flux_of_an_ill_conditioned_node(stages, k, node):
+    """A node with density 2^-30 and momentum 2^-16 beside averages of about 1: its flux is that of the FP64 state, so
+    u* is within 64 roundings of 2^-24 of the terms' magnitudes of the FP64 evaluation (2 n + 4 products, n^2 terms
+    of the mean, and the well-conditioned fluxes' own roundings); an FP32 momentum there is wrong by 2^-9."""
+    n, ncell, rh = k + 1, 300, (2.0, 3.0)
+    rng = np.random.default_rng(node)
+    dv = 0.1 * rng.normal(size=(4, ncell, n * n))
+    dv[0] = 0.6 + 0.05 * rng.normal(size=dv[0].shape)
+    dv = dv.astype(np.float32)
+    dv[:3, :, node] = -rng.uniform(0.5, 0.99, (3, ncell)).astype(np.float32)
+    ub = np.empty((4, ncell))
+    ub[0] = -dv[0, :, node].astype(np.float64) + 2.0 ** -30 * rng.uniform(1.0, 2.0, ncell)
+    ub[1:3] = -dv[1:3, :, node].astype(np.float64) + 2.0 ** -16 * rng.uniform(0.5, 1.0, (2, ncell))
+    ub[3] = rng.uniform(2.0, 3.0, ncell)
+    got, _, _, _ = stages(k, 60, 5, "euler1", 1.0, rh, 1e-13, ub, dv)
+    D, lm, lp, w = _line(n)
+    u = (ub[..., None] + dv).reshape(4, ncell, n, n)  # [b][a]
+    G, S = np.zeros_like(u), np.zeros_like(u)
+    for d in range(2):
+        at = (lambda M, v: v @ M.T) if d == 0 else (lambda M, v: np.moveaxis(np.moveaxis(v, -2, -1) @ M.T, -1, -2))
+        ends = (lambda l: u @ l) if d == 0 else (lambda l: np.moveaxis(u, -2, -1) @ l)
+        spread = (lambda f, l: f[..., None] * l) if d == 0 else (lambda f, l: f[..., None, :] * l[:, None])
+        f, fm, fp = _flux(u, d), _flux(ends(lm), d), _flux(ends(lp), d)
+        G += rh[d] * (at(D, f) + spread(fm, lm / w) - spread(fp, lp / w))
+        S += rh[d] * (at(np.abs(D), np.abs(f)) + spread(np.abs(fm), np.abs(lm / w)) + spread(np.abs(fp), np.abs(lp / w)))
+    w2 = np.outer(w, w) / 4
+    mean = lambda v: (v * w2).sum((-1, -2), keepdims=True)  # noqa: E731
+    ref = dv + (G - mean(G)).reshape(dv.shape)
+    tol = 64 * 2.0 ** -24 * (np.abs(dv) + (S + mean(S)).reshape(dv.shape))
+    assert np.isfinite(got).all() and (np.abs(got - ref) <= tol).all()
