@@ -66,7 +66,7 @@ __device__ __forceinline__ float cell_max(float x, int base) {
 // One line of a cell (direction DIR): u the deviations at its nodes, thin whether a density of the warp may be
 // ill-conditioned, dens the density rule of a trace; g the line's part of G (volume term and lifts), tr
 // its end traces, gsum the face sums with weight wk.  A node with an ill-conditioned density takes
-// no part here (add_ill_nodes).
+// no part here (ill_nodes).
 template <int N, int DIR, class Density>
 __device__ __forceinline__ void line_G(float rh, float gm1, const float *ubf, const float (&u)[M][N], bool thin, Density dens,
                                        float wk, float (&g)[M][N], float (&tr)[2][M], float (&gsum)[M]) {
@@ -185,35 +185,32 @@ __device__ __forceinline__ void add_rows(const float (*buf)[Line<N>::CPB][Line<N
             }
         }
 }
-// The volume terms of this thread's nodes d with an ill-conditioned density (rho_ill), which line_G left out: the
-// flux in FP64 from ub + (double)d, rounded once, added to the node's row and column in the cell's part
-// of the buffer.  The cell's threads take turns (their columns cross); out of line: near vacuum only.
+// The volume terms of a cell's nodes with an ill-conditioned density (rho_ill), which line_G leaves out: the flux
+// in FP64 from ub + (double)d, rounded once, d the node values in the cell's part of the buffer.  The sums over
+// such nodes go to out[c * stride + node], the cell's place in the array that u* is written to at the end.
+// By one thread of the cell and out of line: near vacuum only.
 template <int N>
-__device__ __noinline__ void add_ill_nodes(const Params &P, const double *ub, const float *ubf, const float (*d)[Line<N>::NV],
-                                           float (*buf)[Line<N>::CPB][Line<N>::LD], int cl, int h, bool first) {
-    using K = Line<N>;
+__device__ __noinline__ void ill_nodes(const Params &P, const double *ub, const float *ubf,
+                                       const float (*buf)[Line<N>::CPB][Line<N>::LD], int cl, float *out, size_t stride) {
     const NodalTables &T = c_tab[N - 2];
+    float g[M][N * N];
+    for (int c = 0; c < M; ++c)
+        for (int q = 0; q < N * N; ++q) g[c][q] = 0.0f;
 #pragma unroll 1
-    for (int k = 0; k < K::TPC; ++k) {
-        if (k == h && first) {
-#pragma unroll 1
-            for (int q = 0; q < K::NV; ++q) {
-                if (!rho_ill(ubf[0] + d[0][q], ubf[0], d[0][q])) continue;
-                float x[M], fx[M], fy[M];
-                for (int c = 0; c < M; ++c) x[c] = d[c][q];
-                flux_xy_fallback<2>(P, ub, x, fx, fy);
-                const int b = K::R * h + q / N, a = q % N;
-                for (int c = 0; c < M; ++c) {
-                    float *g = buf[c][cl];
-                    for (int j = 0; j < N; ++j) {
-                        g[N * b + j] = fmaf(T.Dhatf[j][a], P.f.rhx * fx[c], g[N * b + j]);
-                        g[N * j + a] = fmaf(T.Dhatf[j][b], P.f.rhy * fy[c], g[N * j + a]);
-                    }
-                }
+    for (int q = 0; q < N * N; ++q) {
+        float x[M], fx[M], fy[M];
+        for (int c = 0; c < M; ++c) x[c] = buf[c][cl][q];
+        if (!rho_ill(ubf[0] + x[0], ubf[0], x[0])) continue;
+        flux_xy_fallback<2>(P, ub, x, fx, fy);
+        const int b = q / N, a = q - b * N;
+        for (int c = 0; c < M; ++c)
+            for (int j = 0; j < N; ++j) {
+                g[c][N * b + j] = fmaf(T.Dhatf[j][a], P.f.rhx * fx[c], g[c][N * b + j]);
+                g[c][N * j + a] = fmaf(T.Dhatf[j][b], P.f.rhy * fy[c], g[c][N * j + a]);
             }
-        }
-        __syncwarp();
     }
+    for (int c = 0; c < M; ++c)
+        for (int q = 0; q < N * N; ++q) out[c * stride + q] = g[c][q];
 }
 // Consecutive values in global memory (16-byte accesses where rows are whole vectors).
 template <int K>
@@ -379,6 +376,23 @@ __global__ void __launch_bounds__(pc::LT, pc::Line<N>::BLOCKS) k_inner_l(const _
             }
             return r;
         };
+        bool ill = false;  // a node of this cell is
+        if (thin) {
+#pragma unroll
+            for (int q = 0; q < NV; ++q)
+                ill = ill || rho_ill(ubf[0] + dv[0][q / N][q % N], ubf[0], dv[0][q / N][q % N]);
+            const unsigned any = __ballot_sync(0xffffffffu, ill);
+            ill = active && ((any >> base) & ((1u << K::TPC) - 1u)) != 0u;
+            if (ill && h == 0) {
+                double ub[M];
+                float uf[M];
+                average(ub);
+#pragma unroll
+                for (int c = 0; c < M; ++c) uf[c] = ubf[c];
+                ill_nodes<N>(P, ub, uf, S.buf, cl, X.dv_s + (size_t)cell * (N * N), cs * (N * N));
+            }
+            __syncwarp();
+        }
         // ---- lines: rows in registers, columns from (and their part of G back to) the buffer
         const int slot = P.slot[i];
         float g[M][R][N], gsum[M];
@@ -417,24 +431,11 @@ __global__ void __launch_bounds__(pc::LT, pc::Line<N>::BLOCKS) k_inner_l(const _
             }
         }
         __syncwarp();
-        if (thin) {
-            bool ill = false;
+        if (ill)
 #pragma unroll
-            for (int q = 0; q < NV; ++q)
-                ill = ill || rho_ill(ubf[0] + dv[0][q / N][q % N], ubf[0], dv[0][q / N][q % N]);
-            if (__any_sync(0xffffffffu, ill)) {
-                double ub[M];
-                float d[M][NV], uf[M];
-                average(ub);
+            for (int c = 0; c < M; ++c)
 #pragma unroll
-                for (int c = 0; c < M; ++c) {
-                    uf[c] = ubf[c];
-#pragma unroll
-                    for (int q = 0; q < NV; ++q) d[c][q] = dv[c][q / N][q % N];
-                }
-                add_ill_nodes<N>(P, ub, uf, d, S.buf, cl, h, (t & 31) < K::CPW * K::TPC);
-            }
-        }
+                for (int q = 0; q < NV; ++q) g[c][q / N][q % N] += X.dv_s[(c * cs + cell) * (N * N) + NV * h + q];
         add_rows<N>(S.buf, cl, h, g);
         if (slot >= 0) {
 #pragma unroll
