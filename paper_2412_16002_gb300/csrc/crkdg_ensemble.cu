@@ -54,12 +54,13 @@ struct crkdg_ensemble_ctx {
     long long total_cells = 0;
     bool harvest = false;
     // work items: [group n=3,4][0 cell blocks, 1 feature blocks]
+    int inner_kind = ENS_INNER;  // or ENS_INNER_64
     int final_kind = ENS_FINAL;  // or ENS_FINAL_BARE
     EnsItem *ditems[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
     int nitems[2][2] = {{0, 0}, {0, 0}};
     int cap_items[2][2] = {{0, 0}, {0, 0}};
     int tile[NCLASS] = {4, 4, 4, 4, 4, 4};
-    int occ[2][5] = {};  // resident blocks per SM, [group][kind]
+    int occ[2][ENS_KINDS] = {};  // resident blocks per SM, [group][kind]
     cudaGraphExec_t g_step = nullptr, g_attempt = nullptr;
     bool graphs_valid = false;
     bool prof = false;
@@ -143,7 +144,7 @@ crkdg_status enqueue_attempt(crkdg_ens_t e) {
         }
         return cudaSuccess;
     };
-    ECK(e, run(ENS_INNER, 0));
+    ECK(e, run(e->inner_kind, 0));
     ECK(e, run(e->final_kind, 0));
     const int ind = e->opt.indicator;
     if (ind != CRKDG_IND_OFF) {
@@ -355,8 +356,9 @@ crkdg_status crkdg_ensemble_create(int count, const crkdg_ens_problem *problems,
                                                   cudaSuccess)
         return bail(CRKDG_E_CUDA);
     if (cudaStreamCreateWithFlags(&e->st, cudaStreamNonBlocking) != cudaSuccess) return bail(CRKDG_E_CUDA);
+    if (!(flux->gamma < 2.0)) e->inner_kind = ENS_INNER_64;
     for (int g = 0; g < 2; ++g)
-        for (int kind = 0; kind < 5; ++kind) e->occ[g][kind] = crkdg_ens_occupancy(kind, g + 3);
+        for (int kind = 0; kind < ENS_KINDS; ++kind) e->occ[g][kind] = crkdg_ens_occupancy(kind, g + 3);
     NodalTables tab[3];
     crkdg_build_tables(tab);
     if (crkdg_upload_tables_2d(tab) != cudaSuccess || crkdg_upload_tables_ens(tab) != cudaSuccess)
@@ -669,7 +671,7 @@ crkdg_status crkdg_ensemble_autotune(crkdg_ens_t e, int reps, int chosen[6]) {
                 if (err == cudaSuccess) err = cudaEventRecord(ev0, e->st);
                 const int cnt = e->nitems[g][0];
                 if (err == cudaSuccess)
-                    err = crkdg_ens_launch(ENS_INNER, g + 3, grid_of(e, ENS_INNER, g + 3, cnt), e->st, e->dprob,
+                    err = crkdg_ens_launch(e->inner_kind, g + 3, grid_of(e, e->inner_kind, g + 3, cnt), e->st, e->dprob,
                                            e->ditems[g][0], cnt, e->dctl, 0, 0);
                 if (err == cudaSuccess)
                     err = crkdg_ens_launch(e->final_kind, g + 3, grid_of(e, e->final_kind, g + 3, cnt), e->st, e->dprob,

@@ -1056,6 +1056,38 @@ __device__ __noinline__ void eval_G_slow(const Params &P, Smem<C> &S, int lc, in
     eval_G<C>(P, S, lc, node, u, g, trs, want_speed);
 }
 
+// The same with eval_G_fx's results, for the cells with `mine`.
+template <class C, class Put, class Fn>
+__device__ __forceinline__ void eval_G_64(const Params &P, Smem<C> &S, int lc, int node, const double *u, double *g,
+                                          bool mine, bool want_speed, bool want_avg, Put put, Fn avg) {
+    constexpr int M = C::M, NN = C::NN, NF = C::NF, NTR = C::NTR, FPT = C::FPT;
+    CellData<C> &D = S.c[lc];
+    double uu[M], gg[M], tt[FPT][M];
+#pragma unroll
+    for (int c = 0; c < M; ++c) uu[c] = u[c];
+    eval_G_slow<C>(P, S, lc, node, uu, gg, tt, want_speed);
+    cell_sync<C>();
+    if (mine) {
+#pragma unroll
+        for (int c = 0; c < M; ++c) g[c] = gg[c];
+#pragma unroll
+        for (int j = 0; j < FPT; ++j) {
+            const int fp = node + j * NN;
+            if ((j + 1) * NN <= NTR || fp < NTR) {
+                double sp = 0.0;
+                if (want_speed)
+                    for (int q = 0; q < NF; ++q) sp = fmax_nonneg(sp, D.ts[fp / NF * NF + q]);
+                put(j, tt[j], D.tf[fp], sp);
+            }
+        }
+    }
+    if (want_avg)
+        cell_averages<C>(D.u, node, [&](int c, double v) {
+            if (mine) avg(c, v);
+        });
+    cell_sync<C>();
+}
+
 // Fixed-point coefficients and the tableau's products with dt, in shared memory.
 template <class C>
 struct alignas(16) BlockTab {
@@ -1383,32 +1415,7 @@ __device__ __forceinline__ void eval_G_fx(const Params &P, Smem<C> &S, const Blo
             g[c] = fx_double(fx_sum(s), fx_shift(E, P.fx.k));
         }
     }
-    if (any_bad) {
-        double uu[M], gg[M], tt[FPT][M];
-#pragma unroll
-        for (int c = 0; c < M; ++c) uu[c] = u[c];
-        eval_G_slow<C>(P, S, lc, node, uu, gg, tt, want_speed);
-        cell_sync<C>();
-        if (mine) {
-#pragma unroll
-            for (int c = 0; c < M; ++c) g[c] = gg[c];
-#pragma unroll
-            for (int j = 0; j < FPT; ++j) {
-                const int fp = node + j * NN;
-                if (is_point(j)) {
-                    double sp = 0.0;
-                    if (want_speed)
-                        for (int q = 0; q < NF; ++q) sp = fmax_nonneg(sp, D.ts[fp / NF * NF + q]);
-                    put(j, tt[j], D.tf[fp], sp);
-                }
-            }
-        }
-        if (want_avg)
-            cell_averages<C>(D.u, node, [&](int c, double v) {
-                if (mine) avg(c, v);
-            });
-        cell_sync<C>();
-    }
+    if (any_bad) eval_G_64<C>(P, S, lc, node, u, g, mine, want_speed, want_avg, put, avg);
 }
 
 // ----------------------------------------------------------------------------- kernels
@@ -1524,7 +1531,10 @@ __device__ __forceinline__ void add_source(const Params &P, int cell, int node, 
     }
 }
 
-template <int DIM, int N, int PHYS>
+// FX: eval_G_fx; without it the FP64 form alone, for Euler problems out of the fixed-point range (gamma >= 2, cell
+// sizes beyond 2^100), where eval_G_fx would evaluate both (1024^2 Q^2 with gamma = 2.2, 3 Heun steps:
+// 48.0 -> 41.3 ms).  A kernel of its own: a branch inside took 2.5 to 6% of the other problems' time.
+template <int DIM, int N, int PHYS, bool FX = true>
 __device__ __forceinline__ void inner_body(const Params &P, const Bufs &B, int blk) {
     using C = CfgW<DIM, N, PHYS>;
     constexpr int M = C::M, NN = C::NN, NTR = C::NTR;
@@ -1577,23 +1587,25 @@ __device__ __forceinline__ void inner_body(const Params &P, const Bufs &B, int b
         const bool traced = slot >= 0 && active;
         const bool keep_faces = slot >= 0 && B.tsum != nullptr;
         double *dst = B.tr + (size_t)max(slot, 0) * M * P.ncell * NTR;
-        eval_G_fx<C>(
-            P, S, Tb, lc, node, cur, g, keep_faces, slot >= 0,
-            [&](int j, const double *t, const double *f, double sp) {
-                if (traced)
+        auto put = [&](int j, const double *t, const double *f, double sp) {
+            if (traced)
 #pragma unroll
-                    for (int c = 0; c < M; ++c) dst[at + j * NN + c * cstr] = t[c];
-                if (keep_faces) {
+                for (int c = 0; c < M; ++c) dst[at + j * NN + c * cstr] = t[c];
+            if (keep_faces) {
 #pragma unroll
-                    for (int c = 0; c < M; ++c) fs[j][c] = fma(P.b[i], f[c], fs[j][c]);
-                    const int fp = node + j * NN;
-                    if (active && fp % C::NF == 0)
-                        B.tsp[((size_t)slot * P.ncell + cell) * (2 * DIM) + fp / C::NF] = sp;
-                }
-            },
-            [&](int c, double v) {
-                if (active) B.tavg[((size_t)slot * M + c) * P.ncell + cell] = v;  // outflow exterior state
-            });
+                for (int c = 0; c < M; ++c) fs[j][c] = fma(P.b[i], f[c], fs[j][c]);
+                const int fp = node + j * NN;
+                if (active && fp % C::NF == 0)
+                    B.tsp[((size_t)slot * P.ncell + cell) * (2 * DIM) + fp / C::NF] = sp;
+            }
+        };
+        auto avg = [&](int c, double v) {
+            if (active) B.tavg[((size_t)slot * M + c) * P.ncell + cell] = v;  // outflow exterior state
+        };
+        if constexpr (FX)
+            eval_G_fx<C>(P, S, Tb, lc, node, cur, g, keep_faces, slot >= 0, put, avg);
+        else
+            eval_G_64<C>(P, S, lc, node, cur, g, true, keep_faces, slot >= 0, put, avg);
         if (P.source && active) add_source<DIM, N, PHYS>(P, cell, node, i, g);
         if (!sub)
 #pragma unroll
@@ -1619,9 +1631,9 @@ __device__ __forceinline__ void inner_body(const Params &P, const Bufs &B, int b
     store_node<DIM, N, PHYS>(P, B.ustar, cell, node, active, acc);
 }
 
-template <int DIM, int N, int PHYS>
+template <int DIM, int N, int PHYS, bool FX>
 __global__ void __launch_bounds__(kWarpThreads, 4) k_inner(const __grid_constant__ Params P, const __grid_constant__ Bufs B) {
-    inner_body<DIM, N, PHYS>(P, B, blockIdx.x);
+    inner_body<DIM, N, PHYS, FX>(P, B, blockIdx.x);
 }
 
 // u += dt lift(dc) at this thread's node, dc the corrections of this thread's face points (a cell
@@ -2361,7 +2373,12 @@ cudaError_t launch_one(int kernel, cudaStream_t st, const Params &P, const Bufs 
     using C = CfgW<DIM, N, PHYS>;
     const int nblocks = (P.ncell + C::NCB - 1) / C::NCB;
     switch (kernel) {
-    case K_INNER: k_inner<DIM, N, PHYS><<<nblocks, C::NT, 0, st>>>(P, B); break;
+    case K_INNER:
+        if (PHYS != PH_EULER || P.fx.on)  // scalar laws out of the range: eval_G_fx's own fallback
+            k_inner<DIM, N, PHYS, true><<<nblocks, C::NT, 0, st>>>(P, B);
+        else
+            k_inner<DIM, N, PHYS, PHYS != PH_EULER><<<nblocks, C::NT, 0, st>>>(P, B);
+        break;
     case K_FINAL:
         if (!B.tsum) {
             k_final<DIM, N, PHYS, RECOMPUTED><<<nblocks, C::NT, 0, st>>>(P, B);

@@ -15,6 +15,7 @@ cudaError_t crkdg_ens_launch(int kind, int n, int grid, cudaStream_t st, EnsProb
     CRKDG_ENS_CASE(3, ENS_FEATURES) CRKDG_ENS_CASE(4, ENS_INNER) CRKDG_ENS_CASE(4, ENS_FINAL)
     CRKDG_ENS_CASE(4, ENS_TROUBLE) CRKDG_ENS_CASE(4, ENS_FEATURES)
     CRKDG_ENS_CASE(3, ENS_FINAL_BARE) CRKDG_ENS_CASE(4, ENS_FINAL_BARE)
+    CRKDG_ENS_CASE(3, ENS_INNER_64) CRKDG_ENS_CASE(4, ENS_INNER_64)
 #undef CRKDG_ENS_CASE
     return cudaErrorInvalidValue;
 }
@@ -26,6 +27,7 @@ int crkdg_ens_occupancy(int kind, int n) {
     CRKDG_ENS_OCC(3, ENS_FEATURES) CRKDG_ENS_OCC(4, ENS_INNER) CRKDG_ENS_OCC(4, ENS_FINAL)
     CRKDG_ENS_OCC(4, ENS_TROUBLE) CRKDG_ENS_OCC(4, ENS_FEATURES)
     CRKDG_ENS_OCC(3, ENS_FINAL_BARE) CRKDG_ENS_OCC(4, ENS_FINAL_BARE)
+    CRKDG_ENS_OCC(3, ENS_INNER_64) CRKDG_ENS_OCC(4, ENS_INNER_64)
 #undef CRKDG_ENS_OCC
     return 0;
 }

@@ -44,6 +44,8 @@ template <int N, int KIND>
 __device__ __forceinline__ void ens_body(const Params &P, const Bufs &B, int blk) {
     if constexpr (KIND == ENS_INNER) {
         inner_body<2, N, PH_EULER>(P, B, blk);
+    } else if constexpr (KIND == ENS_INNER_64) {
+        inner_body<2, N, PH_EULER, false>(P, B, blk);
     } else if constexpr (KIND == ENS_FINAL) {
         final_body<2, N, PH_EULER, STORED>(P, B, blk);
     } else if constexpr (KIND == ENS_FINAL_BARE) {

@@ -76,7 +76,8 @@ __device__ bool grid_barrier(RunCtl *R, unsigned target, const RunSlot *SL, Slot
 // final stage combines jumps of the weighted flux sums: of the FP64 instructions of a step, each 64 to
 // 76 cycles behind the one before it, about a quarter is left (4096 cells of the blast tube 20.2 -> 18.9 us a
 // step, where the blocks at the front wait for the limiter's FP64 form; Burgers, 200 cells, 7.7 -> 7.4).
-template <int N, int PHYS>
+// FX as in inner_body.
+template <int N, int PHYS, bool FX>
 __global__ void __launch_bounds__(RunCfg1D<N, PHYS>::NT) k_run1d(const __grid_constant__ Params P, double *U0, double *U1,
                                                                  RunCtl *R, int cown) {
     using C = RunCfg1D<N, PHYS>;
@@ -154,18 +155,20 @@ __global__ void __launch_bounds__(RunCfg1D<N, PHYS>::NT) k_run1d(const __grid_co
                 }
                 const int q = P.slot[i];
                 double g[M];
-                eval_G_fx<C>(
-                    P, S, Tb, lc, node, cur_u, g, q >= 0, q >= 0,
-                    [&](int, const double *tr, const double *f, double sp) {  // one face point per thread
-                        if (q < 0) return;
+                auto put = [&](int, const double *tr, const double *f, double sp) {  // one face point per thread
+                    if (q < 0) return;
 #pragma unroll
-                        for (int c = 0; c < M; ++c) {
-                            sTr[q][lc][node][c] = tr[c];
-                            fs[c] = fma(P.b[i], f[c], fs[c]);
-                        }
-                        sSp[q][lc][node] = sp;
-                    },
-                    [&](int c, double v) { sAv[q][lc][c] = v; });
+                    for (int c = 0; c < M; ++c) {
+                        sTr[q][lc][node][c] = tr[c];
+                        fs[c] = fma(P.b[i], f[c], fs[c]);
+                    }
+                    sSp[q][lc][node] = sp;
+                };
+                auto avg = [&](int c, double v) { sAv[q][lc][c] = v; };
+                if constexpr (FX)
+                    eval_G_fx<C>(P, S, Tb, lc, node, cur_u, g, q >= 0, q >= 0, put, avg);
+                else
+                    eval_G_64<C>(P, S, lc, node, cur_u, g, true, q >= 0, q >= 0, put, avg);
 #pragma unroll
                 for (int c = 0; c < M; ++c) {
                     gh[i][c] = g[c];
@@ -271,12 +274,13 @@ cudaError_t run1d_launch(cudaStream_t st, const Params &P, double *u0, double *u
                          int *nblocks) {
     using C = RunCfg1D<N, PHYS>;
     constexpr int NCB = C::NCB;
+    auto *kernel = PHYS != PH_EULER || P.fx.on ? k_run1d<N, PHYS, true> : k_run1d<N, PHYS, PHYS != PH_EULER>;
     int dev = 0, nsm = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_run1d<N, PHYS>, C::NT, 0);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, C::NT, 0);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     // chunks of NCB - 2 own cells by default: smaller chunks put more blocks on the GPU but
@@ -290,7 +294,7 @@ cudaError_t run1d_launch(cudaStream_t st, const Params &P, double *u0, double *u
     *nblocks = grid;
     Params Pc = P;
     void *args[] = {&Pc, &u0, &u1, &R, &cown};
-    return cudaLaunchCooperativeKernel((void *)k_run1d<N, PHYS>, dim3(grid), dim3(C::NT), args, 0, st);
+    return cudaLaunchCooperativeKernel((void *)kernel, dim3(grid), dim3(C::NT), args, 0, st);
 }
 
 }  // namespace crkdg

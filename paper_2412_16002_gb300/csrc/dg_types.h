@@ -376,8 +376,9 @@ struct EnsItem {
 };
 
 enum { ENS_COUNTERS = 16 };
-// ENS_FINAL_BARE: the final stage of ensembles whose flux sums and radii do not fit (EnsProblem::stored)
-enum EnsKernelKind { ENS_INNER = 0, ENS_FINAL = 1, ENS_TROUBLE = 2, ENS_FEATURES = 3, ENS_FINAL_BARE = 4 };
+// ENS_FINAL_BARE: the final stage of ensembles whose flux sums and radii do not fit (EnsProblem::stored);
+// ENS_INNER_64: the inner stages of ensembles out of the fixed-point range (gamma >= 2)
+enum EnsKernelKind { ENS_INNER = 0, ENS_FINAL = 1, ENS_TROUBLE = 2, ENS_FEATURES = 3, ENS_FINAL_BARE = 4, ENS_INNER_64 = 5, ENS_KINDS = 6 };
 struct EnsCtl {
     unsigned int counter[ENS_COUNTERS];  // one work counter per persistent launch of an attempt
     int any_pending;
