@@ -235,6 +235,9 @@ __device__ __forceinline__ double flux_speed_dir(const Params &P, const double *
 // take: products of three such values and their differences stay far from overflow.  Small
 // momenta and energies need no bound; results below 2^-1022 become zero.
 constexpr int kFxExpLo = 1023 - 150, kFxExpHi = 1023 + 150;
+// Binades below a cell's largest value to which sums of values with its exponent (59 bits, six roundings of 2^-58)
+// are as accurate as FP64's (2^-53): the errors are 0.8 units at 3, 2.4 at 4, 6.1 at 5, FP64's 0.8 (Euler Q^2).
+constexpr int kFxKeep = 3;
 // an Euler state that fx_point takes
 template <int DIM>
 __device__ __forceinline__ bool fx_state(const double *u) {
@@ -1183,6 +1186,22 @@ __device__ __forceinline__ double face_max(double x, int node) {
     return bitsd(k);
 }
 
+// The smaller of the largest x over a node's row and over its column (2D).
+template <class C>
+__device__ __forceinline__ int line_max(int x, int node) {
+    constexpr int N = C::NP;
+    int l = threadIdx.x & 31;
+    if (l >= C::CPW * C::NN) l = C::CPW * C::NN - 1;
+    const int base = l - node, a = node % N;
+    int r = x, c = x;
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+        r = max(r, __shfl_sync(0xffffffffu, x, base + node - a + q));
+        c = max(c, __shfl_sync(0xffffffffu, x, base + q * N + a));
+    }
+    return min(r, c);
+}
+
 // Whether x holds for any thread of this thread's cell.
 template <class C>
 __device__ __forceinline__ bool cell_any(bool x, int node) {
@@ -1209,7 +1228,11 @@ __device__ __forceinline__ unsigned biased_exp(int x) { return (unsigned)max(x +
 // Near vacuum (a density at a node or a trace 2^-20 below the cell's largest, or not positive),
 // for an energy that is not positive and for values outside the exponent range the cell takes the
 // FP64 form: a rule of the cell's own values, so a cell's result does not depend on the cells it
-// shares a warp with.
+// shares a warp with.  So does a 2D cell in which a node's density or energy is 2^-3 below the largest (kFxKeep;
+// scalar laws: a row or a column of nodes): FP64 rounds a sum by its own row and column, which only in 1D always
+// hold the cell's largest value.  At nodes whose row and column are small the error of G, in units of 2^-53
+// of the magnitudes of a node's own terms, is the FP64 form's: 0.8 (Euler Q^2), 0.9 (Burgers Q^2) and 1.4
+// (advection Q^3); without the rule it grew with the contrast (at 2^-9 to 77, 4e3 and 17).
 //
 // Why: with FP64 maps and fluxes a warp issued about 145 FP64 instructions per Q^3 stage, 76 cycles
 // each; now about 30, with 2000 instructions on the other pipes beside them.  Set state, steps, get
@@ -1246,7 +1269,10 @@ __device__ __forceinline__ void eval_G_fx(const Params &P, Smem<C> &S, const Blo
 #pragma unroll
     for (int k = 0; k < W; ++k) eu[k] = cell_max_halves<C>(eu[k], node);
     if constexpr (PHYS == PH_EULER) {
-        if (!fx_state<DIM>(u) || e0 < field(eu, 0) - 20) bad = true;
+        if (!fx_state<DIM>(u) || e0 < field(eu, 0) - (DIM == 2 ? kFxKeep : 20)) bad = true;
+        if (DIM == 2 && fx_exp(u[M - 1]) < field(eu, M - 1) - kFxKeep) bad = true;
+    } else if constexpr (DIM == 2) {  // the flux of Burgers' law is a square
+        if (line_max<C>(e0, node) < field(eu, 0) - (PHYS == PH_BURG ? 2 : kFxKeep)) bad = true;
     }
     cell_sync<C>();  // earlier readers of the cell's arrays are done
 #pragma unroll
@@ -1638,14 +1664,17 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_inner(const __grid_constant
 
 // u += dt lift(dc) at this thread's node, dc the corrections of this thread's face points (a cell
 // collective): the four products per component in fixed point with one exponent per cell and
-// component (dg_fixed.h), as in eval_G_fx; corrections outside its range take the FP64 form.
+// component (dg_fixed.h), as in eval_G_fx; corrections outside its range take the FP64 form.  So do the cells
+// where a node's four corrections are all 2^-3 below the cell's largest, which FP64 would round by their own
+// size, unless what the largest can add is below the node's own value: then 2^-55 of it (six units of 2^-58)
+// does not reach the rounding of the result.
 template <class C>
 __device__ __forceinline__ void lift_faces(const Params &P, double dt, CellData<C> &D, int node, int a, int b,
                                            const double (&dc)[C::FPT][C::M], double *u) {
     constexpr int DIM = C::D, N = C::NP, M = C::M, NN = C::NN, NF = C::NF, NTR = C::NTR, FPT = C::FPT;
     constexpr int W = (M + 1) / 2;
     unsigned ef[W];
-    bool bad = P.fx.on == 0;
+    bool bad = false;
 #pragma unroll
     for (int k = 0; k < W; ++k) ef[k] = 0u;
 #pragma unroll
@@ -1659,30 +1688,6 @@ __device__ __forceinline__ void lift_faces(const Params &P, double dt, CellData<
                 e = max(e, ej);
             }
         ef[c >> 1] |= (unsigned)e << (16 * (c & 1));
-    }
-    double corr[M];
-    const bool any_bad = __any_sync(0xffffffffu, bad);
-    if (any_bad) {  // a cell of the warp takes the FP64 form instead
-        const NodalTables &T = c_tab[N - 2];
-#pragma unroll
-        for (int j = 0; j < FPT; ++j) {
-            const int fp = node + j * NN;
-            if (fp < NTR)
-#pragma unroll
-                for (int c = 0; c < M; ++c) D.tf[fp][c] = dc[j][c];
-        }
-        cell_sync<C>();
-#pragma unroll
-        for (int c = 0; c < M; ++c) {
-            double cx = -T.liftp[a] * D.tf[NF + b][c] + T.liftm[a] * D.tf[b][c];
-            corr[c] = P.rhx * cx;
-            if constexpr (DIM == 2) {
-                double cy = -T.liftp[b] * D.tf[3 * NF + a][c] + T.liftm[b] * D.tf[2 * NF + a][c];
-                corr[c] = fma(P.rhy, cy, corr[c]);
-            }
-        }
-        bad = cell_any<C>(bad, node);
-        cell_sync<C>();
     }
     Fx(&ft)[M][NTR] = reinterpret_cast<Fx(&)[M][NTR]>(D.tf);
 #pragma unroll
@@ -1698,19 +1703,54 @@ __device__ __forceinline__ void lift_faces(const Params &P, double dt, CellData<
     }
     const Fx x0 = P.fx.lx[a][0], x1 = P.fx.lx[a][1], y0 = P.fx.ly[b][0], y1 = P.fx.ly[b][1];
     cell_sync<C>();
+    double v[M];
+    const int reach = 58 - P.fx.k + fx_exp(dt) - 1023;  // exponent of dt times the sum of the coefficients
 #pragma unroll
     for (int c = 0; c < M; ++c) {
         const int E = (int)((ef[c >> 1] >> (16 * (c & 1))) & 0xffffu);
         FxSum s{0, 0};
-        fx_mac(s, ft[c][b], x0);
-        fx_mac(s, ft[c][NF + b], x1);
         if constexpr (DIM == 2) {
-            fx_mac(s, ft[c][2 * NF + a], y0);
-            fx_mac(s, ft[c][3 * NF + a], y1);
+            const Fx f[4] = {ft[c][b], ft[c][NF + b], ft[c][2 * NF + a], ft[c][3 * NF + a]};
+            fx_mac(s, f[0], x0);
+            fx_mac(s, f[1], x1);
+            fx_mac(s, f[2], y0);
+            fx_mac(s, f[3], y1);
+            int top = 0, any = 0;  // leading bits of the four: 2^(30 - j) for a value 2^-j of the largest
+#pragma unroll
+            for (int q = 0; q < 4; ++q) top |= f[q].h ^ (f[q].h >> 31), any |= f[q].h | f[q].l;
+            if (top >> (30 - kFxKeep) == 0 && any != 0 && E + reach >= fx_exp(u[c])) bad = true;
+        } else {
+            fx_mac(s, ft[c][b], x0);
+            fx_mac(s, ft[c][NF + b], x1);
         }
-        const double v = fx_double(fx_sum(s), fx_shift(E, P.fx.k));
-        u[c] = fma(dt, bad ? corr[c] : v, u[c]);
+        v[c] = fx_double(fx_sum(s), fx_shift(E, P.fx.k));
     }
+    if (P.fx.on == 0 || __any_sync(0xffffffffu, bad)) {
+        const NodalTables &T = c_tab[N - 2];
+        cell_sync<C>();  // the cell's corrections have been read
+#pragma unroll
+        for (int j = 0; j < FPT; ++j) {
+            const int fp = node + j * NN;
+            if (fp < NTR)
+#pragma unroll
+                for (int c = 0; c < M; ++c) D.tf[fp][c] = dc[j][c];
+        }
+        cell_sync<C>();
+        bad = cell_any<C>(bad || P.fx.on == 0, node);
+#pragma unroll
+        for (int c = 0; c < M; ++c) {
+            double cx = -T.liftp[a] * D.tf[NF + b][c] + T.liftm[a] * D.tf[b][c];
+            double w = P.rhx * cx;
+            if constexpr (DIM == 2) {
+                double cy = -T.liftp[b] * D.tf[3 * NF + a][c] + T.liftm[b] * D.tf[2 * NF + a][c];
+                w = fma(P.rhy, cy, w);
+            }
+            if (bad) v[c] = w;
+        }
+        cell_sync<C>();
+    }
+#pragma unroll
+    for (int c = 0; c < M; ++c) u[c] = fma(dt, v[c], u[c]);
 }
 
 // Corrections of the interior faces of a 2D mesh, one thread per face point (a cell's lower faces): for the
