@@ -220,7 +220,6 @@ void build_tables(NodalTables *tab) {
             }
         }
         for (int a = 0; a < n; ++a) {
-            T.pm1x[a] = fx_coef(T.pm1[a], kFxAvg);
             T.xgf[0][a] = (float)T.xg[a];
             T.xgf[1][a] = (float)(T.xg[a] - (double)T.xgf[0][a]);
         }

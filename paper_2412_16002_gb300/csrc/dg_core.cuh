@@ -2101,22 +2101,40 @@ __device__ __forceinline__ long long fx_whole(double x, int E) {
     const Fx f = fx_of(x, E);
     return ((long long)f.h << 28) + f.l;
 }
-// The plain indicator's decision of one direction and component: sR, sL the face averages in units of
-// 2^(En - 1081) (sums of node values with the weights scaled by 2^kFxTrace), own, lo, hi the averages of the
-// cell and its neighbours.  FP64 sums of the node values took 18 fused multiply-adds (76 cycles each) in Q^2:
-// 501 x 397 Q^2, troubled-cell pass 186 -> 110 us, features 247 -> 164 us.
-__device__ __forceinline__ bool tvb_pair(long long sR, long long sL, int En, double own, double lo, double hi,
-                                         double thr) {
+// The plain indicator's decision of one direction and component in fixed point: sR, sL the face averages in units
+// of 2^(En - 1081) (sums of node values with the weights scaled by 2^kFxTrace), own, lo, hi the averages of the
+// cell and its neighbours.  0 kept, 1 troubled, 2 left to FP64 (tvb_pair_64): infinities and NaN, a neighbour's
+// average 2^kFxKeep above the node values (whose units would then be too coarse), and a deviation and a threshold
+// that are both within FP64's own rounding (2^-52 of the largest value: constant cells without a
+// threshold).  FP64 sums of the node values took 18 fused multiply-adds (76 cycles each) in Q^2: 501 x
+// 397 Q^2, troubled-cell pass 186 -> 110 us, features 247 -> 164 us.
+__device__ __forceinline__ int tvb_pair(long long sR, long long sL, int En, double own, double lo, double hi,
+                                        double thr) {
     const int E = max(max(En, fx_exp(own)), max(fx_exp(lo), fx_exp(hi)));
-    if (E == 0x7ff) return true;  // infinities and NaN
-    const int sh = min(E - En, 63);
+    if (E == 0x7ff || E > En + kFxKeep) return 2;
+    const int sh = E - En;
     const long long o = fx_whole(own, E), l = fx_whole(lo, E), h = fx_whole(hi, E);
     const int et = fx_exp(thr);
     long long th = 1ll << 62;  // larger than every deviation
     if (!(thr >= 0.0)) th = -1;
     else if (et <= E) th = fx_whole(thr, E);
     else if (et <= E + 3) th = fx_whole(thr, et) << (et - E);
-    return tvb_changes_fx((sR >> sh) - o, h - o, o - l, th) || tvb_changes_fx(o - (sL >> sh), h - o, o - l, th);
+    const long long tR = (sR >> sh) - o, tL = o - (sL >> sh);
+    constexpr long long kNoise = 64;  // units of 2^-58
+    if (th < kNoise && ((tR < 0 ? -tR : tR) < kNoise || (tL < 0 ? -tL : tL) < kNoise)) return 2;
+    return tvb_changes_fx(tR, h - o, o - l, th) || tvb_changes_fx(tL, h - o, o - l, th) ? 1 : 0;
+}
+// The same in FP64 from the node values u of a component.  Out of line: rare.
+template <int DIM, int N>
+__device__ __noinline__ bool tvb_pair_64(const double *u, int d, double own, double lo, double hi, double thr) {
+    const NodalTables &T = c_tab[N - 2];
+    double fr = 0.0, fl = 0.0;
+    for (int q = 0; q < (DIM == 2 ? N * N : N); ++q) {
+        fr = fma(DIM == 2 ? T.trw2[d][0][q] : T.lp[q], u[q], fr);
+        fl = fma(DIM == 2 ? T.trw2[d][1][q] : T.lm[q], u[q], fl);
+    }
+    const double dp = hi - own, dm = own - lo;
+    return tvb_changes(fr - own, dp, dm, thr, thr >= 0.0) || tvb_changes(own - fl, dp, dm, thr, thr >= 0.0);
 }
 
 // 2^k, k in [-126, 127]
@@ -2205,10 +2223,11 @@ __device__ __forceinline__ void trouble_body(const Params &P, const Bufs &B, int
                 fx_mac(sr, v, wr[q]);
                 fx_mac(sl, v, wl[q]);
             }
-            if (tvb_pair(fx_sum(sr), fx_sum(sl), field(c), B.aux[(size_t)cell * M + c],
-                         nb_average<PHYS, DIM>(P, B.aux, cell, 2 * d, c),
-                         nb_average<PHYS, DIM>(P, B.aux, cell, 2 * d + 1, c), P.thr[d]))
-                atomicOr(&sTr[lc], 1);
+            const double own = B.aux[(size_t)cell * M + c], lo = nb_average<PHYS, DIM>(P, B.aux, cell, 2 * d, c),
+                         hi = nb_average<PHYS, DIM>(P, B.aux, cell, 2 * d + 1, c);
+            int t = tvb_pair(fx_sum(sr), fx_sum(sl), field(c), own, lo, hi, P.thr[d]);
+            if (t == 2) t = tvb_pair_64<DIM, N>(B.unew + ((size_t)c * P.ncell + cell) * NN, d, own, lo, hi, P.thr[d]);
+            if (t) atomicOr(&sTr[lc], 1);
         }
         cell_sync<C>();
     }
@@ -2220,13 +2239,12 @@ __device__ __forceinline__ void trouble_body(const Params &P, const Bufs &B, int
     if (__any_sync(0xffffffffu, troubled)) {  // the limited first moments, spread likewise
         for (int j = node; j < DIM * M && troubled; j += NN) {
             const int d = j / M, c = j - d * M;
-            const Fx *w = DIM == 2 ? T.pm2x[d] : T.pm1x;
-            FxSum s{0, 0};
+            const double *v = B.unew + ((size_t)c * P.ncell + cell) * NN;
+            double p1 = 0.0;  // FP64: a moment has no part of the nodes in the middle, which may be the largest
 #pragma unroll
-            for (int q = 0; q < NN; ++q) fx_mac(s, fu[c][q], w[q]);
+            for (int q = 0; q < NN; ++q) p1 = fma(DIM == 2 ? T.pm2[d][q] : T.pm1[q], v[q], p1);
             const double own = B.aux[(size_t)cell * M + c];
-            sP1[lc][d][c] = minmod3_bits(fx_double(fx_sum(s), fx_shift(field(c), kFxAvg)),
-                                         nb_average<PHYS, DIM>(P, B.aux, cell, 2 * d + 1, c) - own,
+            sP1[lc][d][c] = minmod3_bits(p1, nb_average<PHYS, DIM>(P, B.aux, cell, 2 * d + 1, c) - own,
                                          own - nb_average<PHYS, DIM>(P, B.aux, cell, 2 * d, c));
         }
         cell_sync<C>();
@@ -2390,8 +2408,10 @@ __device__ __forceinline__ void features_body(const Params &P, const Bufs &B, in
             for (int d = 0; d < 2; ++d) {
                 const double m = En == 0x7ff ? NAN : fx_double(fx_sum(s[d]), fx_shift(En, kFxAvg));
                 f[36 + 2 * c + d] = (float)(m * scale[c]);
-                if (tvb_pair(fx_sum(r[d]), fx_sum(l[d]), En, v[4][c], v[d == 0 ? 3 : 1][c], v[d == 0 ? 5 : 7][c], P.thr[d]))
-                    trouble = 1;
+                const double lo = v[d == 0 ? 3 : 1][c], hi = v[d == 0 ? 5 : 7][c];
+                int t = tvb_pair(fx_sum(r[d]), fx_sum(l[d]), En, v[4][c], lo, hi, P.thr[d]);
+                if (t == 2) t = tvb_pair_64<2, N>(u, d, v[4][c], lo, hi, P.thr[d]);
+                if (t) trouble = 1;
             }
         }
         if (B.tflags) B.tflags[cell] = trouble;

@@ -71,7 +71,7 @@ struct NodalTables {
     // fixed-point copies (dg_fixed.h): l_a(-1), l_a(+1) scaled by 2^kFxTrace, the average weights
     // by 2^kFxAvg
     Fx tlx[2][MAXN], w1x[MAXN], w2x[MAXN * MAXN];
-    Fx pm2x[2][MAXN * MAXN], pm1x[MAXN];  // pm2, pm1 scaled by 2^kFxAvg (their magnitudes sum to less than 2)
+    Fx pm2x[2][MAXN * MAXN];              // pm2 scaled by 2^kFxAvg (its magnitudes sum to less than 2)
     Fx trw2x[2][2][MAXN * MAXN];          // trw2 scaled by 2^kFxTrace (their magnitudes sum to less than 4)
     float xgf[2][MAXN];       // xg as a sum of two floats
 };
