@@ -781,7 +781,7 @@ __device__ bool limit_block(const Params &P, const Bufs &B, Smem<C> &S, int lc, 
             if (!screen_point<PHYS, DIM>(P, v, e)) unsafe = true;
             if (want_rate) {
                 const float r = rate_bound<PHYS, DIM>(P, v, e);
-                rhi = r <= rhi ? rhi : r;  // a NaN stays
+                rhi = fmaxf(rhi, r == r ? r : INFINITY);  // a bound that fails bounds nothing
             }
         }
     }
