@@ -51,6 +51,13 @@ struct NodalTables {
     double Dhat[MAXN][MAXN];    // Dhat[a][q] = w_q l_a'(x_q) / w_a  (volume term)
     double lm[MAXN], lp[MAXN];  // l_a(-1), l_a(+1)                 (traces)
     double liftm[MAXN], liftp[MAXN];  // l_a(-1)/w_a, l_a(+1)/w_a    (lift)
+// The 1D step loop: threads of a block, and cells of its chunk including the two halo cells.
+__host__ __device__ constexpr int run1d_threads(int n) { return n == 2 ? 64 : 128; }
+__host__ __device__ constexpr int run1d_cells(int n) { return (32 / n) * (run1d_threads(n) / 32); }
+
+// Device memory that an optional array leaves for what is allocated after it (work items, graphs, features).
+constexpr size_t kSpareBytes = (size_t)256 << 20;
+
     double Igl[MAXN][MAXN];     // Igl[alpha][a] = l_a(xl_alpha)   (S_K interpolation)
     double w1[MAXN];            // w_a / 2                          (1D average weights)
     double w2[MAXN * MAXN];     // (w_a/2)(w_b/2) at node b*n+a      (2D average weights)
