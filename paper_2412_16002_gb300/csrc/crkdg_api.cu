@@ -774,7 +774,7 @@ crkdg_status crkdg_set_tensor_cores(crkdg_t h, int on) {
 }
 
 crkdg_status crkdg_set_run1d_chunk(crkdg_t h, int cells) {
-    if (!h || cells < 0 || cells > 30) return CRKDG_E_ARG;
+    if (!h || cells < 0 || cells > run1d_cells(h->n) - 2) return CRKDG_E_ARG;
     h->run1d_chunk = cells;
     return CRKDG_OK;
 }

@@ -20,8 +20,8 @@ namespace crkdg {
 // step is one warp's chain of instructions.
 template <int N, int PHYS>
 struct RunCfg1D : CfgW<1, N, PHYS> {
-    static constexpr int NT = N == 2 ? 64 : 128;
-    static constexpr int NCB = (32 / N) * (NT / 32);  // cells per chunk including the two halo cells
+    static constexpr int NT = run1d_threads(N);
+    static constexpr int NCB = run1d_cells(N);  // cells per chunk including the two halo cells
 };
 
 __device__ __forceinline__ unsigned long long global_ns() {

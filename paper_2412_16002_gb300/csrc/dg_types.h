@@ -44,6 +44,10 @@ __host__ __device__ constexpr int cells_per_block(int dim, int n) {
 constexpr int kWarpThreads = 128;
 __host__ __device__ constexpr int warp_cells_per_block(int nn) { return (32 / nn) * (kWarpThreads / 32); }
 
+// The 1D step loop: threads of a block, and cells of its chunk including the two halo cells.
+__host__ __device__ constexpr int run1d_threads(int n) { return n == 2 ? 64 : 128; }
+__host__ __device__ constexpr int run1d_cells(int n) { return (32 / n) * (run1d_threads(n) / 32); }
+
 // One-dimensional nodal tables for n = k+1 Gauss points on [-1, 1].
 struct NodalTables {
     double xg[MAXN], wg[MAXN];  // Gauss--Legendre nodes / weights (sum 2)
