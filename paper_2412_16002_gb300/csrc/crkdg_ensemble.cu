@@ -401,9 +401,12 @@ crkdg_status crkdg_ensemble_create(int count, const crkdg_ens_problem *problems,
              alloc((void **)&e->arena_prob, sizeof(float) * (size_t)tot_cells) &&
              alloc((void **)&e->mlp, sizeof(float) * CRKDG_MLP_NPARAM);
     }
-    // last: where the flux sums and radii do not fit beside the traces, the final kernel recomputes them
-    bool stored = true;
-    if (ok && !alloc((void **)&e->arena_tr, tot_tr * 8)) {
+    // last: where the flux sums and radii do not fit beside the traces, with room for the work items and graphs
+    // that follow, the final kernel recomputes them
+    size_t free_bytes = 0, total = 0;
+    const size_t spare = kSpareBytes + sizeof(EnsItem) * ((size_t)tot_cells / 4 + 2 * (size_t)count);
+    bool stored = cudaMemGetInfo(&free_bytes, &total) == cudaSuccess && free_bytes >= tot_tr * 8 + spare;
+    if (ok && !(stored && alloc((void **)&e->arena_tr, tot_tr * 8))) {
         cudaGetLastError();
         stored = false;
         e->final_kind = ENS_FINAL_BARE;

@@ -48,6 +48,9 @@ __host__ __device__ constexpr int warp_cells_per_block(int nn) { return (32 / nn
 __host__ __device__ constexpr int run1d_threads(int n) { return n == 2 ? 64 : 128; }
 __host__ __device__ constexpr int run1d_cells(int n) { return (32 / n) * (run1d_threads(n) / 32); }
 
+// Device memory that an optional array leaves for what is allocated after it (work items, graphs, features).
+constexpr size_t kSpareBytes = (size_t)256 << 20;
+
 // One-dimensional nodal tables for n = k+1 Gauss points on [-1, 1].
 struct NodalTables {
     double xg[MAXN], wg[MAXN];  // Gauss--Legendre nodes / weights (sum 2)
