@@ -250,6 +250,7 @@ struct crkdg_ctx {
     cudaStream_t st = nullptr;
     double *u = nullptr, *unew = nullptr, *ustar = nullptr, *tr = nullptr, *aux = nullptr;
     int tr_slots = 0;
+    bool tr_fc = false;           // tr also holds the faces' corrections
     DevScal *scal = nullptr;
     DevScal *hs = nullptr;      // pinned readback
     DevScal *hinit = nullptr;   // pinned initial values
@@ -359,7 +360,7 @@ Bufs base_bufs(const crkdg_ctx *h) {
     B.tavg = h->tr ? h->tr + (size_t)h->tr_slots * h->m * h->ncell * h->ntr : nullptr;
     B.tsum = h->tr ? h->tr + (size_t)h->tr_slots * h->m * h->ncell * (h->ntr + 1) : nullptr;
     B.tsp = h->tr ? B.tsum + (size_t)h->m * h->ncell * h->ntr : nullptr;
-    B.fc = h->tr && h->dim == 2 ? B.tsp + (size_t)h->tr_slots * h->ncell * 4 : nullptr;
+    B.fc = h->tr && h->tr_fc ? B.tsp + (size_t)h->tr_slots * h->ncell * 4 : nullptr;
     B.flag = &h->scal->flag;
     B.nlim = &h->scal->nlim;
     B.thmin = &h->scal->thmin;
@@ -519,12 +520,22 @@ crkdg_status ensure_traces(crkdg_ctx *h, int slots) {
     h->tr = nullptr;
     h->tr_slots = 0;
     // traces [slot][m][cell][face point], the traced stages' cell averages [slot][m][cell], then
-    // the weighted sum of the traces' normal fluxes [m][cell][face point], each stage's
-    // largest radius per face [slot][cell][face], and in 2D the faces' corrections (Bufs::fc)
-    size_t bytes = ((size_t)slots * h->m * h->ncell * (h->ntr + 1) + (size_t)h->m * h->ncell * h->ntr +
-                    (size_t)slots * h->ncell * 2 * h->dim + (h->dim == 2 ? (size_t)h->m * h->ncell * h->ntr : 0)) *
-                   sizeof(double);
-    CK(h, cudaMalloc(&h->tr, bytes));
+    // the weighted sum of the traces' normal fluxes [m][cell][face point] and each stage's
+    // largest radius per face [slot][cell][face]; in 2D from faces_cells on also the faces' corrections
+    // (Bufs::fc), where they leave room for what a program allocates after them: without them the final
+    // stage forms the corrections itself
+    const size_t face_values = (size_t)h->m * h->ncell * h->ntr * sizeof(double);
+    const size_t base = slots * (face_values + (size_t)h->m * h->ncell * sizeof(double)) + face_values +
+                        (size_t)slots * h->ncell * 2 * h->dim * sizeof(double);
+    h->tr_fc = h->dim == 2 && h->ncell >= faces_cells(h->n);
+    size_t free_bytes = 0, total = 0;
+    if (h->tr_fc && (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess ||
+                     free_bytes < base + face_values + kSpareBytes || cudaMalloc(&h->tr, base + face_values) != cudaSuccess)) {
+        cudaGetLastError();
+        h->tr = nullptr;
+        h->tr_fc = false;
+    }
+    if (!h->tr) CK(h, cudaMalloc(&h->tr, base));
     h->tr_slots = slots;
     return CRKDG_OK;
 }

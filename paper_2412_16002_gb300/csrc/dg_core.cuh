@@ -2423,11 +2423,6 @@ __global__ void k_features(Params P, Bufs B) {
     features_body<DIM, N, PHYS>(P, B, blockIdx.x);
 }
 
-// Meshes from this size on take the faces' corrections in a pass of their own (k_faces): below it a step is
-// bound by latency, and the pass is one more launch (64^2 Q^2 9 + 18 us against 20 for the final kernel alone;
-// 1024^2 Q^2 0.43 + 0.56 ms against 1.86, 513^2 Q^3 0.24 + 0.21 against 0.67).  The bits are the same.
-constexpr int kFacesCells = 16384;
-
 template <int DIM, int N, int PHYS>
 cudaError_t launch_one(int kernel, cudaStream_t st, const Params &P, const Bufs &B) {
     using C = CfgW<DIM, N, PHYS>;
@@ -2442,7 +2437,7 @@ cudaError_t launch_one(int kernel, cudaStream_t st, const Params &P, const Bufs 
     case K_FINAL:
         if (!B.tsum) {
             k_final<DIM, N, PHYS, RECOMPUTED><<<nblocks, C::NT, 0, st>>>(P, B);
-        } else if (DIM == 2 && P.ncell >= kFacesCells) {
+        } else if (DIM == 2 && B.fc) {
             const size_t points = 2 * (size_t)P.ncell * N;
             k_faces<N, PHYS><<<(unsigned)((points + 127) / 128), 128, 0, st>>>(P, B);
             k_final<DIM, N, PHYS, FACES><<<nblocks, C::NT, 0, st>>>(P, B);

@@ -40,6 +40,13 @@ __host__ __device__ constexpr int cells_per_block(int dim, int n) {
            (warp_cells(dim == 2 ? n * n : n) >= 128 ? 1 : 128 / warp_cells(dim == 2 ? n * n : n));
 }
 
+// 2D meshes from this many cells on take the faces' corrections in a pass of their own (k_faces): below, the pass
+// is one launch too many.  Final stage with it and without, Riemann problem: Q^1 192^2 44 against 43 us, 256^2 58
+// against 59, 362^2 83 against 90; Q^2 64^2 32 against 30, 80^2 35.2 against 35.1, 96^2 45 against 48, 128^2 52
+// against 60, 512^2 294 against 489; Q^3 64^2 42 against 37, 80^2 51 against 53, 128^2 75 against 80, 512^2
+// 465 against 668.  The bits are the same.
+__host__ __device__ constexpr int faces_cells(int n) { return n == 2 ? 65536 : 6400; }
+
 // The FP64 kernels instead keep whole cells per warp (32 / nn of them, see CfgW).
 constexpr int kWarpThreads = 128;
 __host__ __device__ constexpr int warp_cells_per_block(int nn) { return (32 / nn) * (kWarpThreads / 32); }
@@ -297,7 +304,7 @@ struct Bufs {
     // the traces [m][cell][face point], and each traced stage's largest radius over a face's
     // points [slot][cell][face]
     double *tsum = nullptr, *tsp = nullptr;
-    // 2D, with tsum: the faces' corrections for the cells above and below them
+    // 2D, with tsum, from faces_cells on: the faces' corrections for the cells above and below them
     // [direction][above, below][m][cell of the lower face][face point]
     double *fc = nullptr;
     int *flag;          // set when a stage average leaves B

@@ -41,6 +41,30 @@ def _free():
     return torch.cuda.mem_get_info()[0]
 
 
+def test_handle_without_face_corrections():
+    """Q^2 with the midpoint rule (one traced stage): state and traces take 8 (3 m nn + m (1 + ntr) + m ntr + 4) bytes a
+    cell, the corrections 8 m ntr more; with room for the former only, a step runs and has the bits of one with room
+    for both."""
+    from paper_2412_16002_gb300.solver import Solver
+
+    n, k = 1000, 2
+    U = torch.from_numpy(np.broadcast_to(inputs.random_euler(2, n, 1, k, seed=1, osc=0.2), (4, n, n, 3, 3)).copy()).cuda()
+    cells, m, nn, ntr = n * n, 4, 9, 12
+    need = 8 * cells * (3 * m * nn + m + m * (1 + ntr) + m * ntr + 4)
+    out = []
+    for keep in (need + 8 * cells * m * ntr + 512 * MB, need + 96 * MB):
+        with _Leave(keep):
+            g = Solver(2, n, n, k, (0.0, 1.0, 0.0, 1.0), "euler", bc=("outflow",) * 4)
+            g.set_state(U)
+            free = _free()
+            g.step(1e-5, "midpoint2")
+            used = free - _free()
+        out.append((used, g.get_state()))
+        g.close()
+    assert out[1][0] < out[0][0] - 0.9 * 8 * cells * m * ntr  # the corrections are not there
+    assert np.array_equal(out[0][1], out[1][1])
+
+
 @pytest.mark.parametrize("indicator", ["off", "tvb"])
 def test_ensemble_without_flux_sums(indicator):
     """Between room for the traces alone and room for everything, creating and stepping work at every amount, with the
