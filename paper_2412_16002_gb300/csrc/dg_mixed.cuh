@@ -1553,14 +1553,24 @@ __global__ void k_avg_x(Params P, MixBufs X) {
 template <int DIM, int N, int PHYS>
 cudaError_t launch_one_x(int kernel, int nblocks, cudaStream_t st, const Params &P, const MixBufs &X) {
     using C = Cfg<DIM, N, PHYS>;
+    constexpr bool CELL = DIM == 2 && PHYS == PH_EULER;  // its split, merge and troubled-cell pass: dg_cell.cuh
     switch (kernel) {
-    case KX_SPLIT: k_split_x<C><<<nblocks, C::NT, 0, st>>>(P, X); break;
-    case KX_MERGE: k_merge_x<C><<<nblocks, C::NT, 0, st>>>(P, X); break;
+    case KX_SPLIT:
+        if constexpr (CELL) return cudaErrorInvalidValue;
+        else k_split_x<C><<<nblocks, C::NT, 0, st>>>(P, X);
+        break;
+    case KX_MERGE:
+        if constexpr (CELL) return cudaErrorInvalidValue;
+        else k_merge_x<C><<<nblocks, C::NT, 0, st>>>(P, X);
+        break;
     case KX_LIMIT: k_limit_x<C><<<nblocks, C::NT, 0, st>>>(P, X); break;
     case KX_INNER: k_inner_x<C><<<nblocks, C::NT, 0, st>>>(P, X); break;
     case KX_FINAL: k_final_x<C><<<nblocks, C::NT, 0, st>>>(P, X); break;
     case KX_SCAN: k_scan_x<C><<<nblocks, C::NT, 0, st>>>(P, X); break;
-    case KX_TROUBLE: k_trouble_x<C><<<nblocks, C::NT, 0, st>>>(P, X); break;
+    case KX_TROUBLE:  // the indicator is Euler's
+        if constexpr (CELL || PHYS != PH_EULER) return cudaErrorInvalidValue;
+        else k_trouble_x<C><<<nblocks, C::NT, 0, st>>>(P, X);
+        break;
     case KX_FEATURES: k_features_x<C><<<(P.ncell + 127) / 128, 128, 0, st>>>(P, X); break;
     case KX_AVG: {
         int tot = P.ncell * C::M;
