@@ -74,18 +74,17 @@ DEFAULT_STEPS = {"euler1d": 2000, "burgers": 2000, "sedov": 50, "sedov_shell": 5
                  "double_mach": 50, "shock_diffraction": 50}
 
 
-def launches_per_attempt(precision, indicator, cells=0):
-    """Kernels one step attempt launches: the inner and final stages; in FP64 on a 2D mesh of 16384
-    cells and more the face pass; the indicator: the
-    troubled-cell pass, after (learned) the feature kernel and the network's forward pass, on
-    the split path also the merge to FP64 nodal values the feature kernel reads; then the
-    component totals of the new state for the step's conservation drift (two reduction
-    kernels, after the FP64 path's cell-average kernel)."""
-    n = 2 + (2 if precision == "mixed" else 3) + (precision != "mixed" and cells >= 16384)
+def launches_per_attempt(precision, indicator, cells=0, k=2):
+    """Kernels one step attempt launches: the inner and final stages; in FP64 on a 2D mesh of 6400
+    cells and more (Q^1 65536) the face pass; the indicator: the troubled-cell pass, after
+    (learned) the feature kernel and the network's forward pass; then the component totals of the
+    new state for the step's conservation drift (two reduction kernels, after the FP64 path's
+    cell-average kernel)."""
+    n = 2 + (2 if precision == "mixed" else 3) + (precision != "mixed" and cells >= (65536 if k == 1 else 6400))
     if indicator == "tvb":
         n += 1
     elif indicator == "mlp":
-        n += 3 + (1 if precision == "mixed" else 0)
+        n += 3
     return n
 
 
@@ -524,7 +523,7 @@ def run_decomposed(args, wl, name):
                          "note": "rank 0's dominant kernel over its local cells (owned block and halo ring)"},
             "e2e": {"value": e2e_value, "unit": "cell-DOF-stage/s", "h2d_bytes_per_step": nbytes,
                     "d2h_bytes_per_step": nbytes},
-            "gpu_launches": int(kn["inner"]) * launches_per_attempt(precision, "off", lay.nxl * lay.nyl) * world,
+            "gpu_launches": int(kn["inner"]) * launches_per_attempt(precision, "off", lay.nxl * lay.nyl if wl.dim == 2 else 0, wl.k) * world,
             "clocks": clocks,
         }
         print(json.dumps(line))
@@ -680,7 +679,7 @@ def run_gb300(args, wl, name):
                          "flops_per_cell": {"k_inner": inner_f, "k_final": final_f}},
             "e2e": {"value": e2e_value, "unit": "cell-DOF-stage/s", "h2d_bytes_per_step": nbytes,
                     "d2h_bytes_per_step": nbytes},
-            "gpu_launches": int(kn["run"]) if kn["run"] else int(kn["inner"]) * launches_per_attempt(precision, indicator, wl.nx * wl.ny if wl.dim == 2 else 0),
+            "gpu_launches": int(kn["run"]) if kn["run"] else int(kn["inner"]) * launches_per_attempt(precision, indicator, wl.nx * wl.ny if wl.dim == 2 else 0, wl.k),
             "clocks": clocks,
         }
         if world == 1 and not args.no_cpu_baseline:

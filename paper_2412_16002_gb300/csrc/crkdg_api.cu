@@ -414,7 +414,7 @@ MixBufs base_xbufs(const crkdg_ctx *h) {
 bool euler_2d(const crkdg_ctx *h) { return h->dim == 2 && h->phys == PH_EULER; }
 
 // 2D Euler steps whose tableau has only a sub-diagonal (every tableau of the paper) run the inner
-// stages by lines (2048^2 Q^3 3.40 ms), or for Q^3 on request on the tensor cores (7.07 ms); other cases
+// stages by lines (2048^2 Q^3 3.08 ms), or for Q^3 on request on the tensor cores (7.07 ms); other cases
 // run k_inner_x.
 bool sub_diagonal_euler(const crkdg_ctx *h, const Params &P) {
     if (!euler_2d(h) || P.mode != MODE_STEP) return false;

@@ -1234,12 +1234,10 @@ __device__ __forceinline__ unsigned biased_exp(int x) { return (unsigned)max(x +
 // of the magnitudes of a node's own terms, is the FP64 form's: 0.8 (Euler Q^2), 0.9 (Burgers Q^2) and 1.4
 // (advection Q^3); without the rule it grew with the contrast (at 2^-9 to 77, 4e3 and 17).
 //
-// Why: with FP64 maps and fluxes a warp issued about 145 FP64 instructions per Q^3 stage, 76 cycles
-// each; now about 30, with 2000 instructions on the other pipes beside them.  Set state, steps, get
-// state: 513^2 Q^3, 2 RK4 steps 15.9 -> 11.8 (maps) -> 5.8 (fluxes and the final stage) -> 5.0 ms (no
-// fallback for small momenta); 1024^2 Q^2, 3 Heun steps 49.7 -> 40.0 -> 22.2 ms.  The integer root of the
-// sound speed, a sub-diagonal tableau's G in registers and face rounds without a branch: a launch 1.56 ->
-// 1.43 ms and 4.92 -> 4.50 ms.
+// Why: with FP64 maps and fluxes a warp issues about 145 FP64 instructions per Q^3 stage, 76 cycles
+// each; this form about 30, with 2000 instructions on the other pipes beside them: bound by issue and the
+// FP64 pipe together.  Set state, steps, get state: 513^2 Q^3, 2 RK4 steps 15.9 ms with FP64 forms throughout,
+// 4.20 with the integer ones here and in the final stage; 1024^2 Q^2, 3 Heun steps 49.6 and 17.0 ms.
 template <class C, class Put, class Fn>
 __device__ __forceinline__ void eval_G_fx(const Params &P, Smem<C> &S, const BlockTab<C> &Tb, int lc, int node,
                                           const double *u, double *g, bool want_speed, bool want_avg, Put put,

@@ -1,14 +1,12 @@
 // dg_line.cuh -- the split-precision step of 2D Euler by lines: N / R threads per cell, each with R node rows and R
 // node columns (Q^1: two threads with one, Q^2: three with one, Q^3: two with two).
 //
-// One thread per cell (dg_cell.cuh) holds all of its deviations and G, so that only two warps fit a
-// scheduler, and a stage waits on its own dependent chains and shared-memory reads (2048^2 Q^3: 31% of
-// the issue slots used, stalls on short scoreboards and fixed latencies).  The volume term, both
-// end traces, their fluxes and lifts, and the S_K points of a line need that line only.  Rows live in
-// registers; a component's values go through shared memory once to be read as columns, and the columns'
-// part comes back the same way.  Half the registers a thread or fewer, and two or three times the threads
-// on a small mesh.  The FP64 conversions of a stage (64 cycles of the FP64 pipe each) become sums of two
-// floats.
+// The volume term, both end traces, their fluxes and lifts, and the S_K points of a line need that line
+// only.  Rows live in registers; a component's values go through shared memory once to be read as columns,
+// and the columns' part comes back the same way.  One thread for a whole cell would hold all of its
+// deviations and G: two warps a scheduler, 31% of the issue slots, and a half or a third of the
+// threads on a small mesh.  Averages of a stage are sums of two floats (an FP64 conversion takes its pipe 64
+// cycles).
 #pragma once
 
 #include "dg_cell.cuh"
@@ -242,8 +240,9 @@ __device__ __forceinline__ void store_run(float *p, const float *v) {
 
 }  // namespace pc
 
-// Inner stages (tableaux whose A has only a sub-diagonal).  Against one thread per cell: 2048^2 Q^3 5.40 ->
-// 3.40 ms a launch, 131^2 Q^3 49 -> 27 us, 1024^2 Q^2 684 -> 352 us.
+// Inner stages (tableaux whose A has only a sub-diagonal).  Bound by issue (Q^2 83% of the slots, Q^3 64% at three
+// blocks an SM): 2048^2 Q^3 3.08 ms a launch, 131^2 Q^3 27 us, 1024^2 Q^2 350 us (one thread per cell: 5.40 ms, 49
+// and 684 us; Q^3 on the tensor cores 7.07 ms).
 template <int N>
 __global__ void __launch_bounds__(pc::LT, pc::Line<N>::BLOCKS) k_inner_l(const __grid_constant__ Params P, const __grid_constant__ MixBufs X) {
     using namespace pc;
@@ -526,8 +525,8 @@ __device__ __forceinline__ bool line_rate(const Params &P, float eps, const floa
 }
 
 // The two faces of a cell across direction DIR (this thread's R points of each): the sums over the traced stages
-// of b_i (fhat - f_int) (dc) and of b_i fhat (fh).  A stage's loads for both faces are issued together:
-// the kernel waits on them with three to five warps a scheduler (face by face 3.14 ms, 26 and 370 us).
+// of b_i (fhat - f_int) (dc) and of b_i fhat (fh).  A stage's loads for both faces are issued together: the kernel
+// waits on them with three to five warps a scheduler (face by face the meshes below take 3.14 ms, 26 and 370 us).
 template <int N, int DIR>
 __device__ __forceinline__ void face_sums(const Params &P, const MixBufs &X, int cell, bool active, int h, int base,
                                           float (&dc)[2][M][Line<N>::R], float (&fh)[2][M][Line<N>::R]) {
@@ -621,8 +620,8 @@ __device__ __forceinline__ RunSum cell_run(const RunSum &p, int base) {
 // Final stage (see k_final_x for the formulas): the fluxes of every traced stage at this thread's points of the
 // four faces, their lifts along its rows and columns, and their fixed-point sums into the averages; then
 // the limiter, or with the indicator the averages and the unlimited deviations for the troubled-cell
-// pass.  The FP64 part of the averages is spread over the cell's threads.  Against one thread per cell:
-// 2048^2 Q^3 3.53 -> 3.11 ms a launch, 131^2 Q^3 47 -> 23 us, 1024^2 Q^2 376 -> 347 us.
+// pass.  The FP64 part of the averages is spread over the cell's threads.  Bound by the latency of the trace
+// loads: 2048^2 Q^3 3.11 ms a launch, 131^2 Q^3 23 us, 1024^2 Q^2 347 us (one thread per cell: 3.53 ms, 47 and 376 us).
 template <int N>
 __global__ void __launch_bounds__(pc::LT, pc::Line<N>::BLOCKS) k_final_l(const __grid_constant__ Params P, const __grid_constant__ MixBufs X) {
     using namespace pc;

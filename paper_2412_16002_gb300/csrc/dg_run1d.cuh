@@ -74,8 +74,9 @@ __device__ bool grid_barrier(RunCtl *R, unsigned target, const RunSlot *SL, Slot
 
 // The stages run on the integer units as in the per-step kernels (eval_G_fx, lift_faces), and the
 // final stage combines jumps of the weighted flux sums: of the FP64 instructions of a step, each 64 to
-// 76 cycles behind the one before it, about a quarter is left (4096 cells of the blast tube 20.2 -> 18.9 us a
-// step, where the blocks at the front wait for the limiter's FP64 form; Burgers, 200 cells, 7.7 -> 7.4).
+// 76 cycles behind the one before it, about a quarter is left.  Latency bounds the loop: 4096 cells of the blast
+// tube 17.4 us a step (FP64 forms 20.2), where the blocks at the front wait for the limiter's FP64 form; Burgers,
+// 200 cells, 7.4 (7.7).
 // FX as in inner_body.
 template <int N, int PHYS, bool FX>
 __global__ void __launch_bounds__(RunCfg1D<N, PHYS>::NT) k_run1d(const __grid_constant__ Params P, double *U0, double *U1,
